@@ -132,6 +132,8 @@ cudaError_t launch_bwd_weight_tc(const ConvShape& s, const void* x, const void* 
                                  float* const dw[4], int num_sms,
                                  unsigned long long wait_limit_ns, cudaStream_t stream,
                                  char* err, size_t errlen);
+// Four fp32 arrays of n elements set to zero in one launch.
+cudaError_t launch_zero4(float* const t[4], long long n, int num_sms, cudaStream_t stream);
 // dW_L fp32 [Qout][kh][kw][Qin] (zeroed, then accumulated) on CUDA cores.
 cudaError_t launch_bwd_weight_simt(const ConvShape& s, const void* x, const void* dy,
                                    float* const dw[4], int num_sms, cudaStream_t stream);

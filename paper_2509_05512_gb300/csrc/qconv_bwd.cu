@@ -219,7 +219,31 @@ __global__ void __launch_bounds__(256) bwd_upsample_kernel(const uint4* __restri
     }
 }
 
+// The four weight gradients set to zero before a kernel adds to them: one launch that takes
+// part in the dependent-launch chain (four memset nodes cost four launches and end it).
+__global__ void __launch_bounds__(256) zero4_kernel(float* __restrict__ a, float* __restrict__ b,
+                                                    float* __restrict__ c, float* __restrict__ d,
+                                                    long long n) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+         i += static_cast<long long>(gridDim.x) * blockDim.x) {
+        a[i] = 0.f;
+        b[i] = 0.f;
+        c[i] = 0.f;
+        d[i] = 0.f;
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_zero4(float* const t[4], long long n, int num_sms, cudaStream_t stream) {
+    if (n == 0) return cudaSuccess;
+    long long blocks = (n + 255) / 256;
+    if (blocks > num_sms * 8LL) blocks = num_sms * 8LL;
+    return launch_pdl(zero4_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream,
+                      t[0], t[1], t[2], t[3], n);
+}
 
 cudaError_t launch_bwd_upsample(const void* dy, int N, int Ho, int Wo, int C, int s, int Hu,
                                 int Wu, void* u, int num_sms, cudaStream_t stream) {
@@ -276,11 +300,8 @@ cudaError_t launch_bwd_data_simt(const ConvShape& s, const void* dy, const void*
 cudaError_t launch_bwd_weight_simt(const ConvShape& s, const void* x, const void* dy,
                                    float* const dw[4], int num_sms, cudaStream_t stream) {
     const long long outs = static_cast<long long>(s.Qout) * s.kh * s.kw * s.Qin;
-    const size_t bytes = static_cast<size_t>(outs) * sizeof(float);
-    for (int L = 0; L < 4; ++L) {
-        cudaError_t e = cudaMemsetAsync(dw[L], 0, bytes, stream);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = launch_zero4(dw, outs, num_sms, stream);
+    if (e != cudaSuccess) return e;
     if (outs == 0 || s.M == 0) return cudaSuccess;
     // enough pixel chunks to give every SM a few thousand threads
     const long long oblocks = (outs + 255) / 256;

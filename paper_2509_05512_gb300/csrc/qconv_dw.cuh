@@ -11,9 +11,12 @@
 //
 // Both MMA operands come straight from the NHWC tensors: a TMA box of 64 channels x P
 // pixels (P = Ht rows x Wbox columns of one image) lands as P rows of 128 bytes, the
-// MN-major SWIZZLE_128B layout (channels along M or N, pixels along K).  For a strided
-// convolution the x box traverses every stride-th input pixel (the tensor map's element
-// strides), so it lands in the same layout as the dy box of the output pixels it serves.  A holds two such
+// MN-major SWIZZLE_128B layout (channels along M or N, pixels along K).  For a stride-2
+// convolution x is seen as four tensors, one per parity (a, b) of the input row and column
+// (every second row and column, four tensor maps): tap dh reads input row
+// 2 ho + dh - pad, row ho + floor((dh - pad) / 2) of the maps with a = (dh - pad) mod 2, so
+// the box is dense in its map and lands in the layout of the dy box of the output pixels it
+// serves (one map with element strides of 2 reads the pixels it skips as well).  A holds two such
 // boxes ("units": one tap's window of x, one 64-channel chunk) stacked to M = 128; B holds
 // ncols / 64 boxes of dy, N = ncols.  A CTA owns a_per unit pairs (one TMEM accumulator of
 // ncols fp32 columns each) and one ncols-wide group of output channels, for a contiguous
@@ -25,23 +28,33 @@
 
 namespace dwk {
 
-constexpr int THREADS = 256;  // warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner,
+constexpr int THREADS = 256;  // warp 1 MMA issuer, warp 2 TMEM owner,
 constexpr int EPI_WARP0 = 4;  // warps 4-7 epilogue (TMEM lane quarters 0-3)
+// Every warp but the issuer produces: box k of a stage is loaded by producer k mod 7.  A TMA
+// instruction costs its thread 0.1-0.25 us, and a stage of 8 boxes feeds only 0.5 us of MMAs
+// (11 boxes and 0.1 us for 64 -> 64 channels), so one producing thread set the pace.
+constexpr int PRODUCERS = 7;
 constexpr int MAX_PAIRS = 8;
 constexpr int MAX_STAGES = 4;
 constexpr int BOX_ROW = 128;  // bytes of one pixel's 64 channels
 constexpr int BAR_BYTES = 256;
+constexpr int LONE_COORD = 1 << 20;  // past the end of any map (rows and columns)
 // Shared memory reserved past the barriers: the MMA reads of the last stage stay inside the
 // CTA's allocation even for a descriptor whose two byte offsets were read the other way
-// round (one pixel block plus 4 KB beyond the stage), and a strided x box (stride s) stays
-// inside it even if the copy brought its s * s untraversed elements as well.
-__host__ __device__ constexpr int tail_bytes(int P, int stride = 1) {
-    return P * BOX_ROW + 4096 + (stride * stride - 1) * P * BOX_ROW;
-}
+// round (one pixel block plus 4 KB beyond the stage).
+__host__ __device__ constexpr int tail_bytes(int P) { return P * BOX_ROW + 4096; }
+
+// Tensor maps of x: [0] for stride 1; [2 a + b] for stride 2, parity (a, b) of the input row
+// and column.
+struct DwMaps {
+    CUtensorMap x[4];
+};
 
 struct DwParams {
     int Ho, Wo, Qin, Qout, kh, kw, pad, taps;
-    int stride;              // the x boxes traverse every stride-th pixel (element strides)
+    int stride;              // 1 or 2 (four parity maps of x)
+    int lone;                // stride 2: bit 0 (1) set when x has one row (column), so that
+                             // the odd parity's map is empty and its boxes are zero
     int Wbox, Ht, P;         // pixel block: Ht rows x Wbox columns = P pixels
     int rblocks;             // pixel blocks per image
     long long kblocks;       // N * rblocks
@@ -50,6 +63,7 @@ struct DwParams {
     int ncols, nyb;          // output channels per CTA (N of each MMA); dy boxes per stage
     int groups, splits, stages;
     int sep;                 // 1: fold for the separable form
+    int producers;           // TMA-issuing threads: min(PRODUCERS, boxes of a full stage)
     uint32_t tmem_cols;
     uint32_t stage_bytes;
     unsigned long long wait_limit_ns;
@@ -75,7 +89,7 @@ __device__ __forceinline__ float* letter_ptr(const DwParams& p, int L) {
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
-    qconv_dw_kernel(const __grid_constant__ CUtensorMap tmap_x,
+    qconv_dw_kernel(const __grid_constant__ DwMaps tmaps,
                     const __grid_constant__ CUtensorMap tmap_dy, const DwParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -105,7 +119,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     griddep_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) {
-            mbar_init(full_bar(i), 1);
+            mbar_init(full_bar(i), p.producers);
             mbar_init(empty_bar(i), 1);
         }
         mbar_init(done_bar, 1);
@@ -113,7 +127,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         fence_barrier_init();
     }
     if (warp == 0 && lane == 0) {
-        tma_prefetch_desc(&tmap_x);
+        for (int i = 0; i < (p.stride == 1 ? 1 : 4); ++i) tma_prefetch_desc(&tmaps.x[i]);
         tma_prefetch_desc(&tmap_dy);
     }
     if (warp == 2) {
@@ -126,11 +140,14 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t tmem_base = *tmem_slot;
     griddep_wait();  // x and dy complete, the zeroed outputs visible
 
-    if (warp == 0) {
-        // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
+    if (warp != 1) {
+        // ---------------------------------------------------------------- TMA producers
+        const int me = warp == 0 ? 0 : warp - 1;  // 0 .. PRODUCERS - 1
+        if (lane == 0 && me < p.producers) {
             const uint64_t pol = l2_policy_evict_normal();
-            const uint32_t tx = static_cast<uint32_t>(2 * npair + p.nyb) * box_bytes;
+            const int boxes = 2 * npair + p.nyb;
+            const uint32_t tx =
+                static_cast<uint32_t>((boxes - me + p.producers - 1) / p.producers) * box_bytes;
             uint32_t filled = 0, fill_parity = 0;
             bool ok = true;
             int stage = 0;
@@ -148,18 +165,30 @@ __global__ void __launch_bounds__(THREADS, 1)
                 filled |= 1u << stage;
                 fill_parity = (fill_parity & ~(1u << stage)) | (phase << stage);
                 const uint32_t dst = sbase + stage * p.stage_bytes;
-                for (int k = 0; k < 2 * npair; ++k) {
+                for (int k = me; k < boxes; k += p.producers) {
+                    if (k >= 2 * npair) {  // dy
+                        const int c = k - 2 * npair;
+                        tma_load_4d(dst + (2 * p.a_per + c) * box_bytes, &tmap_dy, fb,
+                                    cg * p.ncols + c * 64, 0, r0, n, pol);
+                        continue;
+                    }
                     int u = 2 * pair0 + k;
                     if (u >= p.units) u = p.units - 1;  // odd unit count: repeat the last
                     const int tap = u / p.nxc, xc = u - tap * p.nxc;
                     const int dh = tap / p.kw, dw = tap - dh * p.kw;
-                    tma_load_4d(dst + k * box_bytes, &tmap_x, fb, xc * 64, dw - p.pad,
-                                r0 * p.stride - p.pad + dh, n, pol);
+                    int row = r0 + dh - p.pad, col = dw - p.pad, map = 0;
+                    if (p.stride == 2) {
+                        const int th = dh - p.pad, tw = dw - p.pad;
+                        map = 2 * (th & 1) + (tw & 1);
+                        row = r0 + (th >> 1);
+                        col = tw >> 1;
+                        // an empty parity class: a box past the end of its stand-in map
+                        if ((th & 1) && (p.lone & 1)) row = LONE_COORD;
+                        if ((tw & 1) && (p.lone & 2)) col = LONE_COORD;
+                    }
+                    tma_load_4d(dst + k * box_bytes, &tmaps.x[map], fb, xc * 64, col, row, n,
+                                pol);
                 }
-                const uint32_t ydst = dst + 2 * p.a_per * box_bytes;
-                for (int c = 0; c < p.nyb; ++c)
-                    tma_load_4d(ydst + c * box_bytes, &tmap_dy, fb, cg * p.ncols + c * 64, 0, r0,
-                                n, pol);
                 if (++stage == p.stages) {
                     stage = 0;
                     phase ^= 1u;
@@ -168,7 +197,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             if (!ok || *abort_flag)
                 drain_fills(full_bar(0), p.stages, filled, fill_parity, limit);
         }
-    } else if (warp == 1) {
+        __syncwarp();
+    } else {
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0) {
             const uint32_t idesc = make_idesc_mn(128, p.ncols);
@@ -203,7 +233,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             // the teardown can wait for them before TMEM is released)
             umma_commit(done_bar);
         }
-    } else if (warp >= EPI_WARP0) {
+    }
+    if (warp >= EPI_WARP0) {
         // ---------------------------------------------------------------- epilogue
         const int q = warp - EPI_WARP0;  // TMEM lane quarter
         const bool ok = wait_or_abort(done_bar, 0, limit, abort_flag, STATUS_TIMEOUT_EPILOGUE);

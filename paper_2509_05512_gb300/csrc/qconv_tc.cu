@@ -1337,14 +1337,14 @@ bool dw_plan(const ConvShape& s, int num_sms, dwk::DwParams* p) {
         const int wcand[2] = {(s.Wo + 7) / 8 * 8, (s.Wo + 15) / 16 * 16};
         for (int wc = 0; wc < 2; ++wc) {
             const int Wbox = wcand[wc];
-            if (Wbox * s.stride > 256) continue;  // the x box spans stride * Wbox columns
+            if (Wbox * s.stride > 256) continue;
             for (int Ht = 1; Ht <= 8; ++Ht) {
                 const int P = Wbox * Ht;
                 if (P % 16 != 0 || P > 256 || Ht * s.stride > 256) continue;
                 const long long stage =
                     static_cast<long long>(2 * a_per + q.nyb) * P * dwk::BOX_ROW;
                 long long stages = (DW_SMEM_MAX - 1024 - dwk::BAR_BYTES -
-                                    dwk::tail_bytes(P, s.stride)) /
+                                    dwk::tail_bytes(P)) /
                                    stage;
                 if (stages > dwk::MAX_STAGES) stages = dwk::MAX_STAGES;
                 if (stages < 2) continue;
@@ -1366,6 +1366,12 @@ bool dw_plan(const ConvShape& s, int num_sms, dwk::DwParams* p) {
     if (!found) return false;
     q.pair_groups = (q.npairs + q.a_per - 1) / q.a_per;
     q.groups = q.pair_groups * (s.Cout / q.ncols);
+    // the last group of unit pairs may hold fewer boxes than the others: every producer
+    // needs at least one box of the smallest stage
+    const int last_pairs = q.npairs - (q.pair_groups - 1) * q.a_per;
+    q.producers = 2 * last_pairs + q.nyb;
+    if (q.producers > dwk::PRODUCERS) q.producers = dwk::PRODUCERS;
+    q.lone = s.stride == 2 ? (s.H == 1 ? 1 : 0) | (s.W == 1 ? 2 : 0) : 0;
     q.kblocks = static_cast<long long>(s.N) * q.rblocks;
     long long splits = num_sms / q.groups;
     if (splits < 1) splits = 1;
@@ -1379,23 +1385,24 @@ bool dw_plan(const ConvShape& s, int num_sms, dwk::DwParams* p) {
     return true;
 }
 
-// [N][H][W][C] bf16, boxes of 64 channels x Wbox columns x Ht rows of one image, SW128;
-// with `step` > 1 the box traverses every step-th column and row (it spans step * Wbox
-// columns and step * Ht rows, and the copy brings Wbox x Ht pixels).
+// [N][H][W][C] bf16, boxes of 64 channels x Wbox columns x Ht rows of one image, SW128; with
+// step = 2 the pixels of parity (a, b): rows a, a + 2, .. and columns b, b + 2, ..
 bool encode_dw_map(CUtensorMap* map, const void* t, int C, int W, int H, int N, int Wbox,
-                   int Ht, int step = 1) {
-    const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W),
-                                static_cast<cuuint64_t>(H), static_cast<cuuint64_t>(N)};
-    const cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2,
-                                   static_cast<cuuint64_t>(C) * 2 * W,
-                                   static_cast<cuuint64_t>(C) * 2 * W * H};
-    const cuuint32_t box[4] = {64, static_cast<cuuint32_t>(Wbox * step),
-                               static_cast<cuuint32_t>(Ht * step), 1};
-    const cuuint32_t estr[4] = {1, static_cast<cuuint32_t>(step), static_cast<cuuint32_t>(step),
-                                1};
+                   int Ht, int step = 1, int a = 0, int b = 0) {
+    const cuuint64_t e = static_cast<cuuint64_t>(C) * 2;  // bytes per pixel
+    if (a >= H) a = 0;  // an empty class: any map stands in (its boxes are read past the end)
+    if (b >= W) b = 0;
+    const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C),
+                                static_cast<cuuint64_t>((W - b + step - 1) / step),
+                                static_cast<cuuint64_t>((H - a + step - 1) / step),
+                                static_cast<cuuint64_t>(N)};
+    const cuuint64_t strides[3] = {e * step, e * W * step, e * W * H};
+    const cuuint32_t box[4] = {64, static_cast<cuuint32_t>(Wbox), static_cast<cuuint32_t>(Ht), 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const char* base = static_cast<const char*>(t) + (static_cast<size_t>(a) * W + b) * e;
     const CUresult r = g_encode_tiled(
-        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(t), dims, strides, box, estr,
-        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<char*>(base), dims, strides, box,
+        estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
@@ -1819,24 +1826,28 @@ cudaError_t launch_bwd_weight_tc(const ConvShape& s, const void* x, const void* 
         snprintf(err, errlen, "cuTensorMapEncodeTiled is not available");
         return cudaErrorInvalidValue;
     }
-    CUtensorMap mx, mdy;
-    if (!encode_dw_map(&mx, x, s.Cin, s.W, s.H, s.N, p.Wbox, p.Ht, s.stride) ||
-        !encode_dw_map(&mdy, dy, s.Cout, s.Wo, s.Ho, s.N, p.Wbox, p.Ht)) {
+    CUtensorMap mdy;
+    dwk::DwMaps mx;
+    bool ok = encode_dw_map(&mdy, dy, s.Cout, s.Wo, s.Ho, s.N, p.Wbox, p.Ht);
+    for (int i = 0; ok && i < 4; ++i)
+        ok = i > 0 && s.stride == 1
+                 ? (mx.x[i] = mx.x[0], true)
+                 : encode_dw_map(&mx.x[i], x, s.Cin, s.W, s.H, s.N, p.Wbox, p.Ht, s.stride,
+                                 i >> 1, i & 1);
+    if (!ok) {
         snprintf(err, errlen, "tensor-map encode failed for the weight gradient");
         return cudaErrorInvalidValue;
     }
-    const size_t bytes = static_cast<size_t>(s.Qout) * s.kh * s.kw * s.Qin * sizeof(float);
-    for (int L = 0; L < 4; ++L) {
-        cudaError_t e = cudaMemsetAsync(dw[L], 0, bytes, stream);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t ez = launch_zero4(
+        dw, static_cast<long long>(s.Qout) * s.kh * s.kw * s.Qin, num_sms, stream);
+    if (ez != cudaSuccess) return ez;
     p.wait_limit_ns = wait_limit_ns;
     p.dwr = dw[0];
     p.dwi = dw[1];
     p.dwj = dw[2];
     p.dwk = dw[3];
     const int smem = p.stages * static_cast<int>(p.stage_bytes) + dwk::BAR_BYTES +
-                     dwk::tail_bytes(p.P, s.stride) + 1024;
+                     dwk::tail_bytes(p.P) + 1024;
     static std::atomic<unsigned long long> attr_done{0};
     cudaError_t e = set_smem_once(dwk::qconv_dw_kernel, DW_SMEM_MAX, attr_done);
     if (e != cudaSuccess) return e;

@@ -249,6 +249,24 @@ def test_bwd_weight_tensor_cores(case):
     check_weight(d, path=quan.QUAN_PATH_TC)
 
 
+PARITY_WEIGHT_CASES = [
+    # stride 2 through the four parity maps of x, and a short last group of unit pairs
+    ("dwp_one_row", 3, 1, 17, 64, 64, 3, 2, 1),      # the odd row parity is empty
+    ("dwp_one_col", 2, 14, 1, 128, 64, 3, 2, 1),     # the odd column parity is empty
+    ("dwp_pad0", 1, 9, 8, 64, 128, 3, 2, 0),
+    ("dwp_pad2", 1, 8, 9, 64, 64, 3, 2, 2),          # taps start two rows above the image
+    ("dwp_k1_odd", 2, 13, 15, 64, 192, 1, 2, 0),
+    ("dwp_short_group", 1, 9, 10, 128, 256, 3, 2, 1),  # 9 pairs, 2 per CTA, the last alone
+]
+
+
+@pytest.mark.parametrize("case", PARITY_WEIGHT_CASES, ids=[c[0] for c in PARITY_WEIGHT_CASES])
+def test_bwd_weight_parity_maps(case):
+    name, N, H, W, Cin, Cout, k, s, p = case
+    d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(614, len(name))))
+    check_weight(d, path=quan.QUAN_PATH_TC)
+
+
 def test_bwd_weight_paths_agree():
     d = layer(inputs.small_layer("dw_both", 2, 9, 10, 64, 128, 3, 1, 1, seed=(611, 0)))
     tc = check_weight(d, path=quan.QUAN_PATH_TC)
