@@ -55,6 +55,12 @@ bool tc_supported(const ConvShape& s, const void* x, const void* const w[4], con
 cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const w[4],
                             const EpilogueArgs& ep, void* out, const TcOptions& opt,
                             int num_sms, cudaStream_t stream, char* err, size_t errlen);
+// Input gradient of a stride-2 forward convolution f by the parity classes of its pixels
+// (f.sep: 0 or 2), letters in bwd_transform's layout.
+bool tc_parity_supported(const ConvShape& f);
+cudaError_t launch_qconv_tc_parity(const ConvShape& f, const void* dy, const void* const w[4],
+                                   void* dx, const TcOptions& opt, int num_sms,
+                                   cudaStream_t stream, char* err, size_t errlen);
 cudaError_t read_and_clear_status(unsigned* status, cudaStream_t stream);
 // Workspace bytes that let a quad/pair-kernel launch on a device of num_sms SMs split its
 // K ranges evenly over its CTAs (one fp32 partial tile and one flag per CTA).

@@ -9,10 +9,11 @@
 //     conjugated, their channel axes swapped and the filter rotated by 180 degrees, padding
 //     kh - 1 - pad, stride 1 (for a stride-1 forward).  bwd_transform_kernel writes those
 //     letters into a caller workspace and the forward tensor-core kernels run the rest.
-//     A stride-s forward's input gradient is the same stride-1 convolution of dy with
+//     A stride-2 forward's input gradient runs by the parity classes of its pixels
+//     (qconv_tc.cu), and one of any other stride as the same stride-1 convolution of dy with
 //     s - 1 zero rows and columns inserted between its pixels (bwd_upsample_kernel, into
-//     the workspace after the letters), when the caller's workspace holds it; otherwise
-//     the direct CUDA-core kernel below runs;
+//     the workspace after the letters), when the caller's workspace would hold that tensor;
+//     otherwise the direct CUDA-core kernel below runs;
 //   * the weight gradient is a reduction over output pixels, done on CUDA cores: every
 //     thread owns one (co, tap, ci) quaternion of dW for a chunk of pixels and adds its
 //     fp32 partial sum to the zeroed output with atomicAdd.

@@ -55,6 +55,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -101,6 +102,66 @@ struct ScMaps {
     CUtensorMap w[4];
 };
 
+// Pixel classes (PAR form): the input gradient of a stride-2 convolution.  dx at
+// (2 i + a, 2 j + b) is a stride-1 convolution of dy with the filter taps of matching parity
+// only, so its output pixels are four classes (a, b), each with its own im2col map, taps and
+// output positions, and together they run each (pixel, tap) product once.  Spreading dy out
+// with zeros between its pixels instead runs four times the MMAs and writes and reads a
+// tensor four times dy's size: 352 us for 256 -> 512 channels, 64 images of 56 x 56, against
+// 106 us.  Tiles never straddle classes; the classes with most taps come first.
+constexpr int PAR_CLASSES = 4;
+struct PixClass {
+    int Hc, Wc;              // Hc x Wc output pixels of the class per image
+    int kh, kw;              // its filter taps
+    int tap0, tap_h, tap_w;  // letter tap of (dh, dw): tap0 + dh tap_h + dw tap_w
+    int h0, w0;              // input row and column of output (0, 0)'s first tap
+    int ktiles;              // kh * kw * kchunks (0: no tap reaches the class, dx is zero)
+    int tile0;               // first tile of the class
+    int oh, ow;              // a, b
+    long long M;             // N * Hc * Wc
+};
+struct ParArgs {
+    CUtensorMap x[PAR_CLASSES];
+    PixClass cls[PAR_CLASSES];
+    int ncls, H, W;          // the output's size
+};
+struct NoPar {};
+template <bool PAR>
+using ParOf = typename std::conditional<PAR, ParArgs, NoPar>::type;
+
+__device__ __forceinline__ int par_class(const ParArgs& a, int tile) {
+    int c = 0;
+    while (c + 1 < a.ncls && tile >= a.cls[c + 1].tile0) ++c;
+    return c;
+}
+
+struct ParGeo {
+    static constexpr bool kScattered = true;
+    const ParArgs& a;
+    int num_n;
+    __device__ __forceinline__ EpiTile operator()(int tile) const {
+        const PixClass& c = a.cls[par_class(a, tile)];
+        const int t = tile - c.tile0, m_tile = t / num_n;
+        EpiTile g;
+        g.n_tile = t - m_tile * num_n;
+        g.m0 = static_cast<long long>(m_tile) * BM;
+        const long long left = c.M - g.m0;
+        g.rows = left < BM ? static_cast<int>(left) : BM;
+        return g;
+    }
+    __device__ __forceinline__ long long pixel(const EpiTile& g, int tile, int row) const {
+        if (row >= g.rows) return 0;
+        const PixClass& c = a.cls[par_class(a, tile)];
+        const int m = static_cast<int>(g.m0) + row;  // fewer than 2^31 pixels
+        const int r = m / c.Wc, j = m - r * c.Wc;
+        const int n = r / c.Hc, i = r - n * c.Hc;
+        return (static_cast<long long>(n) * a.H + 2 * i + c.oh) * a.W + 2 * j + c.ow;
+    }
+    __device__ __forceinline__ bool empty(int tile) const {
+        return a.cls[par_class(a, tile)].ktiles == 0;
+    }
+};
+
 template <int KAPPA, int BNQ, int MODE>
 struct Cfg {
     static constexpr int A_ROW_BYTES = KAPPA * 2;
@@ -134,14 +195,16 @@ struct Cfg {
 // SC: N tiles from p.sc.n_conv on belong to a 1x1 shortcut on the same input, fused into
 // the launch (ScParams): their K blocks are the filter tap p.sc.tap's only, their letters
 // come from `scm`, and the epilogue writes them to the shortcut's output.
-template <int KAPPA, int BNQ, int MODE, bool SC = false>
+// PAR: the pixel classes of `par` (tmap_x unused).
+template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     qconv_tc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                     const __grid_constant__ CUtensorMap tmap_wr,
                     const __grid_constant__ CUtensorMap tmap_wi,
                     const __grid_constant__ CUtensorMap tmap_wj,
                     const __grid_constant__ CUtensorMap tmap_wk, const TcParams p,
-                    const __grid_constant__ ScMaps scm) {
+                    const __grid_constant__ ScMaps scm, const __grid_constant__ ParOf<PAR> par) {
+    static_assert(!PAR || (!SC && (MODE == MODE_PAIR || MODE == MODE_SEPT)), "class modes");
     static_assert(!SC || MODE == MODE_PAIR || MODE == MODE_QUAD, "fused shortcut modes");
     using C = Cfg<KAPPA, BNQ, MODE>;
     constexpr int STAGES = C::STAGES;
@@ -183,7 +246,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         fence_barrier_init();
     }
     if (warp == 0 && lane == 0) {
-        tma_prefetch_desc(&tmap_x);
+        if constexpr (PAR)
+            for (int c = 0; c < par.ncls; ++c) tma_prefetch_desc(&par.x[c]);
+        else
+            tma_prefetch_desc(&tmap_x);
         tma_prefetch_desc(&tmap_wr);
         tma_prefetch_desc(&tmap_wi);
         tma_prefetch_desc(&tmap_wj);
@@ -216,18 +282,41 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             Unit unit;
             while (ok && units.next(unit)) {
                 const int tile = unit.tile;
-                const int m_tile = tile / p.num_n_tiles;
-                const int n_tile = tile - m_tile * p.num_n_tiles;
-                const long long m0 = static_cast<long long>(m_tile) * BM;
-                const int img = static_cast<int>(m0 / hw);
-                const int rem = static_cast<int>(m0 - static_cast<long long>(img) * hw);
-                const int ho = rem / s.Wo, wo = rem - (rem / s.Wo) * s.Wo;
-                const int wbase = wo * s.stride - s.pad, hbase = ho * s.stride - s.pad;
+                int m_tile = tile / p.num_n_tiles;
+                int n_tile = tile - m_tile * p.num_n_tiles;
+                const CUtensorMap* map_x = &tmap_x;
+                int img, wbase, hbase;
+                int kw = s.kw, tap0 = 0, tap_h = s.kw, tap_w = 1;
+                if constexpr (PAR) {
+                    const int ci = par_class(par, tile);
+                    const PixClass& c = par.cls[ci];
+                    const int t = tile - c.tile0;
+                    m_tile = t / p.num_n_tiles;
+                    n_tile = t - m_tile * p.num_n_tiles;
+                    const int r = m_tile * BM / c.Wc;
+                    img = r / c.Hc;
+                    wbase = m_tile * BM - r * c.Wc + c.w0;
+                    hbase = r - img * c.Hc + c.h0;
+                    map_x = &par.x[ci];
+                    kw = c.kw;
+                    tap0 = c.tap0;
+                    tap_h = c.tap_h;
+                    tap_w = c.tap_w;
+                    unit.k1 = c.ktiles;
+                } else {
+                    const long long m0 = static_cast<long long>(m_tile) * BM;
+                    img = static_cast<int>(m0 / hw);
+                    const int rem = static_cast<int>(m0 - static_cast<long long>(img) * hw);
+                    const int ho = rem / s.Wo, wo = rem - (rem / s.Wo) * s.Wo;
+                    wbase = wo * s.stride - s.pad;
+                    hbase = ho * s.stride - s.pad;
+                }
                 // K block kt = (tap, chunk), tap = dh * kw + dw: walked without divisions
                 // from the unit's first block
                 int tap = unit.k0 / p.kchunks;
                 int chunk = unit.k0 - tap * p.kchunks;
                 int dh = tap / s.kw, dw = tap - (tap / s.kw) * s.kw;
+                if constexpr (PAR) tap = tap0;  // (classes run whole tiles: k0 = 0)
                 int k1 = unit.k1;
                 bool sct = false;  // a fused shortcut's tile: one tap, its own letters
                 if constexpr (SC) {
@@ -246,10 +335,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     } else if (kt > unit.k0 && ++chunk == p.kchunks) {
                         chunk = 0;
                         ++tap;
-                        if (++dw == s.kw) {
+                        if (++dw == kw) {
                             dw = 0;
                             ++dh;
                         }
+                        if constexpr (PAR) tap = tap0 + dh * tap_h + dw * tap_w;
                     }
                     if (!wait_or_abort(empty_bar(stage), phase ^ 1u, limit, abort_flag,
                                        STATUS_TIMEOUT_PRODUCER)) {
@@ -267,7 +357,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     if (role == 0) {
 #pragma unroll
                         for (int comp = 0; comp < 4; ++comp)
-                            tma_load_im2col_4d(a0 + comp * C::A_TILE, &tmap_x, fb,
+                            tma_load_im2col_4d(a0 + comp * C::A_TILE, map_x, fb,
                                                comp * s.Qin + cin0, wbase, hbase, img,
                                                static_cast<uint16_t>(dw),
                                                static_cast<uint16_t>(dh), pol_x);
@@ -347,6 +437,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 int k1 = unit.k1;
                 if constexpr (SC)
                     if (unit.tile % p.num_n_tiles >= p.sc.n_conv) k1 = p.sc.ktiles;
+                if constexpr (PAR) k1 = par.cls[par_class(par, unit.tile)].ktiles;
                 for (int kt = unit.k0; kt < k1; ++kt) {
                     // pixels and letter tiles landed (pair mode: with the negated copies)
                     if (!flag_wait_or_abort(ready_word(stage), round + 1u, limit, abort_flag,
@@ -442,6 +533,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             int k1 = unit.k1;
             if constexpr (SC)
                 if (unit.tile % p.num_n_tiles >= p.sc.n_conv) k1 = p.sc.ktiles;
+            if constexpr (PAR) k1 = par.cls[par_class(par, unit.tile)].ktiles;
             for (int kt = unit.k0; kt < k1; ++kt) {
                 if (!wait_or_abort(fullw_bar(stage), phase, limit, abort_flag,
                                    STATUS_TIMEOUT_PRODUCER)) {
@@ -495,9 +587,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         else if constexpr (SC)
             epilogue_direct_pair_sc<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
                                          p.ktiles, p.sk, limit, abort_flag, geo, &p.sc);
+        else if constexpr (PAR)
+            epilogue_direct_pair<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
+                                      p.ktiles, p.sk, limit, abort_flag,
+                                      ParGeo{par, p.num_n_tiles});
         else
             epilogue_direct_pair<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
-                                      p.ktiles, p.sk, limit, abort_flag, geo);
+                                      p.ktiles, p.sk, limit, abort_flag, linear_geo(geo));
     }
 
     tc_fence_before();
@@ -545,17 +641,15 @@ CUtensorMapSwizzle swizzle_for_row(int row_bytes) {
                                                : CU_TENSOR_MAP_SWIZZLE_32B);
 }
 
-// Activation im2col map: boxes of BM output pixels x `channels` channels.
-bool encode_x_im2col(CUtensorMap* map, const ConvShape& s, const void* x, int channels) {
+// im2col map over x: boxes of BM pixels x `channels` channels, walking the filter origins
+// from (lower) to (dim - 1 + upper) of each spatial dimension, innermost (W) first.
+bool encode_im2col(CUtensorMap* map, const ConvShape& s, const void* x, int channels,
+                   const int lower[2], const int upper[2]) {
     const cuuint64_t dims[4] = {static_cast<cuuint64_t>(s.Cin), static_cast<cuuint64_t>(s.W),
                                 static_cast<cuuint64_t>(s.H), static_cast<cuuint64_t>(s.N)};
     const cuuint64_t strides[3] = {static_cast<cuuint64_t>(s.Cin) * 2,
                                    static_cast<cuuint64_t>(s.Cin) * 2 * s.W,
                                    static_cast<cuuint64_t>(s.Cin) * 2 * s.W * s.H};
-    // Bounding box of filter origins: from -pad to (dim - 1) + pad - (k - 1), per
-    // spatial dimension, innermost (W) first.
-    const int lower[2] = {-s.pad, -s.pad};
-    const int upper[2] = {s.pad - (s.kw - 1), s.pad - (s.kh - 1)};
     const cuuint32_t estr[4] = {1, static_cast<cuuint32_t>(s.stride),
                                 static_cast<cuuint32_t>(s.stride), 1};
     const CUresult r = g_encode_im2col(
@@ -564,6 +658,13 @@ bool encode_x_im2col(CUtensorMap* map, const ConvShape& s, const void* x, int ch
         swizzle_for_row(channels * 2), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
+}
+
+// Activation im2col map: boxes of BM output pixels x `channels` channels.
+bool encode_x_im2col(CUtensorMap* map, const ConvShape& s, const void* x, int channels) {
+    const int lower[2] = {-s.pad, -s.pad};
+    const int upper[2] = {s.pad - (s.kw - 1), s.pad - (s.kh - 1)};
+    return encode_im2col(map, s, x, channels, lower, upper);
 }
 
 // Activation tiled map for halo boxes: `channels` x `cols` columns (Wo if 0) x `rows` rows
@@ -637,21 +738,22 @@ cudaError_t set_smem_once(K kern, int bytes, std::atomic<unsigned long long>& do
     return cudaSuccess;
 }
 
-template <int KAPPA, int BNQ, int MODE, bool SC = false>
+template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false>
 cudaError_t launch_cfg(const CUtensorMap maps[6], const TcParams& prm, int grid,
-                       cudaStream_t stream, const ScMaps* scm = nullptr) {
+                       cudaStream_t stream, const ScMaps* scm = nullptr,
+                       const ParOf<PAR>& par = {}) {
     using C = Cfg<KAPPA, BNQ, MODE>;
     if constexpr (!C::FITS || (SC && MODE != MODE_PAIR && MODE != MODE_QUAD)) {
         return cudaErrorInvalidValue;
     } else {
-        auto kern = qconv_tc_kernel<KAPPA, BNQ, MODE, SC>;
+        auto kern = qconv_tc_kernel<KAPPA, BNQ, MODE, SC, PAR>;
         static std::atomic<unsigned long long> attr_done{0};
         cudaError_t e = set_smem_once(kern, C::SMEM_BYTES, attr_done);
         if (e != cudaSuccess) return e;
         ScMaps none;
         memset(&none, 0, sizeof(none));
         return launch_pdl(kern, dim3(grid), dim3(NUM_THREADS), C::SMEM_BYTES, stream, maps[0],
-                          maps[1], maps[2], maps[3], maps[4], prm, scm != nullptr ? *scm : none);
+                          maps[1], maps[2], maps[3], maps[4], prm, scm != nullptr ? *scm : none, par);
     }
 }
 
@@ -733,6 +835,25 @@ int grid_for(const TcOptions& opt, int num_sms, int num_tiles) {
     int grid = opt.max_ctas > 0 ? opt.max_ctas : num_sms;
     if (grid > num_tiles) grid = num_tiles;
     return grid < 1 ? 1 : grid;
+}
+
+// Channel tile of the class form: the BNQ dividing Qout with the fewest estimated clocks over
+// the waves of tiles.  Per 16 input channels a tile's copies (16 KB of pixels, 128 BNQ bytes of
+// letters, at about 33 bytes per clock and SM with every SM loading) outlast its MMAs.
+int par_pick_bnq(int Qout, long long m_tiles, int sms) {
+    const int bs[3] = {64, 32, 16}, cost[3] = {727, 606, 545};
+    int best = 16;
+    double best_t = 1e30;
+    for (int i = 0; i < 3; ++i) {
+        if (Qout % bs[i] != 0) continue;
+        const long long tiles = m_tiles * (Qout / bs[i]);
+        const double t = static_cast<double>((tiles + sms - 1) / sms) * cost[i];
+        if (t < best_t) {
+            best_t = t;
+            best = bs[i];
+        }
+    }
+    return best;
 }
 
 template <bool HALO, int KH, int NI, bool SEP>
@@ -1620,6 +1741,151 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     QUAN_TC_CASE(64, 64)
 #undef QUAN_TC_CASE
     snprintf(err, errlen, "no kernel instance for kappa=%d bnq=%d mode=%d", kappa, bnq, mode);
+    return cudaErrorInvalidValue;
+}
+
+// Input gradient of the stride-2 forward convolution f, from dy with the letters w in the
+// transformed layout [Qin][kh][kw][Qout] (rotated; conjugated for the full form), on the
+// pixel classes above.  false: no class form for this shape.
+bool tc_parity_supported(const ConvShape& f) {
+    if (f.stride != 2 || f.Qin % 16 != 0 || f.Qout % 16 != 0) return false;
+    // im2col corner offsets and filter offsets within their encodings
+    return f.kh <= 128 && f.kw <= 128 && f.pad < f.kh && f.pad < f.kw &&
+           static_cast<long long>(f.N) * f.H * f.W < 0x7fffffffLL - BM;
+}
+
+cudaError_t launch_qconv_tc_parity(const ConvShape& f, const void* dy, const void* const w[4],
+                                   void* dx, const TcOptions& opt, int num_sms,
+                                   cudaStream_t stream, char* err, size_t errlen) {
+    if (!load_encoders()) {
+        snprintf(err, errlen, "tensor-map encoders unavailable from the CUDA driver");
+        return cudaErrorNotSupported;
+    }
+    // the stride-1 convolution of dy as a layer: Cout -> Cin channels
+    ConvShape s = f;
+    s.H = f.Ho; s.W = f.Wo; s.Cin = f.Cout; s.Cout = f.Cin; s.Qin = f.Qout; s.Qout = f.Qin;
+    s.stride = 1;
+    s.act = 0;
+    const int kappa = s.Qin % 32 == 0 ? 32 : 16;
+    ParArgs par = {};
+    par.H = f.H;
+    par.W = f.W;
+    const int kchunks = s.Qin / kappa;
+    // the parity classes, most taps first
+    struct Side { int n, taps, first, pad; } sh[2], sw[2];
+    for (int a = 0; a < 2; ++a) {
+        auto side = [&](int dim, int k) {
+            Side r;
+            const int e = (a + f.pad) & 1;       // taps dh = 2 u + e reach this parity
+            r.n = (dim - a + 1) / 2;             // outputs
+            r.taps = e < k ? (k - e + 1) / 2 : 0;
+            r.first = k - 1 - e - 2 * (r.taps - 1);           // rotated index of the first tap
+            r.pad = r.taps - 1 - (a + f.pad - e) / 2;         // zero padding before row 0
+            return r;
+        };
+        sh[a] = side(f.H, f.kh);
+        sw[a] = side(f.W, f.kw);
+    }
+    int order[4] = {0, 1, 2, 3};
+    for (int i = 1; i < 4; ++i)
+        for (int j = i; j > 0; --j) {
+            auto taps = [&](int c) { return sh[c >> 1].taps * sw[c & 1].taps; };
+            if (taps(order[j]) <= taps(order[j - 1])) break;
+            const int t = order[j];
+            order[j] = order[j - 1];
+            order[j - 1] = t;
+        }
+    long long m_tiles = 0;
+    for (int c = 0; c < 4; ++c)
+        m_tiles += (static_cast<long long>(f.N) * sh[c >> 1].n * sw[c & 1].n + BM - 1) / BM;
+    const int bnq = s.sep ? pick_bnq(s.Qout, 0)
+                          : par_pick_bnq(s.Qout, m_tiles, opt.max_ctas > 0 ? opt.max_ctas : num_sms);
+    const int num_n = s.Qout / bnq;
+    if (m_tiles * num_n > 0x7fffffffLL) {
+        snprintf(err, errlen, "too many tiles");
+        return cudaErrorInvalidValue;
+    }
+    int tiles = 0;
+    for (int i = 0; i < 4; ++i) {
+        const int a = order[i] >> 1, b = order[i] & 1;
+        const long long M = static_cast<long long>(f.N) * sh[a].n * sw[b].n;
+        if (M == 0) continue;
+        PixClass& c = par.cls[par.ncls];
+        c.Hc = sh[a].n; c.Wc = sw[b].n;
+        c.kh = sh[a].taps; c.kw = sw[b].taps;
+        if (c.kh == 0 || c.kw == 0) c.kh = c.kw = 0;
+        c.tap0 = sh[a].first * f.kw + sw[b].first;
+        c.tap_h = 2 * f.kw;
+        c.tap_w = 2;
+        c.h0 = -sh[a].pad;
+        c.w0 = -sw[b].pad;
+        c.ktiles = c.kh * c.kw * kchunks;
+        c.tile0 = tiles;
+        c.oh = a; c.ow = b;
+        c.M = M;
+        tiles += static_cast<int>((M + BM - 1) / BM) * num_n;
+        ++par.ncls;
+    }
+    const MapKey kx = make_key(f, dy, w, dx, kappa, bnq, 30);
+    const MapKey kl = make_key(f, dy, w, dx, kappa, bnq, 31);
+    CUtensorMap mx[6], maps[6];
+    if (!cache_lookup(kx, mx)) {
+        bool ok = true;
+        for (int i = 0; ok && i < par.ncls; ++i) {
+            const PixClass& c = par.cls[i];
+            const int lower[2] = {c.w0, c.h0};
+            const int upper[2] = {c.Wc - f.Wo + c.w0, c.Hc - f.Ho + c.h0};
+            if (c.ktiles == 0)
+                mx[i] = mx[0];  // never loaded from
+            else
+                ok = encode_im2col(&mx[i], s, dy, kappa, lower, upper);
+        }
+        for (int i = par.ncls; i < 6; ++i) mx[i] = mx[0];
+        if (!ok) {
+            snprintf(err, errlen, "tensor-map encode failed for the output gradient");
+            return cudaErrorInvalidValue;
+        }
+        cache_store(kx, mx);
+    }
+    if (!cache_lookup(kl, maps)) {
+        bool ok = true;
+        for (int l = 0; ok && l < 4; ++l) ok = encode_w(&maps[1 + l], s, w[l], kappa, bnq);
+        if (!ok) {
+            snprintf(err, errlen, "tensor-map encode failed for the letters");
+            return cudaErrorInvalidValue;
+        }
+        maps[0] = maps[5] = mx[0];
+        cache_store(kl, maps);
+    }
+    for (int i = 0; i < par.ncls; ++i) par.x[i] = mx[i];
+    TcParams prm = {};
+    prm.s = s;
+    prm.ep = EpilogueArgs{nullptr, nullptr, nullptr, nullptr};
+    prm.kchunks = kchunks;
+    prm.ktiles = par.cls[0].ktiles;
+    prm.num_n_tiles = num_n;
+    prm.num_tiles = tiles;
+    prm.y = dx;
+    prm.wait_limit_ns = opt.wait_limit_ns;
+    prm.inject_stall = opt.inject_stall;
+    const int grid = grid_for(opt, num_sms, tiles);
+    set_kernel_name(s.sep ? "qconv_tc_kernel<sep_t,kappa=%d,bnq=%d,parity>"
+                          : "qconv_tc_kernel<pair,kappa=%d,bnq=%d,parity>",
+                    kappa, bnq);
+#define QUAN_PAR_CASE(K, B)                                                                \
+    if (kappa == K && bnq == B)                                                            \
+        return s.sep ? launch_cfg<K, B, MODE_SEPT, false, true>(maps, prm, grid, stream,    \
+                                                                nullptr, par)              \
+                     : launch_cfg<K, B, MODE_PAIR, false, true>(maps, prm, grid, stream,    \
+                                                                nullptr, par);
+    QUAN_PAR_CASE(16, 16)
+    QUAN_PAR_CASE(16, 32)
+    QUAN_PAR_CASE(16, 64)
+    QUAN_PAR_CASE(32, 16)
+    QUAN_PAR_CASE(32, 32)
+    QUAN_PAR_CASE(32, 64)
+#undef QUAN_PAR_CASE
+    snprintf(err, errlen, "no kernel instance for kappa=%d bnq=%d", kappa, bnq);
     return cudaErrorInvalidValue;
 }
 

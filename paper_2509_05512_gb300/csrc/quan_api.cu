@@ -247,7 +247,8 @@ quan_status_t run_bwd_data(const void* dy, const void* const w[4], int N, int H,
                  (!strided || workspace_bytes >= (need + 255) / 256 * 256 + ub) &&
                  geometry(&t, N, strided ? Hu : s.Ho, strided ? Wu : s.Wo, Cout, Cin, kh, kw, 1,
                           kh - 1 - pad) == QUAN_OK &&
-                 t.Ho == H && t.Wo == W && quan::tc_supported(t, src, tw, dx, none);
+                 t.Ho == H && t.Wo == W && quan::tc_supported(t, src, tw, dx, none) &&
+                 reinterpret_cast<uintptr_t>(dy) % 16 == 0;
     // separable form: the transposed-separable MMA mode (Qin, Qout multiples of 16)
     if (separable) t.sep = 2;
     if (separable && (Cin % 64 != 0 || Cout % 64 != 0)) tc_ok = false;
@@ -261,11 +262,6 @@ quan_status_t run_bwd_data(const void* dy, const void* const w[4], int N, int H,
         e = quan::launch_bwd_transform(Cin, Cout, kh, kw, w, !separable, workspace, num_sms,
                                        cs);
         if (e != cudaSuccess) return cuda_fail(e, "bwd_transform launch");
-        if (strided) {
-            e = quan::launch_bwd_upsample(dy, N, s.Ho, s.Wo, Cout, stride, Hu, Wu, u, num_sms,
-                                          cs);
-            if (e != cudaSuccess) return cuda_fail(e, "bwd_upsample launch");
-        }
         quan::TcOptions opt;
         opt.kappa = g_kappa.load();
         opt.bnq = g_bnq.load();
@@ -279,7 +275,21 @@ quan_status_t run_bwd_data(const void* dy, const void* const w[4], int N, int H,
         opt.wait_limit_ns = g_wait_limit.load();
         opt.inject_stall = g_inject.load();
         char err[256] = "";
-        e = quan::launch_qconv_tc(t, src, tw, none, dx, opt, num_sms, cs, err, sizeof(err));
+        // stride 2: the parity classes of dx's pixels (no tile overrides); other strides
+        // spread dy out
+        quan::ConvShape f = s;
+        f.sep = t.sep;
+        const bool parity = strided && opt.kappa == 0 && opt.bnq == 0 && opt.mode == 0 &&
+                            quan::tc_parity_supported(f);
+        if (strided && !parity) {
+            e = quan::launch_bwd_upsample(dy, N, s.Ho, s.Wo, Cout, stride, Hu, Wu, u, num_sms,
+                                          cs);
+            if (e != cudaSuccess) return cuda_fail(e, "bwd_upsample launch");
+        }
+        if (parity)
+            e = quan::launch_qconv_tc_parity(f, dy, tw, dx, opt, num_sms, cs, err, sizeof(err));
+        else
+            e = quan::launch_qconv_tc(t, src, tw, none, dx, opt, num_sms, cs, err, sizeof(err));
         if (err[0] != '\0') return fail(QUAN_ERR_UNSUPPORTED, "%s", err);
         if (e != cudaSuccess) return cuda_fail(e, "qconv_tc launch");
         t_last_path = QUAN_PATH_TC;

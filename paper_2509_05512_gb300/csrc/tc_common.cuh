@@ -176,6 +176,21 @@ struct EpiTile {
     int n_tile;    // quaternion output channel block
 };
 
+// Tile geometry functors of the QUAD/PAIR kernel's epilogue: tile index -> EpiTile, the output
+// pixel of a tile's row (kScattered; else consecutive pixels from m0), and whether a tile has
+// no K blocks (its accumulator is never written and the output is zero).
+template <typename TileOf>
+struct LinearGeo {  // tiles of consecutive output pixels
+    static constexpr bool kScattered = false;
+    TileOf tile_of;
+    __device__ __forceinline__ EpiTile operator()(int tile) const { return tile_of(tile); }
+    __device__ __forceinline__ bool empty(int) const { return false; }
+};
+template <typename TileOf>
+__device__ __forceinline__ LinearGeo<TileOf> linear_geo(TileOf f) {
+    return LinearGeo<TileOf>{f};
+}
+
 // Direct epilogue for 64-channel outputs (Qout = 16: one output-channel tile), used by the
 // weight-stationary and pixel-pair kernels (16 warps: producer, 3 issuers, 12 epilogue).
 // The tensor cores' operand reads keep the shared-memory pipe saturated, so this epilogue
@@ -455,6 +470,17 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
         const EpiTile g = geo(tile);
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) +
                                static_cast<uint32_t>(buf * 4 * BNQ);
+        const bool empty = geo.empty(tile);
+        // output pixels of this lane's rows
+        [[maybe_unused]] long long pixels[NCH];
+        if constexpr (Geo::kScattered) {
+#pragma unroll
+            for (int k = 0; k < NCH; ++k) pixels[k] = geo.pixel(g, tile, row0 + k);
+        }
+        auto pix = [&](int k) {
+            if constexpr (Geo::kScattered) return pixels[k];
+            return g.m0 + row0 + k;
+        };
         const int c_tile = g.n_tile * BNQ + 8 * ci;  // + q Qout + slice offset: lane's channel
         uint32_t va[CH], vb[CH];
         float sca[8], sha[8], scb[8], shb[8];
@@ -481,6 +507,10 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
                 // the tile's accumulator is in registers: hand the buffer back
                 tc_fence_before();
                 mbar_arrive_relaxed(acce0 + 8u * buf);
+            }
+            if (empty) {
+#pragma unroll
+                for (int j = 0; j < CH; ++j) v[j] = 0u;
             }
             if (unit.kind == UNIT_HEAD) {
                 // this CTA's share of the tile: the raw accumulator to the partial slot (L2)
@@ -512,7 +542,7 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
                 for (int k = 0; k < NCH; ++k) {
                     r4[k] = make_uint4(0u, 0u, 0u, 0u);
                     if (row0 + k < g.rows)
-                        r4[k] = ld_global_na(res + (g.m0 + row0 + k) * Cout + cb);
+                        r4[k] = ld_global_na(res + pix(k) * Cout + cb);
                 }
             }
             float E[NCH][8];  // E[j][e]: channel 8 j + e of this lane's row
@@ -551,7 +581,7 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
                     w[t] = pack_bf16x2(activate(z0, s.act), activate(z1, s.act));
                 }
                 if (row0 + k < g.rows)
-                    st_global_na(out + (g.m0 + row0 + k) * Cout + cb,
+                    st_global_na(out + pix(k) * Cout + cb,
                                  make_uint4(w[0], w[1], w[2], w[3]));
             }
             if (b + 1 < NB) tmem_ld_wait();

@@ -141,6 +141,30 @@ def test_bwd_data_tensor_cores(case):
     assert_bf16_close(got, oracle_bwd_data(d), name + " dx")
 
 
+PARITY_DATA_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad: stride 2 by the parity classes of dx's pixels
+    ("par_one_row", 3, 1, 17, 64, 64, 3, 2, 1),      # no odd row
+    ("par_one_col", 2, 14, 1, 128, 64, 3, 2, 1),     # no odd column
+    ("par_k1_odd", 2, 13, 15, 64, 192, 1, 2, 0),     # three classes no tap reaches: zeros
+    ("par_pad0", 1, 9, 8, 64, 128, 3, 2, 0),         # the last row is not read
+    ("par_pad2", 1, 8, 9, 128, 64, 3, 2, 2),         # classes that start past dy's edge
+    ("par_k2", 2, 10, 12, 64, 64, 2, 2, 0),
+    ("par_k5_pad4", 1, 11, 10, 64, 64, 5, 2, 4),
+    ("par_tiles", 5, 30, 29, 256, 128, 3, 2, 1),     # several tiles and a tail per class
+    ("par_wrap", 24, 60, 58, 64, 64, 3, 2, 1),       # more tiles than SMs
+]
+
+
+@pytest.mark.parametrize("sep", [False, True], ids=["full", "sep"])
+@pytest.mark.parametrize("case", PARITY_DATA_CASES, ids=[c[0] for c in PARITY_DATA_CASES])
+def test_bwd_data_parity_classes(case, sep):
+    name, N, H, W, Cin, Cout, k, s, p = case
+    d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(615, len(name))))
+    got, path, kernel = gpu_bwd_data(d, separable=sep, path=quan.QUAN_PATH_TC)
+    assert path == quan.QUAN_PATH_TC and kernel.endswith(",parity>"), kernel
+    assert_bf16_close(got, oracle_bwd_data(d, sep), name + " dx")
+
+
 SIMT_CASES = [
     ("stride2", 2, 15, 17, 64, 128, 3, 2, 1),
     ("stride2_even", 1, 16, 16, 64, 64, 3, 2, 1),
