@@ -68,9 +68,10 @@ typedef enum {
 typedef enum { QUAN_ACT_NONE = 0, QUAN_ACT_RELU = 1, QUAN_ACT_SILU = 2 } quan_act_t;
 
 typedef enum {
-    QUAN_PATH_AUTO = 0, /* tensor-core path when the shape allows it, else CUDA cores */
+    QUAN_PATH_AUTO = 0, /* tensor-core path when the shape allows it, else as SIMT */
     QUAN_PATH_TC = 1,   /* tcgen05 implicit GEMM; UNSUPPORTED if the shape does not allow it */
-    QUAN_PATH_SIMT = 2  /* CUDA-core direct convolution */
+    QUAN_PATH_SIMT = 2  /* kernels without tcgen05: fp32 on CUDA cores, bf16 on warp-level MMAs
+                           (CUDA cores where those do not apply) */
 } quan_path_t;
 
 /*

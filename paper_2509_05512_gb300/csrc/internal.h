@@ -83,9 +83,23 @@ const char* last_tc_kernel();
 
 // CUDA-core path, any shape; T = __nv_bfloat16 or float.
 cudaError_t launch_qconv_simt_bf16(const ConvShape& s, const void* x, const void* const w[4],
-                                   const EpilogueArgs& ep, void* out, cudaStream_t stream);
+                                   const EpilogueArgs& ep, void* out, int num_sms,
+                                   cudaStream_t stream);
 cudaError_t launch_qconv_simt_f32(const ConvShape& s, const void* x, const void* const w[4],
-                                  const EpilogueArgs& ep, void* out, cudaStream_t stream);
+                                  const EpilogueArgs& ep, void* out, int num_sms,
+                                  cudaStream_t stream);
+
+// Warp-level tensor-core kernels (mma.sync) for bf16 layers off the tcgen05 kernels' channel
+// grid: the convolution, its input gradient and its weight gradient (zeroes dW_L, then adds).
+bool mma_fwd_supported(const ConvShape& s, const void* x, const void* out, const void* residual);
+cudaError_t launch_mma_fwd(const ConvShape& s, const void* x, const void* const w[4],
+                           const EpilogueArgs& ep, void* out, int num_sms, cudaStream_t stream);
+bool mma_bwd_data_supported(const ConvShape& s, const void* dy, const void* dx);
+cudaError_t launch_mma_bwd_data(const ConvShape& s, const void* dy, const void* const w[4],
+                                void* dx, int num_sms, cudaStream_t stream);
+bool mma_bwd_weight_supported(const ConvShape& s, const void* x, const void* dy);
+cudaError_t launch_mma_bwd_weight(const ConvShape& s, const void* x, const void* dy,
+                                  float* const dw[4], int num_sms, cudaStream_t stream);
 
 // Launch with programmatic stream serialization: the kernel may start while the previous
 // kernel in the stream is finishing (once all of that grid's CTAs have signalled), runs its
@@ -126,7 +140,7 @@ cudaError_t launch_bwd_upsample(const void* dy, int N, int Ho, int Wo, int C, in
                                 int Wu, void* u, int num_sms, cudaStream_t stream);
 // dx [N][H][W][Cin] from dy [N][Ho][Wo][Cout] on CUDA cores, any stride.
 cudaError_t launch_bwd_data_simt(const ConvShape& s, const void* dy, const void* const w[4],
-                                 void* dx, cudaStream_t stream);
+                                 void* dx, int num_sms, cudaStream_t stream);
 // Library-owned device scratch of quan_qconv2d_bwd_data_static (one per device, in the
 // module's static device memory): its size, and its address on the current device.
 constexpr size_t BWD_STATIC_SCRATCH_BYTES = size_t(2) << 20;

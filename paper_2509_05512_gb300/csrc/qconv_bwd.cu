@@ -14,9 +14,10 @@
 //     s - 1 zero rows and columns inserted between its pixels (bwd_upsample_kernel, into
 //     the workspace after the letters), when the caller's workspace would hold that tensor;
 //     otherwise the direct CUDA-core kernel below runs;
-//   * the weight gradient is a reduction over output pixels, done on CUDA cores: every
-//     thread owns one (co, tap, ci) quaternion of dW for a chunk of pixels and adds its
-//     fp32 partial sum to the zeroed output with atomicAdd.
+//   * the weight gradient is a reduction over output pixels: on the tensor cores
+//     (qconv_dw.cuh), or on CUDA cores chunk by chunk of pixels, fp32 partial sums added to
+//     the zeroed output with atomicAdd.
+// The CUDA-core kernels of both gradients are the tiled products of qgemm_simt.cuh.
 // Separable form (Eq. 7): Eq. 8-10 -- the output gradients are first mixed by the matrix M
 // of Eq. 9 (g_p = sum_m M[p][m] dy_m, M transposed equal to Eq. 7's sign table), then
 // dL/dx_p is the transposed convolution of g_p with W_p alone and dL/dW_p the correlation
@@ -26,24 +27,10 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "qgemm_simt.cuh"
 
 namespace quan {
 namespace {
-
-__device__ __forceinline__ float bf(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-
-// g = M dy for one output channel, M of Eq. 9 (rows p, columns m):
-//   [ 1  1  1  1 ]
-//   [-1  1 -1  1 ]
-//   [-1  1  1 -1 ]
-//   [-1 -1  1  1 ]
-__device__ __forceinline__ void mix_eq9(float dr, float di, float dj, float dk, float& gr,
-                                        float& gi, float& gj, float& gk) {
-    gr = dr + di + dj + dk;
-    gi = -dr + di - dj + dk;
-    gj = -dr + di + dj - dk;
-    gk = -dr - di + dj + dk;
-}
 
 // out_L[ci][dh][dw][co] = s_L * W_L[co][kh-1-dh][kw-1-dw][ci], s = (+1, -1, -1, -1) when
 // conj, else +1.  Its output is the next kernel's weight operand, which the forward
@@ -71,124 +58,6 @@ __global__ void __launch_bounds__(256) bwd_transform_kernel(
         const __nv_bfloat16 v = w[L][src];
         out[i] = (L == 0 || !conj) ? v : __hneg(v);
     }
-}
-
-// dx for one (pixel, input quaternion channel), any stride and padding: the sum over taps
-// and output channels of conj(W) (x) dy (full form), or of W_p g_p per component p
-// (separable form, g = M dy).
-template <bool SEP>
-__global__ void __launch_bounds__(256) bwd_data_simt_kernel(
-    ConvShape s, const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ wr,
-    const __nv_bfloat16* __restrict__ wi, const __nv_bfloat16* __restrict__ wj,
-    const __nv_bfloat16* __restrict__ wk, __nv_bfloat16* __restrict__ dx) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const long long total = static_cast<long long>(s.N) * s.H * s.W * s.Qin;
-    const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    const int ci = static_cast<int>(idx % s.Qin);
-    const long long pix = idx / s.Qin;
-    const int w = static_cast<int>(pix % s.W);
-    const int h = static_cast<int>((pix / s.W) % s.H);
-    const int n = static_cast<int>(pix / (static_cast<long long>(s.W) * s.H));
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int dh = 0; dh < s.kh; ++dh) {
-        const int th = h + s.pad - dh;  // ho * stride
-        if (th < 0 || th % s.stride != 0) continue;
-        const int ho = th / s.stride;
-        if (ho >= s.Ho) continue;
-        for (int dw = 0; dw < s.kw; ++dw) {
-            const int tw = w + s.pad - dw;
-            if (tw < 0 || tw % s.stride != 0) continue;
-            const int wo = tw / s.stride;
-            if (wo >= s.Wo) continue;
-            const __nv_bfloat16* g = dy + ((static_cast<long long>(n) * s.Ho + ho) * s.Wo + wo) *
-                                              s.Cout;
-            for (int co = 0; co < s.Qout; ++co) {
-                const long long widx = ((static_cast<long long>(co) * s.kh + dh) * s.kw + dw) *
-                                           s.Qin + ci;
-                const float dr = bf(g + co), di = bf(g + s.Qout + co);
-                const float dj = bf(g + 2 * s.Qout + co), dk = bf(g + 3 * s.Qout + co);
-                if constexpr (SEP) {
-                    float gr, gi, gj, gk;
-                    mix_eq9(dr, di, dj, dk, gr, gi, gj, gk);
-                    a0 += bf(wr + widx) * gr;
-                    a1 += bf(wi + widx) * gi;
-                    a2 += bf(wj + widx) * gj;
-                    a3 += bf(wk + widx) * gk;
-                } else {
-                    // conj(W) = (a, -b, -c, -d); conj(W) (x) dy by Eq. 3
-                    const float a = bf(wr + widx), b = -bf(wi + widx);
-                    const float c = -bf(wj + widx), d = -bf(wk + widx);
-                    a0 += a * dr - b * di - c * dj - d * dk;
-                    a1 += a * di + b * dr + c * dk - d * dj;
-                    a2 += a * dj - b * dk + c * dr + d * di;
-                    a3 += a * dk + b * dj - c * di + d * dr;
-                }
-            }
-        }
-    }
-    __nv_bfloat16* o = dx + pix * s.Cin;
-    o[ci] = __float2bfloat16_rn(a0);
-    o[s.Qin + ci] = __float2bfloat16_rn(a1);
-    o[2 * s.Qin + ci] = __float2bfloat16_rn(a2);
-    o[3 * s.Qin + ci] = __float2bfloat16_rn(a3);
-}
-
-// dW for one (co, tap, ci) quaternion over the output pixels of chunk blockIdx.y: the sum
-// of dy (x) conj(X) (full form), or of g_p x_p per component p (separable form, g = M dy),
-// added to the fp32 outputs.
-template <bool SEP>
-__global__ void __launch_bounds__(256) bwd_weight_simt_kernel(
-    ConvShape s, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
-    long long chunk, float* __restrict__ dwr, float* __restrict__ dwi, float* __restrict__ dwj,
-    float* __restrict__ dwk) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int taps = s.kh * s.kw;
-    const long long outs = static_cast<long long>(s.Qout) * taps * s.Qin;
-    const long long o = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (o >= outs) return;
-    // o = (co * taps + tap) * Qin + ci, the layout of the letter tensors
-    const int ci = static_cast<int>(o % s.Qin);
-    const int tap = static_cast<int>((o / s.Qin) % taps);
-    const int co = static_cast<int>(o / (static_cast<long long>(s.Qin) * taps));
-    const int dh = tap / s.kw, dw = tap - (tap / s.kw) * s.kw;
-    const long long p0 = blockIdx.y * chunk;
-    long long p1 = p0 + chunk;
-    if (p1 > s.M) p1 = s.M;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (long long p = p0; p < p1; ++p) {
-        const int wo = static_cast<int>(p % s.Wo);
-        const int ho = static_cast<int>((p / s.Wo) % s.Ho);
-        const int n = static_cast<int>(p / (static_cast<long long>(s.Wo) * s.Ho));
-        const int h = ho * s.stride - s.pad + dh, w = wo * s.stride - s.pad + dw;
-        if (h < 0 || h >= s.H || w < 0 || w >= s.W) continue;
-        const __nv_bfloat16* xp = x + ((static_cast<long long>(n) * s.H + h) * s.W + w) * s.Cin;
-        const __nv_bfloat16* g = dy + p * s.Cout;
-        const float xr = bf(xp + ci), xi = bf(xp + s.Qin + ci);
-        const float xj = bf(xp + 2 * s.Qin + ci), xk = bf(xp + 3 * s.Qin + ci);
-        const float dr = bf(g + co), di = bf(g + s.Qout + co);
-        const float dj = bf(g + 2 * s.Qout + co), dk = bf(g + 3 * s.Qout + co);
-        if constexpr (SEP) {
-            float gr, gi, gj, gk;
-            mix_eq9(dr, di, dj, dk, gr, gi, gj, gk);
-            a0 += gr * xr;
-            a1 += gi * xi;
-            a2 += gj * xj;
-            a3 += gk * xk;
-        } else {
-            // dy (x) conj(X), conj(X) = (xr, -xi, -xj, -xk), by Eq. 3
-            a0 += dr * xr + di * xi + dj * xj + dk * xk;
-            a1 += -dr * xi + di * xr - dj * xk + dk * xj;
-            a2 += -dr * xj + di * xk + dj * xr - dk * xi;
-            a3 += -dr * xk - di * xj + dj * xi + dk * xr;
-        }
-    }
-    atomicAdd(dwr + o, a0);
-    atomicAdd(dwi + o, a1);
-    atomicAdd(dwj + o, a2);
-    atomicAdd(dwk + o, a3);
 }
 
 // Scratch of quan_qconv2d_bwd_data_static, the entry point for callers that cannot
@@ -284,40 +153,51 @@ cudaError_t launch_bwd_transform(int Cin, int Cout, int kh, int kw, const void* 
 }
 
 cudaError_t launch_bwd_data_simt(const ConvShape& s, const void* dy, const void* const w[4],
-                                 void* dx, cudaStream_t stream) {
-    auto kern = s.sep ? bwd_data_simt_kernel<true> : bwd_data_simt_kernel<false>;
-    const long long total = static_cast<long long>(s.N) * s.H * s.W * s.Qin;
-    if (total == 0) return cudaSuccess;
-    const long long blocks = (total + 255) / 256;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    return launch_pdl(kern, dim3(static_cast<unsigned>(blocks)), dim3(256), 0,
-                      stream, s, static_cast<const __nv_bfloat16*>(dy),
-                      static_cast<const __nv_bfloat16*>(w[0]),
-                      static_cast<const __nv_bfloat16*>(w[1]),
-                      static_cast<const __nv_bfloat16*>(w[2]),
-                      static_cast<const __nv_bfloat16*>(w[3]), static_cast<__nv_bfloat16*>(dx));
+                                 void* dx, int num_sms, cudaStream_t stream) {
+    if (mma_bwd_data_supported(s, dy, dx))
+        return launch_mma_bwd_data(s, dy, w, dx, num_sms, stream);
+    qg::Params p = {};
+    p.s = s;
+    for (int l = 0; l < 4; ++l) p.a[l] = w[l];
+    p.b = dy;
+    p.out = dx;
+    // pixel classes: rows and columns modulo the stride (at most the image's); the largest
+    // is rows and columns 0, stride, 2 stride, ..
+    p.cw = s.W < s.stride ? s.W : s.stride;
+    const long long classes = static_cast<long long>(s.H < s.stride ? s.H : s.stride) * p.cw;
+    const long long J = static_cast<long long>(s.N) * ((s.H + s.stride - 1) / s.stride) *
+                        ((s.W + s.stride - 1) / s.stride);
+    return s.sep ? qg::launch<__nv_bfloat16, qg::DGRAD, true>(p, s.Qin, J, classes, num_sms, stream)
+                 : qg::launch<__nv_bfloat16, qg::DGRAD, false>(p, s.Qin, J, classes, num_sms,
+                                                               stream);
 }
 
 cudaError_t launch_bwd_weight_simt(const ConvShape& s, const void* x, const void* dy,
                                    float* const dw[4], int num_sms, cudaStream_t stream) {
-    const long long outs = static_cast<long long>(s.Qout) * s.kh * s.kw * s.Qin;
-    const cudaError_t e = launch_zero4(dw, outs, num_sms, stream);
+    if (mma_bwd_weight_supported(s, x, dy))
+        return launch_mma_bwd_weight(s, x, dy, dw, num_sms, stream);
+    const long long J = static_cast<long long>(s.kh) * s.kw * s.Qin;
+    const cudaError_t e = launch_zero4(dw, J * s.Qout, num_sms, stream);
     if (e != cudaSuccess) return e;
-    if (outs == 0 || s.M == 0) return cudaSuccess;
-    // enough pixel chunks to give every SM a few thousand threads
-    const long long oblocks = (outs + 255) / 256;
-    long long chunks = (static_cast<long long>(num_sms) * 16 + oblocks - 1) / oblocks;
-    if (chunks > s.M) chunks = s.M;
+    if (J == 0 || s.M == 0) return cudaSuccess;
+    qg::Params p = {};
+    p.s = s;
+    p.a[0] = dy;
+    p.b = x;
+    for (int l = 0; l < 4; ++l) p.dw[l] = dw[l];
+    // pixel chunks that give every SM about four blocks; more only adds atomics
+    qg::Params t = p;
+    qg::layout(&t, s.Qout, J, 2, 4);
+    const long long tiles = qg::jtiles(t, J) * t.itiles;
+    long long chunks = (4LL * num_sms + tiles - 1) / tiles;
+    if (chunks > (s.M + qg::KC - 1) / qg::KC) chunks = (s.M + qg::KC - 1) / qg::KC;
+    if (chunks < (s.M >> 30) + 1) chunks = (s.M >> 30) + 1;  // a chunk's pixels fit an int
     if (chunks > 65535) chunks = 65535;
-    if (chunks < 1) chunks = 1;
-    const long long chunk = (s.M + chunks - 1) / chunks;
-    chunks = (s.M + chunk - 1) / chunk;
-    if (oblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    auto kern = s.sep ? bwd_weight_simt_kernel<true> : bwd_weight_simt_kernel<false>;
-    return launch_pdl(kern,
-                      dim3(static_cast<unsigned>(oblocks), static_cast<unsigned>(chunks)),
-                      dim3(256), 0, stream, s, static_cast<const __nv_bfloat16*>(x),
-                      static_cast<const __nv_bfloat16*>(dy), chunk, dw[0], dw[1], dw[2], dw[3]);
+    p.chunk = ((s.M + chunks - 1) / chunks + qg::KC - 1) / qg::KC * qg::KC;
+    chunks = (s.M + p.chunk - 1) / p.chunk;
+    return s.sep ? qg::launch<__nv_bfloat16, qg::WGRAD, true>(p, s.Qout, J, chunks, num_sms, stream)
+                 : qg::launch<__nv_bfloat16, qg::WGRAD, false>(p, s.Qout, J, chunks, num_sms,
+                                                               stream);
 }
 
 }  // namespace quan

@@ -195,7 +195,7 @@ quan_status_t run_bf16(const void* x, const void* wr, const void* wi, const void
         t_last_path = QUAN_PATH_TC;
         t_last_kernel = quan::last_tc_kernel();
     } else {
-        e = quan::launch_qconv_simt_bf16(s, x, w, ep, out, cs);
+        e = quan::launch_qconv_simt_bf16(s, x, w, ep, out, num_sms, cs);
         if (e != cudaSuccess) return cuda_fail(e, "qconv_simt launch");
         t_last_path = QUAN_PATH_SIMT;
         t_last_kernel = s.sep ? "qconv_simt_kernel<bf16,sep>" : "qconv_simt_kernel<bf16>";
@@ -296,7 +296,7 @@ quan_status_t run_bwd_data(const void* dy, const void* const w[4], int N, int H,
         t_last_kernel = quan::last_tc_kernel();
         return QUAN_OK;
     }
-    e = quan::launch_bwd_data_simt(s, dy, w, dx, cs);
+    e = quan::launch_bwd_data_simt(s, dy, w, dx, num_sms, cs);
     if (e != cudaSuccess) return cuda_fail(e, "bwd_data_simt launch");
     t_last_path = QUAN_PATH_SIMT;
     t_last_kernel = separable ? "bwd_data_simt_kernel<sep>" : "bwd_data_simt_kernel";
@@ -482,8 +482,11 @@ quan_status_t quan_qconv2d_fwd_f32(const float* x, const float* wr, const float*
     if (g_path.load() == QUAN_PATH_TC)
         return fail(QUAN_ERR_UNSUPPORTED, "fp32 convolution runs on CUDA cores only");
     const quan::EpilogueArgs ep{bias, iqbn_scale, iqbn_shift, nullptr};
-    cudaError_t e = quan::launch_qconv_simt_f32(s, x, w, ep, out,
-                                                reinterpret_cast<cudaStream_t>(stream));
+    int num_sms = 0, cc = 0;
+    cudaError_t e;
+    if (!device_info(&num_sms, &cc, &e)) return cuda_fail(e, "device query");
+    e = quan::launch_qconv_simt_f32(s, x, w, ep, out, num_sms,
+                                    reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "qconv_simt_f32 launch");
     t_last_path = QUAN_PATH_SIMT;
     t_last_kernel = "qconv_simt_kernel<f32>";

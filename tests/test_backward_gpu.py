@@ -185,6 +185,36 @@ def test_bwd_data_cuda_cores(case):
     assert_bf16_close(got, oracle_bwd_data(d), name + " dx")
 
 
+EDGE_SIMT_CASES = [
+    # the warp-level MMA gradients: K and row tails, several row tiles, one and many pixel
+    # chunks, tap groups, strides beyond the filter
+    ("qs_one", 1, 1, 1, 4, 4, 1, 1, 0),
+    ("qs_q17", 2, 6, 5, 68, 68, 3, 1, 1),            # 17 rows: two row tiles
+    ("qs_q15_q1", 3, 11, 9, 60, 4, 3, 1, 1),
+    ("qs_many", 16, 45, 37, 24, 40, 3, 1, 1),
+    ("qs_groups", 2, 9, 8, 60, 60, 3, 1, 1),         # three groups of three taps
+    ("qs_s2_odd", 9, 33, 21, 20, 56, 3, 2, 1),
+    ("qs_s3_k1", 2, 10, 7, 12, 8, 1, 3, 0),          # eight classes no tap reaches
+    ("qs_s4_small", 2, 3, 2, 8, 12, 3, 4, 1),        # stride larger than the image
+    ("qs_k5_pad3", 1, 9, 12, 36, 20, 5, 2, 3),
+    # too wide for those: the tiled CUDA-core products
+    ("qs_core_s5", 1, 12, 11, 20, 28, 3, 5, 1),      # dx: more than 16 pixel classes
+    ("qs_core_c260", 1, 6, 5, 260, 8, 3, 1, 1),      # dW
+    ("qs_core_k", 1, 7, 6, 20, 132, 5, 1, 2),        # dx: K = 3300
+]
+
+
+@pytest.mark.parametrize("sep", [False, True], ids=["full", "sep"])
+@pytest.mark.parametrize("case", EDGE_SIMT_CASES, ids=[c[0] for c in EDGE_SIMT_CASES])
+def test_cuda_core_gradients(case, sep):
+    name, N, H, W, Cin, Cout, k, s, p = case
+    d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(616, len(name))))
+    got, path, _ = gpu_bwd_data(d, separable=sep, path=quan.QUAN_PATH_SIMT)
+    assert path == quan.QUAN_PATH_SIMT
+    assert_bf16_close(got, oracle_bwd_data(d, sep), name + " dx")
+    check_weight(d, separable=sep, path=quan.QUAN_PATH_SIMT)
+
+
 def test_bwd_data_rectangular_filter():
     d = layer(inputs.small_layer("k3x1", 2, 9, 8, 64, 64, 3, 1, 1, kw=1, seed=(602, 0)))
     got, path, _ = gpu_bwd_data(d)

@@ -586,6 +586,43 @@ def test_simt_small_layers(case):
     check(spec, expect_path=quan.QUAN_PATH_SIMT)
 
 
+NARROW_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad, extra: bf16 layers off the tcgen05 channel
+    # grid on warp-level MMAs: K tails, channel tiles past 64, one pixel buffer, few pixels
+    ("nw_one", 1, 1, 1, 4, 4, 1, 1, 0, {}),
+    ("nw_k_tail", 3, 13, 11, 12, 20, 3, 1, 1, {"bias": True, "act": quan.QUAN_ACT_SILU}),
+    ("nw_res", 16, 45, 37, 24, 40, 3, 1, 1, {"residual": True}),
+    ("nw_two_tiles", 2, 9, 10, 20, 132, 3, 2, 1, {"iqbn": False}),
+    ("nw_one_buffer", 1, 10, 9, 100, 24, 3, 1, 1, {}),   # K = 900
+    ("nw_wide_k", 1, 6, 7, 60, 36, 7, 1, 3, {}),         # K = 2940: CUDA cores
+    ("nw_wrap", 40, 33, 35, 8, 28, 1, 1, 0, {}),         # several tiles per block
+]
+
+
+@pytest.mark.parametrize("case", NARROW_CASES, ids=[c[0] for c in NARROW_CASES])
+def test_narrow_layers(case):
+    name, N, H, W, Cin, Cout, k, s, p, extra = case
+    check(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(304, len(name)), **extra))
+
+
+F32_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad: every thread tile of the CUDA-core kernel,
+    # row and column tails
+    ("f32_one", 1, 1, 1, 4, 4, 1, 1, 0),
+    ("f32_q17", 2, 6, 5, 12, 68, 3, 1, 1),
+    ("f32_2x2", 8, 32, 32, 64, 64, 3, 1, 1),
+    ("f32_2x4", 16, 40, 40, 36, 20, 3, 1, 1),
+    ("f32_s3_pad2", 3, 13, 10, 20, 28, 5, 3, 2),
+]
+
+
+@pytest.mark.parametrize("case", F32_CASES, ids=[c[0] for c in F32_CASES])
+def test_f32_layers(case):
+    name, N, H, W, Cin, Cout, k, s, p = case
+    check(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, dtype="f32", bias=True,
+                             act=quan.QUAN_ACT_SILU, seed=(303, len(name))))
+
+
 def test_simt_fp32_shapes():
     spec = inputs.small_layer("f32", 2, 9, 7, 8, 12, 3, 2, 1, dtype="f32", bias=True,
                               act=quan.QUAN_ACT_RELU, seed=(301, 0))
