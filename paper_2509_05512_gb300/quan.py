@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import os
 import re
+import struct
 import threading
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
@@ -106,6 +107,10 @@ def load():
         lib.quan_last_error_message.argtypes = []
         lib.quan_last_error_message.restype = ctypes.c_char_p
         lib.quan_version.argtypes = []
+        lib.quan_packed_call.argtypes = [_i, ctypes.c_char_p]
+        lib.quan_packed_call.restype = _i
+        lib.quan_packed_bwd_workspace.argtypes = [ctypes.c_char_p]
+        lib.quan_packed_bwd_workspace.restype = ctypes.c_size_t
         for name in ("quan_qconv2d_fwd", "quan_qconv2d_fwd_f32", "quan_qconv2d_fwd_res",
                      "quan_qconv2d_fwd_ex", "quan_qconv2d_fwd_shortcut",
                      "quan_qconv2d_sep_fwd", "quan_poincare_fwd", "quan_qconv2d_bwd_data",
@@ -132,13 +137,52 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _addr(t):
+    """_ptr as an integer (None: 0)."""
+    if t is None:
+        return 0
+    if isinstance(t, int):
+        return t
+    return t.data_ptr()
+
+
+_raw_stream = None
+
+
 def _stream(stream):
+    global _raw_stream
     if stream is None:
+        # the handle of torch.cuda.current_stream() without building the Stream object
+        # (0.4 us against 3)
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _raw_stream is None:
+            _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+                lambda device: torch.cuda.current_stream(device).cuda_stream)
+        return _raw_stream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+# Packed calls (csrc/packed.cu): entry point number and the layout of its arguments, every
+# integer and pointer a 64-bit word, in the order of the C function's.
+_CONV = struct.Struct("20q").pack           # x, 4 letters, 3 vectors, 10 sizes, out, stream
+_CONV_RES = struct.Struct("21q").pack
+_CONV_EX = struct.Struct("23q").pack
+_CONV_WS = struct.Struct("22q").pack
+_CONV_RGB = struct.Struct("19q").pack
+_BWD_DATA = struct.Struct("18q").pack
+_BWD_WEIGHT = struct.Struct("16q").pack
+_STATS = struct.Struct("8q").pack
+_TRAIN = struct.Struct("7qd3q").pack
+_SIZES = struct.Struct("9q").pack
+
+
+def _call(op: int, words: bytes) -> None:
+    lib = _lib if _lib is not None else load()
+    st = lib.quan_packed_call(op, words)
+    if st != QUAN_OK:
+        _check(st)
 
 
 def _check(st: int):
@@ -149,35 +193,32 @@ def _check(st: int):
 
 def quan_qconv2d_fwd(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin, Cout, kh, kw,
                      stride, pad, act, out, stream=None) -> None:
-    _check(load().quan_qconv2d_fwd(_ptr(x), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk), _ptr(bias),
-                                   _ptr(iqbn_scale), _ptr(iqbn_shift), N, H, W, Cin, Cout, kh, kw,
-                                   stride, pad, act, _ptr(out), _stream(stream)))
+    _call(0, _CONV(_addr(x), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                   _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cin, Cout, kh, kw, stride, pad,
+                   act, _addr(out), _stream(stream)))
 
 
 def quan_qconv2d_fwd_f32(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin, Cout, kh,
                          kw, stride, pad, act, out, stream=None) -> None:
-    _check(load().quan_qconv2d_fwd_f32(_ptr(x), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk),
-                                       _ptr(bias), _ptr(iqbn_scale), _ptr(iqbn_shift), N, H, W,
-                                       Cin, Cout, kh, kw, stride, pad, act, _ptr(out),
-                                       _stream(stream)))
+    _call(1, _CONV(_addr(x), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                   _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cin, Cout, kh, kw, stride, pad,
+                   act, _addr(out), _stream(stream)))
 
 
 def quan_qconv2d_fwd_res(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin, Cout, kh,
                          kw, stride, pad, act, residual, out, stream=None) -> None:
-    _check(load().quan_qconv2d_fwd_res(_ptr(x), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk),
-                                       _ptr(bias), _ptr(iqbn_scale), _ptr(iqbn_shift), N, H, W,
-                                       Cin, Cout, kh, kw, stride, pad, act, _ptr(residual),
-                                       _ptr(out), _stream(stream)))
+    _call(2, _CONV_RES(_addr(x), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                   _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cin, Cout, kh, kw, stride, pad,
+                   act, _addr(residual), _addr(out), _stream(stream)))
 
 
 def quan_qconv2d_fwd_ex(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin, Cout, kh,
                         kw, stride, pad, act, residual, workspace, workspace_bytes, out,
                         stream=None) -> None:
-    _check(load().quan_qconv2d_fwd_ex(_ptr(x), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk),
-                                      _ptr(bias), _ptr(iqbn_scale), _ptr(iqbn_shift), N, H, W,
-                                      Cin, Cout, kh, kw, stride, pad, act, _ptr(residual),
-                                      _ptr(workspace), workspace_bytes, _ptr(out),
-                                      _stream(stream)))
+    _call(3, _CONV_EX(_addr(x), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                   _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cin, Cout, kh, kw, stride, pad,
+                   act, _addr(residual), _addr(workspace), workspace_bytes,
+                   _addr(out), _stream(stream)))
 
 
 def quan_qconv2d_fwd_shortcut(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin,
@@ -283,10 +324,9 @@ def quan_version() -> int:
 
 def quan_qconv2d_sep_fwd(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin, Cout, kh,
                          kw, stride, pad, act, out, stream=None) -> None:
-    _check(load().quan_qconv2d_sep_fwd(_ptr(x), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk),
-                                       _ptr(bias), _ptr(iqbn_scale), _ptr(iqbn_shift), N, H, W,
-                                       Cin, Cout, kh, kw, stride, pad, act, _ptr(out),
-                                       _stream(stream)))
+    _call(4, _CONV(_addr(x), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                   _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cin, Cout, kh, kw, stride, pad,
+                   act, _addr(out), _stream(stream)))
 
 
 # ------------------------------------------------------------------ tensor helpers
@@ -353,15 +393,14 @@ def quan_qconv2d_bwd_data_workspace_size(Cin, Cout, kh, kw) -> int:
 
 
 def quan_qconv2d_bwd_data_workspace_size_ex(N, H, W, Cin, Cout, kh, kw, stride, pad) -> int:
-    return load().quan_qconv2d_bwd_data_workspace_size_ex(N, H, W, Cin, Cout, kh, kw, stride,
-                                                          pad)
+    return load().quan_packed_bwd_workspace(_SIZES(N, H, W, Cin, Cout, kh, kw, stride, pad))
 
 
 def quan_qconv2d_bwd_data(dy, wr, wi, wj, wk, N, H, W, Cin, Cout, kh, kw, stride, pad, workspace,
                           workspace_bytes, dx, stream=None) -> None:
-    _check(load().quan_qconv2d_bwd_data(_ptr(dy), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk), N, H,
-                                        W, Cin, Cout, kh, kw, stride, pad, _ptr(workspace),
-                                        workspace_bytes, _ptr(dx), _stream(stream)))
+    _call(5, _BWD_DATA(_addr(dy), _addr(wr), _addr(wi), _addr(wj), _addr(wk), N, H, W, Cin, Cout, kh,
+                       kw, stride, pad, _addr(workspace), workspace_bytes, _addr(dx),
+                       _stream(stream)))
 
 
 def quan_qconv2d_bwd_data_static(dy, wr, wi, wj, wk, N, H, W, Cin, Cout, kh, kw, stride, pad,
@@ -373,24 +412,21 @@ def quan_qconv2d_bwd_data_static(dy, wr, wi, wj, wk, N, H, W, Cin, Cout, kh, kw,
 
 def quan_qconv2d_sep_bwd_data(dy, wr, wi, wj, wk, N, H, W, Cin, Cout, kh, kw, stride, pad,
                               workspace, workspace_bytes, dx, stream=None) -> None:
-    _check(load().quan_qconv2d_sep_bwd_data(_ptr(dy), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk), N,
-                                            H, W, Cin, Cout, kh, kw, stride, pad,
-                                            _ptr(workspace), workspace_bytes, _ptr(dx),
-                                            _stream(stream)))
+    _call(6, _BWD_DATA(_addr(dy), _addr(wr), _addr(wi), _addr(wj), _addr(wk), N, H, W, Cin, Cout, kh,
+                       kw, stride, pad, _addr(workspace), workspace_bytes, _addr(dx),
+                       _stream(stream)))
 
 
 def quan_qconv2d_bwd_weight(x, dy, N, H, W, Cin, Cout, kh, kw, stride, pad, dwr, dwi, dwj, dwk,
                             stream=None) -> None:
-    _check(load().quan_qconv2d_bwd_weight(_ptr(x), _ptr(dy), N, H, W, Cin, Cout, kh, kw, stride,
-                                          pad, _ptr(dwr), _ptr(dwi), _ptr(dwj), _ptr(dwk),
-                                          _stream(stream)))
+    _call(7, _BWD_WEIGHT(_addr(x), _addr(dy), N, H, W, Cin, Cout, kh, kw, stride, pad, _addr(dwr),
+                         _addr(dwi), _addr(dwj), _addr(dwk), _stream(stream)))
 
 
 def quan_qconv2d_sep_bwd_weight(x, dy, N, H, W, Cin, Cout, kh, kw, stride, pad, dwr, dwi, dwj,
                                 dwk, stream=None) -> None:
-    _check(load().quan_qconv2d_sep_bwd_weight(_ptr(x), _ptr(dy), N, H, W, Cin, Cout, kh, kw,
-                                              stride, pad, _ptr(dwr), _ptr(dwi), _ptr(dwj),
-                                              _ptr(dwk), _stream(stream)))
+    _call(8, _BWD_WEIGHT(_addr(x), _addr(dy), N, H, W, Cin, Cout, kh, kw, stride, pad, _addr(dwr),
+                         _addr(dwi), _addr(dwj), _addr(dwk), _stream(stream)))
 
 
 def qconv2d_backward_data(dy, wr, wi, wj, wk, *, H, W, stride=1, pad=0, separable=False,
@@ -435,20 +471,18 @@ def quan_qconv2d_maxpool_workspace_size(N, H, W, Cout, kh, kw, stride, pad) -> i
 
 def quan_qconv2d_maxpool_rgb_fwd(rgb, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W,
                                  Cout, kh, kw, stride, pad, act, out, stream=None) -> None:
-    _check(load().quan_qconv2d_maxpool_rgb_fwd(_ptr(rgb), _ptr(wr), _ptr(wi), _ptr(wj),
-                                               _ptr(wk), _ptr(bias), _ptr(iqbn_scale),
-                                               _ptr(iqbn_shift), N, H, W, Cout, kh, kw, stride,
-                                               pad, act, _ptr(out), _stream(stream)))
+    _call(11, _CONV_RGB(_addr(rgb), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                        _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cout, kh, kw, stride,
+                        pad, act, _addr(out), _stream(stream)))
 
 
 def quan_qconv2d_maxpool_fwd(x, wr, wi, wj, wk, bias, iqbn_scale, iqbn_shift, N, H, W, Cin,
                              Cout, kh, kw, stride, pad, act, workspace, workspace_bytes, out,
                              stream=None) -> None:
-    _check(load().quan_qconv2d_maxpool_fwd(_ptr(x), _ptr(wr), _ptr(wi), _ptr(wj), _ptr(wk),
-                                           _ptr(bias), _ptr(iqbn_scale), _ptr(iqbn_shift), N,
-                                           H, W, Cin, Cout, kh, kw, stride, pad, act,
-                                           _ptr(workspace), workspace_bytes, _ptr(out),
-                                           _stream(stream)))
+    _call(12, _CONV_WS(_addr(x), _addr(wr), _addr(wi), _addr(wj), _addr(wk), _addr(bias),
+                   _addr(iqbn_scale), _addr(iqbn_shift), N, H, W, Cin, Cout, kh, kw, stride, pad,
+                   act, _addr(workspace), workspace_bytes, _addr(out),
+                   _stream(stream)))
 
 
 def quan_iqbn_batch_stats_workspace_size(C) -> int:
@@ -457,13 +491,13 @@ def quan_iqbn_batch_stats_workspace_size(C) -> int:
 
 def quan_iqbn_batch_stats(x, npix, C, workspace, workspace_bytes, mean, var,
                           stream=None) -> None:
-    _check(load().quan_iqbn_batch_stats(_ptr(x), npix, C, _ptr(workspace), workspace_bytes,
-                                        _ptr(mean), _ptr(var), _stream(stream)))
+    _call(9, _STATS(_addr(x), npix, C, _addr(workspace), workspace_bytes, _addr(mean),
+                    _addr(var), _stream(stream)))
 
 
 def quan_iqbn_train_fwd(x, npix, C, mean, var, gamma, beta, eps, act, out, stream=None) -> None:
-    _check(load().quan_iqbn_train_fwd(_ptr(x), npix, C, _ptr(mean), _ptr(var), _ptr(gamma),
-                                      _ptr(beta), eps, act, _ptr(out), _stream(stream)))
+    _call(10, _TRAIN(_addr(x), npix, C, _addr(mean), _addr(var), _addr(gamma), _addr(beta), eps,
+                     act, _addr(out), _stream(stream)))
 
 
 def iqbn_batch_stats(x, *, workspace=None, stream=None):
