@@ -3,8 +3,8 @@
 // quaternion channel) over N, H, W, and the normalisation with them.
 //
 // x is bf16 [npix][C] (NHWC flattened).  Both kernels are HBM-bound streams; every thread
-// keeps one fixed group of channels (8 channels read as one 16-byte vector, or a single
-// channel when C is not a multiple of 8) and walks the pixels with a grid-wide stride, so
+// keeps one fixed group of channels (8 or 4 channels read as one 16- or 8-byte vector, or a
+// single channel when C is not a multiple of 4) and walks the pixels with a grid-wide stride, so
 // its per-channel state stays in registers.
 //
 // Statistics: each thread sums d = x - K_c and d^2 in fp32 over its pixels, with the shift
@@ -21,20 +21,57 @@
 namespace quan {
 namespace {
 
-__device__ __forceinline__ void unpack8(const uint4 v, float (&f)[8]) {
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
+// W channels of one pixel in one access: 16, 8 or 2 bytes.
+template <int W>
+struct Vec;
+template <>
+struct Vec<8> {
+    using T = uint4;
+};
+template <>
+struct Vec<4> {
+    using T = uint2;
+};
+template <>
+struct Vec<1> {
+    using T = unsigned short;
+};
+
+template <int W>
+__device__ __forceinline__ void unpack(const typename Vec<W>::T& v, float (&f)[W]) {
+    if constexpr (W == 1) {
+        f[0] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(&v));
+    } else {
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 t = __bfloat1622float2(h[i]);
-        f[2 * i] = t.x;
-        f[2 * i + 1] = t.y;
+        for (int i = 0; i < W / 2; ++i) {
+            const float2 t = __bfloat1622float2(h[i]);
+            f[2 * i] = t.x;
+            f[2 * i + 1] = t.y;
+        }
     }
 }
 
-// W channels per thread (8: one 16-byte vector, 1: scalar); G = C / W channel groups;
-// blockDim.x = G * R, R pixel rows per block.
 template <int W>
-__global__ void __launch_bounds__(256) iqbn_stats_kernel(const __nv_bfloat16* __restrict__ x,
+__device__ __forceinline__ typename Vec<W>::T pack(const float (&f)[W]) {
+    typename Vec<W>::T v;
+    if constexpr (W == 1) {
+        const __nv_bfloat16 t = __float2bfloat16_rn(f[0]);
+        v = *reinterpret_cast<const unsigned short*>(&t);
+    } else {
+        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&v);
+#pragma unroll
+        for (int i = 0; i < W / 2; ++i) h[i] = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+    }
+    return v;
+}
+
+// W channels per thread (one 16- or 8-byte vector, or a scalar); G = C / W channel groups;
+// blockDim.x = G * R, R pixel rows per block.
+// Four blocks per SM, the grid's share: at 72 registers only three fit, and the rest ran as a
+// second wave of a quarter of the work.
+template <int W>
+__global__ void __launch_bounds__(256, 4) iqbn_stats_kernel(const __nv_bfloat16* __restrict__ x,
                                                          long long npix, int C, int G,
                                                          float* __restrict__ part) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -43,23 +80,15 @@ __global__ void __launch_bounds__(256) iqbn_stats_kernel(const __nv_bfloat16* __
     const int slot = threadIdx.x % G, row = threadIdx.x / G;
     const int R = blockDim.x / G;
     const int c0 = slot * W;
+    using V = typename Vec<W>::T;
     float K[W], a1[W], a2[W];
-    if constexpr (W == 8) {
-        unpack8(__ldg(reinterpret_cast<const uint4*>(x + c0)), K);
-    } else {
-        K[0] = __bfloat162float(x[c0]);
-    }
+    unpack<W>(__ldg(reinterpret_cast<const V*>(x + c0)), K);
 #pragma unroll
     for (int i = 0; i < W; ++i) a1[i] = a2[i] = 0.f;
     const long long stride = static_cast<long long>(gridDim.x) * R;
-    auto load = [&](long long p, float (&v)[W]) {
-        if constexpr (W == 8) {
-            unpack8(__ldg(reinterpret_cast<const uint4*>(x + p * C + c0)), v);
-        } else {
-            v[0] = __bfloat162float(x[p * C + c0]);
-        }
-    };
-    auto add = [&](const float (&v)[W]) {
+    auto add = [&](const V& raw) {
+        float v[W];
+        unpack<W>(raw, v);
 #pragma unroll
         for (int i = 0; i < W; ++i) {
             const float d = v[i] - K[i];
@@ -69,37 +98,15 @@ __global__ void __launch_bounds__(256) iqbn_stats_kernel(const __nv_bfloat16* __
     };
     long long p = static_cast<long long>(blockIdx.x) * R + row;
     // eight independent loads in flight per thread, then the remainder one at a time
-    if constexpr (W == 8) {
-        for (; p + 7 * stride < npix; p += 8 * stride) {
-            uint4 raw[8];
+    for (; p + 7 * stride < npix; p += 8 * stride) {
+        V raw[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                raw[k] = __ldg(reinterpret_cast<const uint4*>(x + (p + k * stride) * C + c0));
+        for (int k = 0; k < 8; ++k)
+            raw[k] = __ldg(reinterpret_cast<const V*>(x + (p + k * stride) * C + c0));
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                float v[8];
-                unpack8(raw[k], v);
-                add(v);
-            }
-        }
-    } else {
-        for (; p + 3 * stride < npix; p += 4 * stride) {
-            float v0[W], v1[W], v2[W], v3[W];
-            load(p, v0);
-            load(p + stride, v1);
-            load(p + 2 * stride, v2);
-            load(p + 3 * stride, v3);
-            add(v0);
-            add(v1);
-            add(v2);
-            add(v3);
-        }
+        for (int k = 0; k < 8; ++k) add(raw[k]);
     }
-    for (; p < npix; p += stride) {
-        float v[W];
-        load(p, v);
-        add(v);
-    }
+    for (; p < npix; p += stride) add(__ldg(reinterpret_cast<const V*>(x + p * C + c0)));
     float* r1 = red;
     float* r2 = red + blockDim.x * W;
 #pragma unroll
@@ -133,11 +140,13 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
     sum = t;
 }
 
-// Sum of the partial rows per channel in a fixed order (row lane rl takes rows rl, rl + 32,
-// ..., compensated fp32; then the 32 lanes in order), then mean = K + S1 / n and
+// Sum of the partial rows per channel in a fixed order (row lane rl takes rows rl, rl + 128,
+// ..., compensated fp32; then the 128 lanes as a tree in fp64), then mean = K + S1 / n and
 // var = max(S2 / n - (S1 / n)^2, 0) (these last few operations per channel in fp64; the
 // row sums stay in fp32, the double-precision rate of this part being low).
-// Block: 32 channels x 32 row lanes.
+// Block: 8 channels x 128 row lanes, so a lane's chain is a few loads long (32 channels x 32
+// lanes, 19 rows each and 32 lanes added one by one, took 8.4 us for 256 channels).
+constexpr int FIN_C = 8;
 __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16* __restrict__ x,
                                                              long long npix, int C, int rows,
                                                              const float* __restrict__ part,
@@ -145,31 +154,46 @@ __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16
                                                              float* __restrict__ var) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    __shared__ float red[2][32][33];
-    const int cl = threadIdx.x % 32, rl = threadIdx.x / 32;
-    const int c = blockIdx.x * 32 + cl;
+    __shared__ double red[2][FIN_C][32];
+    const int cl = threadIdx.x % FIN_C, rl = threadIdx.x / FIN_C;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int c = blockIdx.x * FIN_C + cl;
     float t1 = 0.f, t2 = 0.f, e1 = 0.f, e2 = 0.f;
     if (c < C) {
 #pragma unroll 4
-        for (int r = rl; r < rows; r += 32) {
+        for (int r = rl; r < rows; r += 1024 / FIN_C) {
             kahan_add(t1, e1, part[static_cast<size_t>(r) * 2 * C + c]);
             kahan_add(t2, e2, part[static_cast<size_t>(r) * 2 * C + C + c]);
         }
     }
-    red[0][rl][cl] = t1 - e1;
-    red[1][rl][cl] = t2 - e2;
+    double d1 = static_cast<double>(t1) - e1, d2 = static_cast<double>(t2) - e2;
+    // the warp's four row lanes of each channel (lanes cl, cl + 8, ..)
+#pragma unroll
+    for (int k = FIN_C; k < 32; k *= 2) {
+        d1 += __shfl_xor_sync(0xffffffffu, d1, k);
+        d2 += __shfl_xor_sync(0xffffffffu, d2, k);
+    }
+    if (lane < FIN_C) {
+        red[0][cl][warp] = d1;
+        red[1][cl][warp] = d2;
+    }
     __syncthreads();
-    if (rl == 0 && c < C) {
-        float s1 = 0.f, s2 = 0.f, f1 = 0.f, f2 = 0.f;
-        for (int k = 0; k < 32; ++k) {
-            kahan_add(s1, f1, red[0][k][cl]);
-            kahan_add(s2, f2, red[1][k][cl]);
+    if (warp < FIN_C) {  // warp w finishes channel w
+        d1 = red[0][warp][lane];
+        d2 = red[1][warp][lane];
+#pragma unroll
+        for (int k = 1; k < 32; k *= 2) {
+            d1 += __shfl_xor_sync(0xffffffffu, d1, k);
+            d2 += __shfl_xor_sync(0xffffffffu, d2, k);
         }
-        const double inv_n = 1.0 / static_cast<double>(npix);
-        const double d1 = (static_cast<double>(s1) - f1) * inv_n;
-        const double m2 = (static_cast<double>(s2) - f2) * inv_n - d1 * d1;
-        mean[c] = static_cast<float>(static_cast<double>(__bfloat162float(x[c])) + d1);
-        var[c] = m2 > 0.0 ? static_cast<float>(m2) : 0.0f;
+        const int cw = blockIdx.x * FIN_C + warp;
+        if (lane == 0 && cw < C) {
+            const double inv_n = 1.0 / static_cast<double>(npix);
+            const double m1 = d1 * inv_n;
+            const double m2 = d2 * inv_n - m1 * m1;
+            mean[cw] = static_cast<float>(static_cast<double>(__bfloat162float(x[cw])) + m1);
+            var[cw] = m2 > 0.0 ? static_cast<float>(m2) : 0.0f;
+        }
     }
 }
 
@@ -179,7 +203,28 @@ __device__ __forceinline__ float act_fn(float z, int act) {
     return z;
 }
 
+// Read for the last time: the line is the first to leave L2.
+__device__ __forceinline__ uint4 ld_last(const uint4* p, uint64_t policy) {
+    uint4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p), "l"(policy)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_last(const uint2* p, uint64_t policy) {
+    uint2 v;
+    asm volatile("ld.global.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;"
+                 : "=r"(v.x), "=r"(v.y)
+                 : "l"(p), "l"(policy)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned short ld_last(const unsigned short* p, uint64_t) { return *p; }
+
 // out = act(gamma (x - mean) / sqrt(var + eps) + beta) (Eq. 11-12), as scale * x + shift.
+// The pixels are walked from the last to the first: the statistics, which usually ran just
+// before, read x from first to last, so its end is what L2 still holds.
 template <int W>
 __global__ void __launch_bounds__(256) iqbn_apply_kernel(
     const __nv_bfloat16* x, long long npix, int C, int G, const float* __restrict__ mean,
@@ -200,58 +245,36 @@ __global__ void __launch_bounds__(256) iqbn_apply_kernel(
         sh[i] = fmaf(-mean[c], sc[i], b);
     }
     const long long stride = static_cast<long long>(gridDim.x) * R;
-    auto one = [&](long long p) {
-        if constexpr (W == 8) {
-            float v[8];
-            unpack8(*reinterpret_cast<const uint4*>(x + p * C + c0), v);
-            uint4 o;
-            uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    const long long end = npix - 1;  // pixel end - p in place of p
+    using V = typename Vec<W>::T;
+    auto load = [&](long long q) {
+        return ld_last(reinterpret_cast<const V*>(x + (end - q) * C + c0), policy);
+    };
+    auto finish = [&](long long q, const V& raw) {
+        float v[W];
+        unpack<W>(raw, v);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const __nv_bfloat162 t =
-                    __floats2bfloat162_rn(act_fn(fmaf(v[2 * i], sc[2 * i], sh[2 * i]), act),
-                                          act_fn(fmaf(v[2 * i + 1], sc[2 * i + 1], sh[2 * i + 1]), act));
-                ow[i] = *reinterpret_cast<const uint32_t*>(&t);
-            }
-            *reinterpret_cast<uint4*>(out + p * C + c0) = o;
-        } else {
-            const float v = __bfloat162float(x[p * C + c0]);
-            out[p * C + c0] = __float2bfloat16_rn(act_fn(fmaf(v, sc[0], sh[0]), act));
-        }
+        for (int i = 0; i < W; ++i) v[i] = act_fn(fmaf(v[i], sc[i], sh[i]), act);
+        *reinterpret_cast<V*>(out + (end - q) * C + c0) = pack<W>(v);
     };
     long long p = static_cast<long long>(blockIdx.x) * R + row;
-    if constexpr (W == 8) {
-        // four loads in flight before the first store (each thread reads only the
-        // elements it writes, so an in-place call is still safe)
-        for (; p + 3 * stride < npix; p += 4 * stride) {
-            uint4 raw[4];
+    // four loads in flight before the first store (each thread reads only the elements it
+    // writes, so an in-place call is still safe)
+    for (; p + 3 * stride < npix; p += 4 * stride) {
+        V raw[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                raw[k] = *reinterpret_cast<const uint4*>(x + (p + k * stride) * C + c0);
+        for (int k = 0; k < 4; ++k) raw[k] = load(p + k * stride);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                float v[8];
-                unpack8(raw[k], v);
-                uint4 o;
-                uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const __nv_bfloat162 t = __floats2bfloat162_rn(
-                        act_fn(fmaf(v[2 * i], sc[2 * i], sh[2 * i]), act),
-                        act_fn(fmaf(v[2 * i + 1], sc[2 * i + 1], sh[2 * i + 1]), act));
-                    ow[i] = *reinterpret_cast<const uint32_t*>(&t);
-                }
-                *reinterpret_cast<uint4*>(out + (p + k * stride) * C + c0) = o;
-            }
-        }
+        for (int k = 0; k < 4; ++k) finish(p + k * stride, raw[k]);
     }
-    for (; p < npix; p += stride) one(p);
+    for (; p < npix; p += stride) finish(p, load(p));
 }
 
 // Channel groups, block size and grid of one launch; false if C has no layout.
-bool iqbn_layout(int C, bool vec, long long npix, int num_sms, int per_sm, int* G, int* block,
+bool iqbn_layout(int C, int W, long long npix, int num_sms, int per_sm, int* G, int* block,
                  int* grid) {
-    const int W = vec ? 8 : 1;
     const int g = C / W;
     if (g < 1 || g > 256) return false;
     const int R = 256 / g;
@@ -262,6 +285,15 @@ bool iqbn_layout(int C, bool vec, long long npix, int num_sms, int per_sm, int* 
     if (blocks > cap) blocks = cap;
     *grid = static_cast<int>(blocks);
     return true;
+}
+
+// Channels per access: 8 (16 bytes), 4 (8 bytes: the quaternion channel counts that are no
+// multiple of 8; a scalar access each instead took 135 us, now 50 us, for the statistics and
+// the normalisation of 40 M elements in 44 channels), or 1.
+int iqbn_width(int C, const void* a, const void* b) {
+    if (iqbn_vec_ok(C, a, b)) return 8;
+    const uintptr_t bits = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
+    return C % 4 == 0 && bits % 8 == 0 ? 4 : 1;
 }
 
 }  // namespace
@@ -281,34 +313,31 @@ size_t iqbn_stats_workspace_bytes(int C) {
 
 cudaError_t launch_iqbn_stats(const void* x, long long npix, int C, void* workspace,
                               float* mean, float* var, int num_sms, cudaStream_t stream) {
-    const bool vec = iqbn_vec_ok(C, x, x);
+    const int W = iqbn_width(C, x, x);
     int G = 0, block = 0, grid = 0;
-    if (!iqbn_layout(C, vec, npix, num_sms, 4, &G, &block, &grid)) return cudaErrorInvalidValue;
+    if (!iqbn_layout(C, W, npix, num_sms, 4, &G, &block, &grid)) return cudaErrorInvalidValue;
     if (grid > IQBN_MAX_PARTIALS) grid = IQBN_MAX_PARTIALS;
     const auto* xb = static_cast<const __nv_bfloat16*>(x);
     auto* part = static_cast<float*>(workspace);
-    const size_t smem = static_cast<size_t>(2) * block * (vec ? 8 : 1) * sizeof(float);
-    cudaError_t e = vec ? launch_pdl(iqbn_stats_kernel<8>, dim3(grid), dim3(block), smem, stream,
-                                     xb, npix, C, G, part)
-                        : launch_pdl(iqbn_stats_kernel<1>, dim3(grid), dim3(block), smem, stream,
-                                     xb, npix, C, G, part);
+    const size_t smem = static_cast<size_t>(2) * block * W * sizeof(float);
+    auto kern = W == 8 ? iqbn_stats_kernel<8> : W == 4 ? iqbn_stats_kernel<4> : iqbn_stats_kernel<1>;
+    cudaError_t e = launch_pdl(kern, dim3(grid), dim3(block), smem, stream, xb, npix, C, G, part);
     if (e != cudaSuccess) return e;
-    return launch_pdl(iqbn_finalize_kernel, dim3((C + 31) / 32), dim3(1024), 0, stream, xb,
+    return launch_pdl(iqbn_finalize_kernel, dim3((C + FIN_C - 1) / FIN_C), dim3(1024), 0, stream, xb,
                       npix, C, grid, static_cast<const float*>(part), mean, var);
 }
 
 cudaError_t launch_iqbn_apply(const void* x, long long npix, int C, const float* mean,
                               const float* var, const float* gamma, const float* beta, float eps,
                               int act, void* out, int num_sms, cudaStream_t stream) {
-    const bool vec = iqbn_vec_ok(C, x, out);
+    const int W = iqbn_width(C, x, out);
     int G = 0, block = 0, grid = 0;
-    if (!iqbn_layout(C, vec, npix, num_sms, 8, &G, &block, &grid)) return cudaErrorInvalidValue;
+    if (!iqbn_layout(C, W, npix, num_sms, 8, &G, &block, &grid)) return cudaErrorInvalidValue;
     const auto* xb = static_cast<const __nv_bfloat16*>(x);
     auto* ob = static_cast<__nv_bfloat16*>(out);
-    return vec ? launch_pdl(iqbn_apply_kernel<8>, dim3(grid), dim3(block), 0, stream, xb, npix,
-                            C, G, mean, var, gamma, beta, eps, act, ob)
-               : launch_pdl(iqbn_apply_kernel<1>, dim3(grid), dim3(block), 0, stream, xb, npix,
-                            C, G, mean, var, gamma, beta, eps, act, ob);
+    auto kern = W == 8 ? iqbn_apply_kernel<8> : W == 4 ? iqbn_apply_kernel<4> : iqbn_apply_kernel<1>;
+    return launch_pdl(kern, dim3(grid), dim3(block), 0, stream, xb, npix, C, G, mean, var, gamma,
+                      beta, eps, act, ob);
 }
 
 }  // namespace quan

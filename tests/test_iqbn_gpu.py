@@ -69,6 +69,22 @@ def test_batch_stats(case):
     check_stats(_dev(bits, off), x64)
 
 
+@pytest.mark.parametrize("shape,off", [
+    ((3, 5, 7, 44), 4),       # 8-byte accesses, x 8- but not 16-byte aligned, odd pixel count
+    ((1, 1, 1, 4), 0),        # one pixel, one channel group
+    ((2, 60, 61, 252), 0),    # 63 groups, several pixels per thread
+    ((2, 9, 11, 2040), 0),    # 255 finishing blocks, the last group of 16-byte accesses
+], ids=["c44", "c4", "c252", "c2040"])
+def test_access_widths(shape, off):
+    rng = np.random.default_rng(840 + shape[-1])
+    C = shape[-1]
+    bits, x64 = _bf16(rng, shape, scale=np.linspace(0.5, 2.0, C), offset=1.0)
+    check_stats(_dev(bits, off), x64)
+    gamma, beta = rng.uniform(0.5, 1.5, C), rng.standard_normal(C) * 0.1
+    if x64.size > C:
+        check_train(_dev(bits, off), x64, gamma, beta, 1e-5, quan.QUAN_ACT_RELU)
+
+
 def test_batch_stats_repeat_bit_identical():
     # partial sums are added in a fixed order: the same input gives the same bits
     rng = np.random.default_rng(811)
