@@ -290,12 +290,13 @@ __device__ __forceinline__ void sp_convert_rgb(const StemPoolParams& p, uint32_t
             for (int c = 0; c < 2; ++c) {
                 const int jb = ct + 64 * c, pi = pair0 + jb;
                 live[a][c] = row_in && jb < gp && pi >= 0 && pi < W2;
-                if (live[a][c]) {
-                    const uint32_t src = slot_sa + r * rgb_rb + 24 * pi;
-                    in[a][c][0] = lds_f2(src);
-                    in[a][c][1] = lds_f2(src + 8);
-                    in[a][c][2] = lds_f2(src + 16);
-                }
+                // a pair outside the image reads the slot's first pixels and is zeroed below:
+                // no branch between the pairs, so that their chains overlap (with one the
+                // two warps took 4100 clocks for a tile's 4 x 120 pairs)
+                const uint32_t src = slot_sa + (live[a][c] ? r * rgb_rb + 24 * pi : 0u);
+                in[a][c][0] = lds_f2(src);
+                in[a][c][1] = lds_f2(src + 8);
+                in[a][c][2] = lds_f2(src + 16);
             }
         }
 #pragma unroll
@@ -303,10 +304,9 @@ __device__ __forceinline__ void sp_convert_rgb(const StemPoolParams& p, uint32_t
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int r = r0 + a, jb = ct + 64 * c;
-                if (r >= p.rows || jb >= gp) continue;
-                sts_u4(stage_sa + r * rb + 16 * jb,
-                       live[a][c] ? sp_poincare_pair(in[a][c][0], in[a][c][1], in[a][c][2])
-                                  : make_uint4(0u, 0u, 0u, 0u));
+                uint4 v = sp_poincare_pair(in[a][c][0], in[a][c][1], in[a][c][2]);
+                if (!live[a][c]) v = make_uint4(0u, 0u, 0u, 0u);
+                if (r < p.rows && jb < gp) sts_u4(stage_sa + r * rb + 16 * jb, v);
             }
     }
 }
