@@ -37,9 +37,10 @@
 //
 // RGB input (RGB = true): the Poincare mapping of Eq. 4 (Sec. III-A) is fused into the
 // loader.  Warp 0's lane 0 loads the tile's kh + 2 rows of fp32 RGB pixels (one TMA box of
-// whole rows) into a ring of SP_RGB_SLOTS staging slots, SP_RGB_SLOTS - 1 tiles ahead;
-// warps 0 and 3 turn the rows a tile does not share with the previous one into the bf16
-// quaternion pairs of the B stage (the MMAs read the shared rows from the previous stage), q = ((1 - n2), 2 r, 2 g, 2 b) / (1 + n2)
+// whole rows) into a ring of SP_RGB_SLOTS staging slots; the epilogue warps, which wait for
+// accumulators much of the time, turn the rows a tile does not share with the previous one
+// into the bf16 quaternion pairs of the B stage, SP_RGB_AHEAD tiles before they pool it (the
+// MMAs read the shared rows from the previous stage), q = ((1 - n2), 2 r, 2 g, 2 b) / (1 + n2)
 // with n2 = r^2 + g^2 + b^2 (the arithmetic of the stand-alone mapping kernel, so the
 // result is bit-identical to mapping first), zero pairs outside the image (the
 // convolution's zero padding of the quaternion input), and hand the stage to its issuer.
@@ -67,7 +68,11 @@ constexpr int SP_EXP_WARP0 = 2;          // warps 2..19 expand the block weight
 constexpr int SP_EXP_WARPS = 18;
 constexpr int SP_EPI_WARP0 = 4;          // warps 4..19: epilogue
 constexpr int SP_EPI_THREADS = 512;
-constexpr int SP_RGB_SLOTS = 3;          // RGB input: staging slots of kh + 2 RGB rows
+constexpr int SP_RGB_SLOTS = 2;          // RGB input: staging slots of kh + 2 RGB rows
+// RGB input: the epilogue warps map tile k + SP_RGB_AHEAD before they pool tile k.  Tile
+// k + 2's stage needs the MMAs of tile k + 1 at most (two stages), which need no epilogue later
+// than tile k - 3's, so the mapping never waits for itself.
+constexpr int SP_RGB_AHEAD = 2;
 
 struct StemPoolParams {
     ConvShape s;
@@ -263,51 +268,28 @@ __device__ __forceinline__ uint4 sp_poincare_pair(float2 a, float2 b, float2 c) 
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Warps 0 and 3 (RGB input): rows r_begin .. rows - 1 of one tile's B stage, mapped from
-// the tile's staging slot of RGB rows (rows 0 .. 3 of a tile that continues an image are
-// rows 4 .. 7 of the previous tile: the MMAs read them from that tile's stage and they are
-// not written again; r_begin is 4 then, else 0).  ct = 0 .. 63 this thread's index among the two warps, which takes the pairs ct
-// and ct + 64 of each row; y0 = the tile's first input row; 32-bit shared addresses.  Under
-// the MMAs' operand reads shared-memory accesses take hundreds of cycles, so all of a
-// thread's loads (at most 2 pairs x MAXR rows) are issued before any pair is mapped.
-template <int MAXR>
+// Epilogue warps (RGB input): rows r_begin .. rows - 1 of one tile's B stage, mapped from the
+// tile's staging slot of RGB rows (rows 0 .. 3 of a tile that continues an image are rows
+// 4 .. 7 of the previous tile: the MMAs read them from that tile's stage and they are not
+// written again; r_begin is 4 then, else 0).  et = 0 .. 511, one pair a pass; y0 = the tile's
+// first input row; 32-bit shared addresses.
 __device__ __forceinline__ void sp_convert_rgb(const StemPoolParams& p, uint32_t stage_sa,
-                                               int r_begin, uint32_t slot_sa, int y0, int ct) {
+                                               int r_begin, uint32_t slot_sa, int y0, int et) {
     const ConvShape& s = p.s;
     const int gp = p.row_bytes / 16;  // pairs per box row
+    const int lg = gp <= 128 ? 7 : 8;
     const int pair0 = p.gx0 * p.group;
     const int W2 = s.W / 2;
-    const uint32_t rb = static_cast<uint32_t>(p.row_bytes);
-    const uint32_t rgb_rb = static_cast<uint32_t>(p.rgb_row_bytes);
-    for (int r0 = r_begin; r0 < p.rows; r0 += MAXR) {
-        float2 in[MAXR][2][3];
-        bool live[MAXR][2];
-#pragma unroll
-        for (int a = 0; a < MAXR; ++a) {
-            const int r = r0 + a, y = y0 + r;
-            const bool row_in = r < p.rows && y >= 0 && y < s.H;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int jb = ct + 64 * c, pi = pair0 + jb;
-                live[a][c] = row_in && jb < gp && pi >= 0 && pi < W2;
-                // a pair outside the image reads the slot's first pixels and is zeroed below:
-                // no branch between the pairs, so that their chains overlap (with one the
-                // two warps took 4100 clocks for a tile's 4 x 120 pairs)
-                const uint32_t src = slot_sa + (live[a][c] ? r * rgb_rb + 24 * pi : 0u);
-                in[a][c][0] = lds_f2(src);
-                in[a][c][1] = lds_f2(src + 8);
-                in[a][c][2] = lds_f2(src + 16);
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < MAXR; ++a)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int r = r0 + a, jb = ct + 64 * c;
-                uint4 v = sp_poincare_pair(in[a][c][0], in[a][c][1], in[a][c][2]);
-                if (!live[a][c]) v = make_uint4(0u, 0u, 0u, 0u);
-                if (r < p.rows && jb < gp) sts_u4(stage_sa + r * rb + 16 * jb, v);
-            }
+    for (int e = et; e < (p.rows - r_begin) << lg; e += SP_EPI_THREADS) {
+        const int r = r_begin + (e >> lg), jb = e & ((1 << lg) - 1);
+        const int y = y0 + r, pi = pair0 + jb;
+        const bool live = y >= 0 && y < s.H && pi >= 0 && pi < W2;
+        const uint32_t src =
+            slot_sa + (live ? static_cast<uint32_t>(r * p.rgb_row_bytes + 24 * pi) : 0u);
+        const float2 a = lds_f2(src), b = lds_f2(src + 8), c = lds_f2(src + 16);
+        uint4 v = sp_poincare_pair(a, b, c);
+        if (!live) v = make_uint4(0u, 0u, 0u, 0u);
+        if (jb < gp) sts_u4(stage_sa + static_cast<uint32_t>(r * p.row_bytes + 16 * jb), v);
     }
 }
 
@@ -351,7 +333,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
     griddep_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < STAGES; ++i) {
-            mbar_init(full_bar(i), RGB ? 2 : 1);  // RGB: the two converter warps
+            mbar_init(full_bar(i), RGB ? SP_EPI_THREADS / 32 : 1);  // RGB: the mapping warps
             // RGB: a stage is also read by the next tile (the rows the two share)
             mbar_init(empty_bar(i), RGB ? 2 : 1);
         }
@@ -363,7 +345,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
         mbar_init(bready_bar, SP_EXP_WARPS);
         for (int i = 0; i < SP_RGB_SLOTS; ++i) {
             mbar_init(rgbf0 + 8u * i, 1);
-            mbar_init(rgbe0 + 8u * i, 2);
+            mbar_init(rgbe0 + 8u * i, SP_EPI_THREADS / 32);
         }
         *abort_flag = 0;
         fence_barrier_init();
@@ -381,80 +363,37 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
     // kernel's last CTAs; the input loaders and the epilogue wait for that kernel before
     // their first access to activations.
 
-    if (RGB && (warp == 0 || warp == 3)) {
-        // ------------------------------------------------- RGB staging and conversion
-        // (warp 3 first helps with the weight expansion)
-        if (warp == 3) sp_expand<RAW>(p, smem, (warp - SP_EXP_WARP0) * 32 + lane, lane, bready_bar);
-        griddep_wait();  // the previous kernel's output (this layer's input) is complete
-        const int ct = (warp == 0 ? 0 : 32) + lane;
-        const uint64_t pol_x = l2_policy_evict_first();
-        const uint32_t tx = static_cast<uint32_t>(p.rows * p.rgb_row_bytes);
-        uint32_t filled = 0, fill_parity = 0;
-        int img = static_cast<int>(rfirst / p.Hp);
-        int i = static_cast<int>(rfirst - static_cast<long long>(img) * p.Hp);
-        int nimg = img, ni = i;  // the next tile to load
-        auto load_next = [&](int k) -> bool {  // warp 0 lane 0: staging slot of tile k
-            const int sl = k % SP_RGB_SLOTS;
-            const uint32_t ph = static_cast<uint32_t>(k / SP_RGB_SLOTS) & 1u;
-            if (!wait_or_abort(rgbe0 + 8u * sl, ph ^ 1u, limit, abort_flag,
-                               STATUS_TIMEOUT_PRODUCER))
-                return false;
-            mbar_arrive_expect_tx(rgbf0 + 8u * sl, tx);
-            filled |= 1u << sl;
-            fill_parity = (fill_parity & ~(1u << sl)) | (ph << sl);
-            tma_load_4d(sbase + p.rgb_off + sl * p.rgb_stage_bytes, &tmap_x, rgbf0 + 8u * sl, 0,
-                        0, 4 * ni - s.pad, nimg, pol_x);
-            if (++ni == p.Hp) {
-                ni = 0;
-                ++nimg;
+    if (RGB && warp == 0) {
+        // ------------------------------------------------------------ RGB staging
+        if (lane == 0) {
+            griddep_wait();  // the previous kernel's output (this layer's input) is complete
+            const uint64_t pol_x = l2_policy_evict_first();
+            const uint32_t tx = static_cast<uint32_t>(p.rows * p.rgb_row_bytes);
+            uint32_t filled = 0, fill_parity = 0;
+            int img = static_cast<int>(rfirst / p.Hp);
+            int i = static_cast<int>(rfirst - static_cast<long long>(img) * p.Hp);
+            bool ok = true;
+            for (int k = 0; k < ntiles; ++k) {
+                const int sl = k % SP_RGB_SLOTS;
+                const uint32_t ph = static_cast<uint32_t>(k / SP_RGB_SLOTS) & 1u;
+                if (!wait_or_abort(rgbe0 + 8u * sl, ph ^ 1u, limit, abort_flag,
+                                   STATUS_TIMEOUT_PRODUCER)) {
+                    ok = false;
+                    break;
+                }
+                mbar_arrive_expect_tx(rgbf0 + 8u * sl, tx);
+                filled |= 1u << sl;
+                fill_parity = (fill_parity & ~(1u << sl)) | (ph << sl);
+                tma_load_4d(sbase + p.rgb_off + sl * p.rgb_stage_bytes, &tmap_x, rgbf0 + 8u * sl,
+                            0, 0, 4 * i - s.pad, img, pol_x);
+                if (++i == p.Hp) {
+                    i = 0;
+                    ++img;
+                }
             }
-            return true;
-        };
-        bool ok = true;
-        if (warp == 0 && lane == 0)
-            for (int k = 0; ok && k < SP_RGB_SLOTS - 1 && k < ntiles; ++k) ok = load_next(k);
-        StageCursor cur(p.per);
-        int ki = 0, prev_stage = -1;
-        for (int k = 0; k < ntiles; ++k) {
-            const int stage = cur.stage(ki);
-            const uint32_t phase = cur.phase;
-            if (++ki == SP_ISSUERS) {
-                ki = 0;
-                cur.next();
-            }
-            // rows shared with the previous tile (same image): copied, not mapped again
-            // (rows 4 .. rows - 1 of every stage are written, so the next tile's rows
-            // 0 .. rows - 6, rows 4 .. rows - 2 here, are always in this tile's stage)
-            const int r_begin = (prev_stage >= 0 && i != 0 && p.rows > 5) ? 4 : 0;
-            const int sl = k % SP_RGB_SLOTS;
-            if (warp == 0 && lane == 0 && ok && k + SP_RGB_SLOTS - 1 < ntiles)
-                ok = load_next(k + SP_RGB_SLOTS - 1);
-            if (lane == 0 && ok)
-                ok = wait_or_abort(rgbf0 + 8u * sl,
-                                   static_cast<uint32_t>(k / SP_RGB_SLOTS) & 1u, limit,
-                                   abort_flag, STATUS_TIMEOUT_PRODUCER) &&
-                     wait_or_abort(empty_bar(stage), phase ^ 1u, limit, abort_flag,
-                                   STATUS_TIMEOUT_PRODUCER);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            // both converter warps leave together; the barrier also orders the previous
-            // tile's stage writes (of both warps) before this tile's copies from it
-            if (named_bar_or(7, 64, !ok)) break;
-            sp_convert_rgb<4>(p, sbase + C::RING_OFF + stage * p.stage_bytes, r_begin,
-                              sbase + p.rgb_off + sl * p.rgb_stage_bytes, 4 * i - s.pad, ct);
-            prev_stage = stage;
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(full_bar(stage));
-                mbar_arrive(rgbe0 + 8u * sl);
-            }
-            if (++i == p.Hp) {
-                i = 0;
-                ++img;
-            }
+            if (!ok || *abort_flag)
+                drain_fills(rgbf0, SP_RGB_SLOTS, filled, fill_parity, limit);
         }
-        if (warp == 0 && lane == 0 && (!ok || *abort_flag))
-            drain_fills(rgbf0, SP_RGB_SLOTS, filled, fill_parity, limit);
     } else if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -614,7 +553,48 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
             for (int u = 0; u < 8; ++u) prev1[u] = -INFINITY;
             int img = static_cast<int>(rfirst / p.Hp);
             int i = static_cast<int>(rfirst - static_cast<long long>(img) * p.Hp);
+            // RGB: map tile k (called for k = 0, 1, .. in order): its RGB rows landed, its
+            // stage free (the MMAs of the tile that used it and of the next one are done)
+            StageCursor ccur(p.per);
+            int cki = 0, ci = i;
+            auto convert = [&](int k) -> bool {
+                const int stage = ccur.stage(cki);
+                const uint32_t phase = ccur.phase;
+                if (++cki == SP_ISSUERS) {
+                    cki = 0;
+                    ccur.next();
+                }
+                const int sl = k % SP_RGB_SLOTS;
+                bool ok = true;
+                if (lane == 0)
+                    ok = wait_or_abort(rgbf0 + 8u * sl,
+                                       static_cast<uint32_t>(k / SP_RGB_SLOTS) & 1u, limit,
+                                       abort_flag, STATUS_TIMEOUT_EPILOGUE) &&
+                         wait_or_abort(empty_bar(stage), phase ^ 1u, limit, abort_flag,
+                                       STATUS_TIMEOUT_EPILOGUE);
+                if (__shfl_sync(0xffffffffu, ok ? 1 : 0, 0) == 0) return false;
+                sp_convert_rgb(p, sbase + C::RING_OFF + stage * p.stage_bytes,
+                               k > 0 && ci != 0 && p.rows > 5 ? 4 : 0,
+                               sbase + p.rgb_off + sl * p.rgb_stage_bytes, 4 * ci - s.pad,
+                               static_cast<int>(threadIdx.x) - 32 * SP_EPI_WARP0);
+                if (++ci == p.Hp) ci = 0;
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(full_bar(stage));
+                    mbar_arrive(rgbe0 + 8u * sl);
+                }
+                return true;
+            };
+            int mapped = 0;  // tiles mapped so far
             for (int k = 0; k < ntiles; ++k) {
+                if constexpr (RGB) {
+                    bool go = true;
+#pragma unroll 1
+                    for (; go && mapped < ntiles && mapped <= k + SP_RGB_AHEAD; ++mapped)
+                        go = convert(mapped);
+                    if (!go) break;
+                }
                 int buf;
                 uint32_t use;
                 issuer_acc_n<SP_ISSUERS>(k, buf, use);
