@@ -1613,8 +1613,10 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
         return cudaErrorInvalidValue;
     }
     // Weight-stationary for 16 -> 16 quaternion channels (the whole expanded weight fits);
-    // pair mode (N = 2 BNQ per MMA) otherwise, unless the tile is so narrow that even
-    // pairs stay far below the tensor pipe's per-instruction cost.
+    // pair mode (N = 2 BNQ per MMA) otherwise, at every tile width: half as many MMAs as quad
+    // mode, each at the same per-instruction cost for the narrow ones (bnq = 16: 151 us against
+    // 196 us for 320 -> 320 channels, 16 images of 40 x 40, 3x3; 28.5 against 37.8 us for
+    // 192 -> 64, 32 of 28 x 28).
     const bool ws_ok = s.Qin == 16 && s.Qout == 16 && s.kh * s.kw <= WS_MAX_TAPS;
     int kappa = pick_kappa(s.Qin, opt.kappa);
     const int bnq = pick_bnq(s.Qout, opt.bnq);
@@ -1624,7 +1626,7 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     else if (opt.mode == 1) mode = MODE_QUAD;
     else if (opt.mode == 2) mode = MODE_PAIR;
     else if (opt.mode == 3) mode = MODE_WS;
-    else mode = ws_ok ? MODE_WS : (bnq >= 32 ? MODE_PAIR : MODE_QUAD);
+    else mode = ws_ok ? MODE_WS : MODE_PAIR;
     if (mode == MODE_WS) {
         if (!ws_ok) {
             snprintf(err, errlen, "weight-stationary mode needs Cin = Cout = 64 and <= %d taps",
@@ -1905,7 +1907,7 @@ bool tc_shortcut_plan(const ConvShape& s, int qout_sc, const TcOptions& opt, int
     int mode;
     if (opt.mode == 1) mode = MODE_QUAD;
     else if (opt.mode == 2) mode = MODE_PAIR;
-    else if (opt.mode == 0) mode = bnq >= 32 ? MODE_PAIR : MODE_QUAD;
+    else if (opt.mode == 0) mode = MODE_PAIR;
     else return false;
     if (mode == MODE_PAIR && kappa == 64 && bnq == 64 && opt.kappa == 0) kappa = 32;
     bool fits = false;
