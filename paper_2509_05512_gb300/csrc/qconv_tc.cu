@@ -185,11 +185,13 @@ struct Cfg {
     static constexpr int SMEM_BYTES = 1024 + BAR_OFF + NUM_BARS * 8 + 16 + 4 * STAGES;
     static_assert(NUM_BARS * 8 + 16 + 4 * STAGES <= FIXED_BYTES - 1024, "barrier area");
     static constexpr bool FITS = SMEM_BYTES <= 227 * 1024;
-    static constexpr uint32_t TMEM_COLS = 8 * BNQ;  // 2 buffers x 4 components x BNQ fp32 columns
+    // 2 buffers x 4 components x BNQ fp32 columns, rounded up to a power of two
+    static constexpr uint32_t TMEM_COLS = BNQ == 48 ? 512 : 8 * BNQ;
     static constexpr int KSTEPS = KAPPA / UMMA_K;
     static constexpr uint32_t DESC_HI = desc_hi(8 * A_ROW_BYTES, desc_layout(A_ROW_BYTES));
     static_assert(KAPPA == 16 || KAPPA == 32 || KAPPA == 64, "KAPPA");
-    static_assert(BNQ == 16 || BNQ == 32 || BNQ == 64, "BNQ");
+    static_assert(BNQ == 16 || BNQ == 32 || BNQ == 64 || (BNQ == 48 && MODE == MODE_PAIR), "BNQ");
+    static_assert(STAGE_BYTES % 1024 == 0, "stages start on swizzle patterns");
 };
 
 // SC: N tiles from p.sc.n_conv on belong to a 1x1 shortcut on the same input, fused into
@@ -587,13 +589,22 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         else if constexpr (SC)
             epilogue_direct_pair_sc<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
                                          p.ktiles, p.sk, limit, abort_flag, geo, &p.sc);
-        else if constexpr (PAR)
-            epilogue_direct_pair<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
-                                      p.ktiles, p.sk, limit, abort_flag,
-                                      ParGeo{par, p.num_n_tiles});
-        else
-            epilogue_direct_pair<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
-                                      p.ktiles, p.sk, limit, abort_flag, linear_geo(geo));
+        else {
+            auto run = [&](auto g) {
+                if (MODE == MODE_PAIR && s.Qout % BNQ != 0)
+                    epilogue_direct_pair<BNQ, true>(s, p.ep, p.y, tmem_base, accf0, acce0,
+                                                    p.num_tiles, p.ktiles, p.sk, limit,
+                                                    abort_flag, g);
+                else
+                    epilogue_direct_pair<BNQ, false>(s, p.ep, p.y, tmem_base, accf0, acce0,
+                                                     p.num_tiles, p.ktiles, p.sk, limit,
+                                                     abort_flag, g);
+            };
+            if constexpr (PAR)
+                run(ParGeo{par, p.num_n_tiles});
+            else
+                run(linear_geo(geo));
+        }
     }
 
     tc_fence_before();
@@ -837,20 +848,26 @@ int grid_for(const TcOptions& opt, int num_sms, int num_tiles) {
     return grid < 1 ? 1 : grid;
 }
 
-// Channel tile of the class form: the BNQ dividing Qout with the fewest estimated clocks over
-// the waves of tiles.  Per 16 input channels a tile's copies (16 KB of pixels, 128 BNQ bytes of
-// letters, at about 33 bytes per clock and SM with every SM loading) outlast its MMAs.
-int par_pick_bnq(int Qout, long long m_tiles, int sms) {
-    const int bs[3] = {64, 32, 16}, cost[3] = {727, 606, 545};
-    int best = 16;
+// Channel tile of the pair mode: the BNQ with the fewest estimated clocks over the waves of
+// tiles.  A K block's copies set the pace, at 1.6-1.9 clocks per row they write (512 of pixels,
+// 4 BNQ of letters, 32- and 64-byte rows alike).  Where no tile of 64 fits, the last tile may
+// reach past Qout (letter rows there are zero, their columns not stored): 80 channels are two
+// tiles of 48 and not five of 16, which copy the pixels five times (145 us against 80 us for
+// 320 -> 320 channels, 16 images of 40 x 40, 3x3).  split: K ranges split evenly between one
+// and two waves.
+int pair_pick_bnq(int Qout, long long m_tiles, int grid, bool split) {
+    int best = 64;
     double best_t = 1e30;
-    for (int i = 0; i < 3; ++i) {
-        if (Qout % bs[i] != 0) continue;
-        const long long tiles = m_tiles * (Qout / bs[i]);
-        const double t = static_cast<double>((tiles + sms - 1) / sms) * cost[i];
+    for (int b = 64; b >= 16; b -= 16) {
+        if (Qout % 64 == 0 && Qout % b != 0) continue;
+        const long long tiles = m_tiles * ((Qout + b - 1) / b);
+        double waves = static_cast<double>((tiles + grid - 1) / grid);
+        if (split && tiles > grid && tiles < 2LL * grid)
+            waves = static_cast<double>(tiles) / grid;
+        const double t = waves * (512 + 4 * b);
         if (t < best_t) {
             best_t = t;
-            best = bs[i];
+            best = b;
         }
     }
     return best;
@@ -1619,7 +1636,7 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     // 192 -> 64, 32 of 28 x 28).
     const bool ws_ok = s.Qin == 16 && s.Qout == 16 && s.kh * s.kw <= WS_MAX_TAPS;
     int kappa = pick_kappa(s.Qin, opt.kappa);
-    const int bnq = pick_bnq(s.Qout, opt.bnq);
+    int bnq = pick_bnq(s.Qout, opt.bnq);
     int mode;
     if (s.sep == 2) mode = MODE_SEPT;
     else if (s.sep) mode = ws_ok ? MODE_WS : MODE_SEP;
@@ -1640,6 +1657,10 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
                  opt.kappa, opt.bnq, s.Qin, s.Qout);
         return cudaErrorInvalidValue;
     }
+    const long long m_tiles = (s.M + BM - 1) / BM;
+    if (mode == MODE_PAIR && opt.mode == 0 && opt.bnq == 0 && opt.kappa == 0)
+        bnq = pair_pick_bnq(s.Qout, m_tiles, opt.max_ctas > 0 ? opt.max_ctas : num_sms,
+                            opt.sk_ws != nullptr);
     // Only two 6-slot stages of 64 x 64 letter blocks plus 64-channel pixel tiles fit in
     // shared memory; 32-channel K blocks give four.
     if (mode == MODE_PAIR && kappa == 64 && bnq == 64 && opt.kappa == 0) kappa = 32;
@@ -1681,9 +1702,8 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     prm.ep = ep;
     prm.kchunks = s.Qin / kappa;
     prm.ktiles = s.kh * s.kw * prm.kchunks;
-    prm.num_n_tiles = s.Qout / bnq;
+    prm.num_n_tiles = (s.Qout + bnq - 1) / bnq;
     prm.y = out;
-    const long long m_tiles = (s.M + BM - 1) / BM;
     const long long tiles = m_tiles * prm.num_n_tiles;
     if (tiles > 0x7fffffffLL) {
         snprintf(err, errlen, "too many tiles");
@@ -1726,6 +1746,9 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
         }
     }
 
+    if (bnq == 48)  // (pair mode without overrides: kappa 16 or 32)
+        return kappa == 32 ? launch_cfg<32, 48, MODE_PAIR>(maps, prm, grid, stream)
+                           : launch_cfg<16, 48, MODE_PAIR>(maps, prm, grid, stream);
 #define QUAN_TC_CASE(K, B)                                                       \
     if (kappa == K && bnq == B)                                                  \
         return mode == MODE_PAIR   ? launch_cfg<K, B, MODE_PAIR>(maps, prm, grid, stream)  \
@@ -1801,8 +1824,9 @@ cudaError_t launch_qconv_tc_parity(const ConvShape& f, const void* dy, const voi
     for (int c = 0; c < 4; ++c)
         m_tiles += (static_cast<long long>(f.N) * sh[c >> 1].n * sw[c & 1].n + BM - 1) / BM;
     const int bnq = s.sep ? pick_bnq(s.Qout, 0)
-                          : par_pick_bnq(s.Qout, m_tiles, opt.max_ctas > 0 ? opt.max_ctas : num_sms);
-    const int num_n = s.Qout / bnq;
+                          : pair_pick_bnq(s.Qout, m_tiles, opt.max_ctas > 0 ? opt.max_ctas : num_sms,
+                                          false);
+    const int num_n = (s.Qout + bnq - 1) / bnq;
     if (m_tiles * num_n > 0x7fffffffLL) {
         snprintf(err, errlen, "too many tiles");
         return cudaErrorInvalidValue;
@@ -1874,6 +1898,11 @@ cudaError_t launch_qconv_tc_parity(const ConvShape& f, const void* dy, const voi
     set_kernel_name(s.sep ? "qconv_tc_kernel<sep_t,kappa=%d,bnq=%d,parity>"
                           : "qconv_tc_kernel<pair,kappa=%d,bnq=%d,parity>",
                     kappa, bnq);
+    if (bnq == 48)
+        return kappa == 32 ? launch_cfg<32, 48, MODE_PAIR, false, true>(maps, prm, grid, stream,
+                                                                        nullptr, par)
+                           : launch_cfg<16, 48, MODE_PAIR, false, true>(maps, prm, grid, stream,
+                                                                        nullptr, par);
 #define QUAN_PAR_CASE(K, B)                                                                \
     if (kappa == K && bnq == B)                                                            \
         return s.sep ? launch_cfg<K, B, MODE_SEPT, false, true>(maps, prm, grid, stream,    \

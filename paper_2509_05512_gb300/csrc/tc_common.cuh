@@ -399,14 +399,17 @@ __device__ __forceinline__ bool gflag_wait_or_abort(const unsigned* flag, uint64
 // each, with the tensor cores busy on the other buffer) overlaps the work on block b.
 // No shared memory is touched (the tensor cores' operand reads keep that pipe busy); the
 // per-channel vectors are read through the L1 cache, 16 bytes at a time.
-template <int BNQ, typename Geo>
+//
+// PAD: the last channel tile may reach past Qout (BNQ does not divide it); its chunks there are
+// computed and not stored.
+template <int BNQ, bool PAD, typename Geo>
 __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const EpilogueArgs& ep,
                                                      void* y, uint32_t tmem_base,
                                                      uint32_t accf0, uint32_t acce0,
                                                      int num_tiles, int ktiles, const SplitK& sk,
                                                      uint64_t limit,
                                                      volatile int* abort_flag, Geo geo) {
-    constexpr int CH = BNQ < 32 ? BNQ : 32;  // columns per TMEM load
+    constexpr int CH = BNQ % 32 == 0 ? 32 : 16;  // columns per TMEM load
     constexpr int NCH = CH / 8;              // 8-channel chunks per load: 2 or 4
     constexpr int SLICES = BNQ / CH;
     constexpr int NB = 2 * SLICES;           // blocks per warp and tile
@@ -482,10 +485,15 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
             return g.m0 + row0 + k;
         };
         const int c_tile = g.n_tile * BNQ + 8 * ci;  // + q Qout + slice offset: lane's channel
+        // block b's first channel in this lane's chunk (past Qout: channel 0's vectors stand in)
+        auto chan_ok = [&](int b) { return !PAD || c_tile + (b % SLICES) * CH < s.Qout; };
+        auto chan = [&](int b) {
+            return chan_ok(b) ? c_tile + (2 * half + b / SLICES) * s.Qout + (b % SLICES) * CH : 0;
+        };
         uint32_t va[CH], vb[CH];
         float sca[8], sha[8], scb[8], shb[8];
         load_block(taddr, 0, va);
-        load_vectors(c_tile + (2 * half) * s.Qout, sca, sha);
+        load_vectors(chan(0), sca, sha);
         tmem_ld_wait();
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -495,14 +503,12 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
             float(&sh)[8] = (b & 1) ? shb : sha;
             float(&scn)[8] = (b & 1) ? sca : scb;
             float(&shn)[8] = (b & 1) ? sha : shb;
-            const int q = 2 * half + b / SLICES;
-            const int cb = c_tile + q * s.Qout + (b % SLICES) * CH;
+            const int cb = chan(b);
+            const bool store = chan_ok(b);
             if (b + 1 < NB) {
                 // next block in flight while this one is processed
                 load_block(taddr, b + 1, vn);
-                load_vectors(c_tile + (2 * half + (b + 1) / SLICES) * s.Qout +
-                                 ((b + 1) % SLICES) * CH,
-                             scn, shn);
+                load_vectors(chan(b + 1), scn, shn);
             } else {
                 // the tile's accumulator is in registers: hand the buffer back
                 tc_fence_before();
@@ -541,7 +547,7 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
 #pragma unroll
                 for (int k = 0; k < NCH; ++k) {
                     r4[k] = make_uint4(0u, 0u, 0u, 0u);
-                    if (row0 + k < g.rows)
+                    if (store && row0 + k < g.rows)
                         r4[k] = ld_global_na(res + pix(k) * Cout + cb);
                 }
             }
@@ -580,7 +586,7 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
                         fmaf(sc[2 * t + 1], E[k][2 * t + 1], sh[2 * t + 1]) + rz[2 * t + 1];
                     w[t] = pack_bf16x2(activate(z0, s.act), activate(z1, s.act));
                 }
-                if (row0 + k < g.rows)
+                if (store && row0 + k < g.rows)
                     st_global_na(out + pix(k) * Cout + cb,
                                  make_uint4(w[0], w[1], w[2], w[3]));
             }

@@ -151,6 +151,7 @@ PARITY_DATA_CASES = [
     ("par_k2", 2, 10, 12, 64, 64, 2, 2, 0),
     ("par_k5_pad4", 1, 11, 10, 64, 64, 5, 2, 4),
     ("par_tiles", 5, 30, 29, 256, 128, 3, 2, 1),     # several tiles and a tail per class
+    ("par_bnq48", 9, 40, 38, 320, 64, 3, 2, 1),      # 80 channels: two tiles of 48
     ("par_wrap", 24, 60, 58, 64, 64, 3, 2, 1),       # more tiles than SMs
 ]
 

@@ -586,6 +586,27 @@ def test_simt_small_layers(case):
     check(spec, expect_path=quan.QUAN_PATH_SIMT)
 
 
+PAIR_TILE_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad, extra, grid, bnq: channel tiles the pair mode
+    # chooses, the last one reaching past the channels where it does not divide them
+    ("bnq48_pad", 2, 13, 11, 192, 320, 3, 1, 1, {"residual": True, "bias": True}, 2, 48),
+    ("bnq64_pad", 2, 25, 21, 128, 448, 3, 2, 1, {"act": quan.QUAN_ACT_SILU}, 2, 64),
+    ("bnq48_kappa16", 2, 13, 11, 64, 192, 5, 1, 2, {}, 2, 48),
+    ("bnq48_exact", 2, 13, 11, 128, 384, 3, 1, 1, {"iqbn": False}, 2, 48),
+    ("bnq16_few", 1, 10, 9, 256, 256, 3, 1, 1, {}, 0, 16),
+]
+
+
+@pytest.mark.parametrize("case", PAIR_TILE_CASES, ids=[c[0] for c in PAIR_TILE_CASES])
+def test_pair_channel_tiles(case):
+    name, N, H, W, Cin, Cout, k, s, p, extra, grid, bnq = case
+    quan.quan_set_tc_tiles(0, 0, grid, 0)
+    check(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(305, len(name)), **extra),
+          path=quan.QUAN_PATH_TC)
+    assert quan.quan_last_kernel().startswith("qconv_tc_kernel<pair,")
+    assert quan.quan_last_kernel().endswith("bnq=%d>" % bnq), quan.quan_last_kernel()
+
+
 NARROW_CASES = [
     # name, N, H, W, Cin, Cout, k, stride, pad, extra: bf16 layers off the tcgen05 channel
     # grid on warp-level MMAs: K tails, channel tiles past 64, one pixel buffer, few pixels
