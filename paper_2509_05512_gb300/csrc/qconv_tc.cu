@@ -197,8 +197,9 @@ struct Cfg {
 // SC: N tiles from p.sc.n_conv on belong to a 1x1 shortcut on the same input, fused into
 // the launch (ScParams): their K blocks are the filter tap p.sc.tap's only, their letters
 // come from `scm`, and the epilogue writes them to the shortcut's output.
-// PAR: the pixel classes of `par` (tmap_x unused).
-template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false>
+// PAR: the pixel classes of `par` (tmap_x unused).  PAD: the last channel tile may reach past
+// Qout (an instance of its own: the epilogue's checks cost the epilogue-bound layers 15%).
+template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     qconv_tc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                     const __grid_constant__ CUtensorMap tmap_wr,
@@ -589,22 +590,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         else if constexpr (SC)
             epilogue_direct_pair_sc<BNQ>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
                                          p.ktiles, p.sk, limit, abort_flag, geo, &p.sc);
-        else {
-            auto run = [&](auto g) {
-                if (MODE == MODE_PAIR && s.Qout % BNQ != 0)
-                    epilogue_direct_pair<BNQ, true>(s, p.ep, p.y, tmem_base, accf0, acce0,
-                                                    p.num_tiles, p.ktiles, p.sk, limit,
-                                                    abort_flag, g);
-                else
-                    epilogue_direct_pair<BNQ, false>(s, p.ep, p.y, tmem_base, accf0, acce0,
-                                                     p.num_tiles, p.ktiles, p.sk, limit,
-                                                     abort_flag, g);
-            };
-            if constexpr (PAR)
-                run(ParGeo{par, p.num_n_tiles});
-            else
-                run(linear_geo(geo));
-        }
+        else if constexpr (PAR)
+            epilogue_direct_pair<BNQ, PAD>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
+                                           p.ktiles, p.sk, limit, abort_flag,
+                                           ParGeo{par, p.num_n_tiles});
+        else
+            epilogue_direct_pair<BNQ, PAD>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
+                                           p.ktiles, p.sk, limit, abort_flag, linear_geo(geo));
     }
 
     tc_fence_before();
@@ -749,7 +741,7 @@ cudaError_t set_smem_once(K kern, int bytes, std::atomic<unsigned long long>& do
     return cudaSuccess;
 }
 
-template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false>
+template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false>
 cudaError_t launch_cfg(const CUtensorMap maps[6], const TcParams& prm, int grid,
                        cudaStream_t stream, const ScMaps* scm = nullptr,
                        const ParOf<PAR>& par = {}) {
@@ -757,7 +749,7 @@ cudaError_t launch_cfg(const CUtensorMap maps[6], const TcParams& prm, int grid,
     if constexpr (!C::FITS || (SC && MODE != MODE_PAIR && MODE != MODE_QUAD)) {
         return cudaErrorInvalidValue;
     } else {
-        auto kern = qconv_tc_kernel<KAPPA, BNQ, MODE, SC, PAR>;
+        auto kern = qconv_tc_kernel<KAPPA, BNQ, MODE, SC, PAR, PAD>;
         static std::atomic<unsigned long long> attr_done{0};
         cudaError_t e = set_smem_once(kern, C::SMEM_BYTES, attr_done);
         if (e != cudaSuccess) return e;
@@ -859,7 +851,7 @@ int pair_pick_bnq(int Qout, long long m_tiles, int grid, bool split) {
     int best = 64;
     double best_t = 1e30;
     for (int b = 64; b >= 16; b -= 16) {
-        if (Qout % 64 == 0 && Qout % b != 0) continue;
+        if (Qout % b != 0 && (Qout % 64 == 0 || b < 48)) continue;
         const long long tiles = m_tiles * ((Qout + b - 1) / b);
         double waves = static_cast<double>((tiles + grid - 1) / grid);
         if (split && tiles > grid && tiles < 2LL * grid)
@@ -1449,99 +1441,159 @@ cudaError_t launch_stem_pool(const ConvShape& s, const void* x, const void* cons
 // ---------------------------------------------------------------- weight gradient
 constexpr int DW_SMEM_MAX = 232448;  // dynamic shared memory a CTA may opt into
 
-// Tiling of the tensor-core weight gradient (see qconv_dw.cuh); false if the shape has none.
-bool dw_plan(const ConvShape& s, int num_sms, dwk::DwParams* p) {
+// First row and column of x's walk: floor(-pad / stride).
+int dw_org(const ConvShape& s) { return s.stride == 1 ? -s.pad : -((s.pad + 1) / 2); }
+
+// Taps of a row per CTA share, and the extra columns of the walk they need.
+void dw_row_share(const ConvShape& s, int* ndw, int* slots, int* n0) {
+    const int g = (s.kw + 7) / 8;
+    *ndw = (s.kw + g - 1) / g;
+    *slots = *ndw < s.stride ? *ndw : s.stride;
+    *n0 = (*ndw + *slots - 1) / *slots;
+}
+
+// The shapes the kernel is offered: output rows of at most 256 pixels (128 at stride 2) whose
+// blocks of whole rows would fit, corner offsets of the walk within the im2col encoding, and a
+// walk of 32-bit positions.
+bool dw_accepts(const ConvShape& s) {
     if (s.stride < 1 || s.stride > 2 || s.Cin % 64 != 0 || s.Cout % 64 != 0) return false;
     if (s.Cout > 256 && s.Cout % 256 != 0) return false;
+    int ndw, slots, n0;
+    dw_row_share(s, &ndw, &slots, &n0);
+    const int org = dw_org(s), Wp = s.Wo + n0 - 1;
+    if (static_cast<long long>(s.N) * s.Ho * Wp > 0x7fffffffLL - 4096) return false;
+    auto corner = [](int v) { return v >= -128 && v <= 127; };
+    if (!corner(org) || n0 > 128) return false;
+    for (int a = 0; a < s.stride; ++a) {
+        const int Hc = (s.H - (a < s.H ? a : 0) + s.stride - 1) / s.stride;
+        const int Wc = (s.W - (a < s.W ? a : 0) + s.stride - 1) / s.stride;
+        if (!corner(Wp - Wc + org) || !corner(s.Ho - Hc + org)) return false;
+    }
+    const long long boxes = 2 + (s.Cout <= 256 ? s.Cout : 256) / 64;
+    for (int m = 8; m <= 16; m += 8) {
+        const long long w = (s.Wo + m - 1) / m * m;
+        if (w * s.stride > 256) continue;
+        for (long long P = w; P <= 256 && P <= 8 * w; P += w)
+            if (P % 16 == 0 &&
+                (DW_SMEM_MAX - 5376 - P * 128 * s.stride * s.stride) / (boxes * P * 128) >= 2)
+                return true;
+    }
+    return false;
+}
+
+// Tiling of the tensor-core weight gradient (see qconv_dw.cuh): the share of a CTA (chunks, tap
+// rows, output channels) and block size with the fewest estimated clocks.  Per 16 pixels a CTA
+// issues one MMA per unit pair (N = 64: 49 clocks, bound by operand reads, about 70 beside the
+// copies; 128, 192, 256: 64, 96, 128 and about 8 more) while its copies bring 16 rows of 128 bytes per
+// box at about 35 bytes per clock and SM.
+bool dw_plan(const ConvShape& s, int num_sms, dwk::DwParams* p) {
     dwk::DwParams q = {};
     q.sep = s.sep ? 1 : 0;
     q.stride = s.stride;
+    q.N = s.N;
     q.Ho = s.Ho; q.Wo = s.Wo; q.Qin = s.Qin; q.Qout = s.Qout;
     q.kh = s.kh; q.kw = s.kw; q.pad = s.pad; q.taps = s.kh * s.kw;
     q.nxc = s.Cin / 64;
-    q.units = q.taps * q.nxc;
-    q.npairs = (q.units + 1) / 2;
-    q.ncols = s.Cout <= 256 ? s.Cout : 256;
-    q.nyb = q.ncols / 64;
-    int a_max = 512 / q.ncols;
-    if (a_max > dwk::MAX_PAIRS) a_max = dwk::MAX_PAIRS;
-    if (a_max > q.npairs) a_max = q.npairs;
-    // the most unit pairs per CTA for which some pixel block fits; for those, the block
-    // shape (Ht rows x Wbox columns, Wbox a multiple of 8 so a block is whole 1024-byte
-    // swizzle atoms) with the least padding, preferring three or more pipeline stages
-    bool found = false;
-    for (int a_per = a_max; a_per >= 1 && !found; --a_per) {
-        double best = 1e30;
-        const int wcand[2] = {(s.Wo + 7) / 8 * 8, (s.Wo + 15) / 16 * 16};
-        for (int wc = 0; wc < 2; ++wc) {
-            const int Wbox = wcand[wc];
-            if (Wbox * s.stride > 256) continue;
-            for (int Ht = 1; Ht <= 8; ++Ht) {
-                const int P = Wbox * Ht;
-                if (P % 16 != 0 || P > 256 || Ht * s.stride > 256) continue;
-                const long long stage =
-                    static_cast<long long>(2 * a_per + q.nyb) * P * dwk::BOX_ROW;
-                long long stages = (DW_SMEM_MAX - 1024 - dwk::BAR_BYTES -
-                                    dwk::tail_bytes(P)) /
-                                   stage;
-                if (stages > dwk::MAX_STAGES) stages = dwk::MAX_STAGES;
-                if (stages < 2) continue;
-                const int rb = (s.Ho + Ht - 1) / Ht;
-                double score = static_cast<double>(P) * rb / (static_cast<double>(s.Wo) * s.Ho);
-                if (stages < 3) score *= 1.15;
-                if (P < 32) score *= 1.2;
-                if (score < best) {
-                    best = score;
-                    q.a_per = a_per;
-                    q.Wbox = Wbox; q.Ht = Ht; q.P = P; q.rblocks = rb;
-                    q.stages = static_cast<int>(stages);
+    q.org = dw_org(s);
+    q.lone = s.stride == 2 ? (s.H == 1 ? 1 : 0) | (s.W == 1 ? 2 : 0) : 0;
+    dw_row_share(s, &q.ndw, &q.slots, &q.n0);
+    q.gdw = (s.kw + q.ndw - 1) / q.ndw;
+    q.Wp = s.Wo + q.n0 - 1;
+    const long long walk = static_cast<long long>(s.N) * s.Ho * q.Wp;
+    // The accumulation error grows with the pixels one accumulator sums: no fewer splits than
+    // two (narrow outputs: up to eight) unit pairs and 256 output channels per CTA would give.
+    long long min_splits;
+    {
+        const int cols = s.Cout < 256 ? s.Cout : 256, all = (q.taps * q.nxc + 1) / 2;
+        int per = 512 / cols < 8 ? 512 / cols : 8;
+        if (per > all) per = all;
+        min_splits = num_sms / (static_cast<long long>((all + per - 1) / per) * (s.Cout / cols));
+        if (min_splits < 1) min_splits = 1;
+    }
+    double best = 1e30;
+    for (int ncols = 64; ncols <= 256; ncols += 64) {
+        if (s.Cout % ncols != 0) continue;
+        for (int ndh = 1; ndh <= s.kh && ndh <= 16; ++ndh)
+            for (int nch = 1; nch <= q.nxc && nch <= 16; ++nch) {
+                const int units = nch * ndh * q.ndw, pairs = (units + 1) / 2;
+                if (pairs > dwk::MAX_PAIRS || pairs * ncols > 512) break;
+                const int nx = nch * ndh * q.slots, nyb = ncols / 64;
+                const int gch = (q.nxc + nch - 1) / nch, gdh = (s.kh + ndh - 1) / ndh;
+                const long long groups = static_cast<long long>(gch) * gdh * q.gdw * (s.Cout / ncols);
+                for (int P = 128; P >= 16; P /= 2) {
+                    const int xstride = ((P + q.n0 - 1) * dwk::BOX_ROW + 1023) / 1024 * 1024;
+                    const int stage = nx * xstride + nyb * P * dwk::BOX_ROW;
+                    int stages = (DW_SMEM_MAX - 1024 - dwk::BAR_BYTES) / stage;
+                    if (stages > dwk::MAX_STAGES) stages = dwk::MAX_STAGES;
+                    if (stages < 2) continue;
+                    const long long kblocks = (walk + P - 1) / P;
+                    const double rows = static_cast<double>(nx) * (P + q.n0 - 1) + nyb * P;
+                    const double mma = pairs * (ncols == 64 ? 70.0 : ncols * 0.5 + 8.0) * (P / 16);
+                    double block = rows * 128.0 / 35.0;
+                    if (mma > block) block = mma;
+                    block += 150.0;                       // the stage's hand-over
+                    if (stages < 3) block *= 1.2;
+                    // splits that fill one or a few waves of CTAs
+                    long long splits = 1;
+                    double t = 1e30;
+                    for (int w = 1; w <= 4; ++w) {
+                        long long n = static_cast<long long>(w) * num_sms / groups;
+                        if (n < min_splits) n = min_splits;
+                        if (n > kblocks) n = kblocks;
+                        const long long waves = (groups * n + num_sms - 1) / num_sms;
+                        const double tn = waves * ((kblocks + n - 1) / n * block +
+                                                   8.0 * pairs * ncols + 4000.0);  // fold, start
+                        if (tn < t) {
+                            t = tn;
+                            splits = n;
+                        }
+                    }
+                    if (t >= best || groups * splits > 0x7fffffffLL) continue;
+                    best = t;
+                    q.nch = nch; q.ndh = ndh;
+                    q.units = units; q.npairs = pairs;
+                    q.gch = gch; q.gdh = gdh;
+                    q.nx = nx; q.ncols = ncols; q.nyb = nyb;
+                    q.groups = static_cast<int>(groups);
+                    q.splits = static_cast<int>(splits);
+                    q.P = P; q.kblocks = kblocks; q.stages = stages;
+                    q.xbox_bytes = static_cast<uint32_t>((P + q.n0 - 1) * dwk::BOX_ROW);
+                    q.xbox_stride = static_cast<uint32_t>(xstride);
+                    q.ybox_bytes = static_cast<uint32_t>(P * dwk::BOX_ROW);
                     q.stage_bytes = static_cast<uint32_t>(stage);
                 }
             }
-        }
-        found = best < 1e29;
     }
-    if (!found) return false;
-    q.pair_groups = (q.npairs + q.a_per - 1) / q.a_per;
-    q.groups = q.pair_groups * (s.Cout / q.ncols);
-    // the last group of unit pairs may hold fewer boxes than the others: every producer
-    // needs at least one box of the smallest stage
-    const int last_pairs = q.npairs - (q.pair_groups - 1) * q.a_per;
-    q.producers = 2 * last_pairs + q.nyb;
-    if (q.producers > dwk::PRODUCERS) q.producers = dwk::PRODUCERS;
-    q.lone = s.stride == 2 ? (s.H == 1 ? 1 : 0) | (s.W == 1 ? 2 : 0) : 0;
-    q.kblocks = static_cast<long long>(s.N) * q.rblocks;
-    long long splits = num_sms / q.groups;
-    if (splits < 1) splits = 1;
-    if (splits > q.kblocks) splits = q.kblocks;
-    q.splits = static_cast<int>(splits);
-    if (static_cast<long long>(q.groups) * q.splits > 0x7fffffffLL) return false;
+    // (one chunk, one tap row, 64 channels and blocks of 16 always fit)
+    q.producers = q.nx + q.nyb < dwk::PRODUCERS ? q.nx + q.nyb : dwk::PRODUCERS;
     uint32_t cols = 32;
-    while (cols < static_cast<uint32_t>(q.a_per * q.ncols)) cols <<= 1;
+    while (cols < static_cast<uint32_t>(q.npairs * q.ncols)) cols <<= 1;
     q.tmem_cols = cols;
     *p = q;
-    return true;
+    return best < 1e29;
 }
 
-// [N][H][W][C] bf16, boxes of 64 channels x Wbox columns x Ht rows of one image, SW128; with
-// step = 2 the pixels of parity (a, b): rows a, a + 2, .. and columns b, b + 2, ..
-bool encode_dw_map(CUtensorMap* map, const void* t, int C, int W, int H, int N, int Wbox,
-                   int Ht, int step = 1, int a = 0, int b = 0) {
+// im2col walk of a [N][H][W][C] tensor for the weight gradient, boxes of 64 channels x `box`
+// positions: rows of Wp columns from column org, Ho rows from row org; with step = 2 over the
+// pixels of parity (a, b): rows a, a + 2, .. and columns b, b + 2, ..
+bool encode_dw_map(CUtensorMap* map, const void* t, int C, int W, int H, int N, int Wp, int Ho,
+                   int org, int box, int step = 1, int a = 0, int b = 0) {
     const cuuint64_t e = static_cast<cuuint64_t>(C) * 2;  // bytes per pixel
     if (a >= H) a = 0;  // an empty class: any map stands in (its boxes are read past the end)
     if (b >= W) b = 0;
-    const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C),
-                                static_cast<cuuint64_t>((W - b + step - 1) / step),
-                                static_cast<cuuint64_t>((H - a + step - 1) / step),
-                                static_cast<cuuint64_t>(N)};
+    const int Wc = (W - b + step - 1) / step, Hc = (H - a + step - 1) / step;
+    const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(Wc),
+                                static_cast<cuuint64_t>(Hc), static_cast<cuuint64_t>(N)};
     const cuuint64_t strides[3] = {e * step, e * W * step, e * W * H};
-    const cuuint32_t box[4] = {64, static_cast<cuuint32_t>(Wbox), static_cast<cuuint32_t>(Ht), 1};
+    const int lower[2] = {org, org};
+    const int upper[2] = {Wp - Wc + org, Ho - Hc + org};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const char* base = static_cast<const char*>(t) + (static_cast<size_t>(a) * W + b) * e;
-    const CUresult r = g_encode_tiled(
-        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<char*>(base), dims, strides, box,
-        estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = g_encode_im2col(
+        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<char*>(base), dims, strides, lower,
+        upper, 64, static_cast<cuuint32_t>(box), estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 
@@ -1746,9 +1798,15 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
         }
     }
 
-    if (bnq == 48)  // (pair mode without overrides: kappa 16 or 32)
-        return kappa == 32 ? launch_cfg<32, 48, MODE_PAIR>(maps, prm, grid, stream)
-                           : launch_cfg<16, 48, MODE_PAIR>(maps, prm, grid, stream);
+#define QUAN_PAD_CASE(K, B)                                     \
+    if (kappa == K && bnq == B && (B == 48 || s.Qout % B != 0)) \
+        return launch_cfg<K, B, MODE_PAIR, false, false, true>(maps, prm, grid, stream);
+    // (pair mode without overrides: kappa 16 or 32)
+    QUAN_PAD_CASE(16, 48)
+    QUAN_PAD_CASE(16, 64)
+    QUAN_PAD_CASE(32, 48)
+    QUAN_PAD_CASE(32, 64)
+#undef QUAN_PAD_CASE
 #define QUAN_TC_CASE(K, B)                                                       \
     if (kappa == K && bnq == B)                                                  \
         return mode == MODE_PAIR   ? launch_cfg<K, B, MODE_PAIR>(maps, prm, grid, stream)  \
@@ -1898,11 +1956,15 @@ cudaError_t launch_qconv_tc_parity(const ConvShape& f, const void* dy, const voi
     set_kernel_name(s.sep ? "qconv_tc_kernel<sep_t,kappa=%d,bnq=%d,parity>"
                           : "qconv_tc_kernel<pair,kappa=%d,bnq=%d,parity>",
                     kappa, bnq);
-    if (bnq == 48)
-        return kappa == 32 ? launch_cfg<32, 48, MODE_PAIR, false, true>(maps, prm, grid, stream,
-                                                                        nullptr, par)
-                           : launch_cfg<16, 48, MODE_PAIR, false, true>(maps, prm, grid, stream,
-                                                                        nullptr, par);
+#define QUAN_PAD_CASE(K, B)                                                                  \
+    if (kappa == K && bnq == B && (B == 48 || s.Qout % B != 0))                              \
+        return launch_cfg<K, B, MODE_PAIR, false, true, true>(maps, prm, grid, stream, nullptr, \
+                                                              par);
+    QUAN_PAD_CASE(16, 48)
+    QUAN_PAD_CASE(16, 64)
+    QUAN_PAD_CASE(32, 48)
+    QUAN_PAD_CASE(32, 64)
+#undef QUAN_PAD_CASE
 #define QUAN_PAR_CASE(K, B)                                                                \
     if (kappa == K && bnq == B)                                                            \
         return s.sep ? launch_cfg<K, B, MODE_SEPT, false, true>(maps, prm, grid, stream,    \
@@ -2105,8 +2167,7 @@ cudaError_t launch_qconv_stem_pool_rgb(const ConvShape& s, const float* rgb,
 }
 
 bool bwd_weight_tc_supported(const ConvShape& s, const void* x, const void* dy) {
-    dwk::DwParams p;
-    return dw_plan(s, 152, &p) && reinterpret_cast<uintptr_t>(x) % 16 == 0 &&
+    return dw_accepts(s) && reinterpret_cast<uintptr_t>(x) % 16 == 0 &&
            reinterpret_cast<uintptr_t>(dy) % 16 == 0;
 }
 
@@ -2115,7 +2176,7 @@ cudaError_t launch_bwd_weight_tc(const ConvShape& s, const void* x, const void* 
                                  unsigned long long wait_limit_ns, cudaStream_t stream,
                                  char* err, size_t errlen) {
     dwk::DwParams p;
-    if (!dw_plan(s, num_sms, &p) || !bwd_weight_tc_supported(s, x, dy)) {
+    if (!bwd_weight_tc_supported(s, x, dy) || !dw_plan(s, num_sms, &p)) {
         snprintf(err, errlen, "no tensor-core weight-gradient tiling for this shape");
         return cudaErrorInvalidValue;
     }
@@ -2125,12 +2186,12 @@ cudaError_t launch_bwd_weight_tc(const ConvShape& s, const void* x, const void* 
     }
     CUtensorMap mdy;
     dwk::DwMaps mx;
-    bool ok = encode_dw_map(&mdy, dy, s.Cout, s.Wo, s.Ho, s.N, p.Wbox, p.Ht);
+    bool ok = encode_dw_map(&mdy, dy, s.Cout, s.Wo, s.Ho, s.N, p.Wp, s.Ho, 0, p.P);
     for (int i = 0; ok && i < 4; ++i)
         ok = i > 0 && s.stride == 1
                  ? (mx.x[i] = mx.x[0], true)
-                 : encode_dw_map(&mx.x[i], x, s.Cin, s.W, s.H, s.N, p.Wbox, p.Ht, s.stride,
-                                 i >> 1, i & 1);
+                 : encode_dw_map(&mx.x[i], x, s.Cin, s.W, s.H, s.N, p.Wp, s.Ho, p.org,
+                                 p.P + p.n0 - 1, s.stride, i >> 1, i & 1);
     if (!ok) {
         snprintf(err, errlen, "tensor-map encode failed for the weight gradient");
         return cudaErrorInvalidValue;
@@ -2143,13 +2204,12 @@ cudaError_t launch_bwd_weight_tc(const ConvShape& s, const void* x, const void* 
     p.dwi = dw[1];
     p.dwj = dw[2];
     p.dwk = dw[3];
-    const int smem = p.stages * static_cast<int>(p.stage_bytes) + dwk::BAR_BYTES +
-                     dwk::tail_bytes(p.P) + 1024;
+    const int smem = p.stages * static_cast<int>(p.stage_bytes) + dwk::BAR_BYTES + 1024;
     static std::atomic<unsigned long long> attr_done{0};
     cudaError_t e = set_smem_once(dwk::qconv_dw_kernel, DW_SMEM_MAX, attr_done);
     if (e != cudaSuccess) return e;
     set_kernel_name(p.sep ? "qconv_dw_kernel<pairs=%d,n=%d,sep>" : "qconv_dw_kernel<pairs=%d,n=%d>",
-                    p.a_per, p.ncols);
+                    p.npairs, p.ncols);
     return launch_pdl(dwk::qconv_dw_kernel, dim3(static_cast<unsigned>(p.groups * p.splits)),
                       dim3(dwk::THREADS), static_cast<size_t>(smem), stream, mx, mdy, p);
 }

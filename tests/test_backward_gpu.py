@@ -311,6 +311,11 @@ PARITY_WEIGHT_CASES = [
     ("dwp_pad0", 1, 9, 8, 64, 128, 3, 2, 0),
     ("dwp_pad2", 1, 8, 9, 64, 64, 3, 2, 2),          # taps start two rows above the image
     ("dwp_k1_odd", 2, 13, 15, 64, 192, 1, 2, 0),
+    ("dwp_k9", 1, 14, 12, 64, 64, 9, 1, 4),          # two groups of taps of a row (5 and 4)
+    ("dwp_k9_s2", 1, 17, 15, 64, 64, 9, 2, 4),
+    ("dwp_odd_chunks", 3, 11, 13, 192, 192, 3, 1, 1),  # three chunks, two per CTA
+    ("dwp_k2_s2", 2, 12, 10, 64, 128, 2, 2, 0),      # no extra column
+    ("dwp_long_walk", 9, 40, 38, 128, 128, 3, 1, 1), # several blocks per CTA, a tail
     ("dwp_short_group", 1, 9, 10, 128, 256, 3, 2, 1),  # 9 pairs, 2 per CTA, the last alone
 ]
 
