@@ -141,12 +141,19 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
 }
 
 // Sum of the partial rows per channel in a fixed order (row lane rl takes rows rl, rl + 128,
-// ..., compensated fp32; then the 128 lanes as a tree in fp64), then mean = K + S1 / n and
-// var = max(S2 / n - (S1 / n)^2, 0) (these last few operations per channel in fp64; the
-// row sums stay in fp32, the double-precision rate of this part being low).
+// ..., compensated fp32; then the 128 lanes as a tree, also compensated), then
+// mean = K + S1 / n and var = max(S2 / n - (S1 / n)^2, 0) (these last few operations per
+// channel in fp64; the sums stay in fp32 pairs, the double-precision rate of this part being
+// low: the tree in fp64 took 9 us).
 // Block: 8 channels x 128 row lanes, so a lane's chain is a few loads long (32 channels x 32
 // lanes, 19 rows each and 32 lanes added one by one, took 8.4 us for 256 channels).
 constexpr int FIN_C = 8;
+// (s, e) += (s2, e2): the sum's rounding error, exact by Knuth's two-sum, goes to e.
+__device__ __forceinline__ void pair_add(float& s, float& e, float s2, float e2) {
+    const float t = s + s2, b = t - s;
+    e = e + e2 + ((s - (t - b)) + (s2 - b));
+    s = t;
+}
 __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16* __restrict__ x,
                                                              long long npix, int C, int rows,
                                                              const float* __restrict__ part,
@@ -154,7 +161,7 @@ __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16
                                                              float* __restrict__ var) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    __shared__ double red[2][FIN_C][32];
+    __shared__ float2 red[2][FIN_C][32];
     const int cl = threadIdx.x % FIN_C, rl = threadIdx.x / FIN_C;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int c = blockIdx.x * FIN_C + cl;
@@ -166,26 +173,32 @@ __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16
             kahan_add(t2, e2, part[static_cast<size_t>(r) * 2 * C + C + c]);
         }
     }
-    double d1 = static_cast<double>(t1) - e1, d2 = static_cast<double>(t2) - e2;
+    e1 = -e1;  // (the running compensation is what to subtract)
+    e2 = -e2;
+    auto merge = [&](int k) {
+        const float u1 = __shfl_xor_sync(0xffffffffu, t1, k);
+        const float f1 = __shfl_xor_sync(0xffffffffu, e1, k);
+        const float u2 = __shfl_xor_sync(0xffffffffu, t2, k);
+        const float f2 = __shfl_xor_sync(0xffffffffu, e2, k);
+        pair_add(t1, e1, u1, f1);
+        pair_add(t2, e2, u2, f2);
+    };
     // the warp's four row lanes of each channel (lanes cl, cl + 8, ..)
 #pragma unroll
-    for (int k = FIN_C; k < 32; k *= 2) {
-        d1 += __shfl_xor_sync(0xffffffffu, d1, k);
-        d2 += __shfl_xor_sync(0xffffffffu, d2, k);
-    }
+    for (int k = FIN_C; k < 32; k *= 2) merge(k);
     if (lane < FIN_C) {
-        red[0][cl][warp] = d1;
-        red[1][cl][warp] = d2;
+        red[0][cl][warp] = make_float2(t1, e1);
+        red[1][cl][warp] = make_float2(t2, e2);
     }
     __syncthreads();
     if (warp < FIN_C) {  // warp w finishes channel w
-        d1 = red[0][warp][lane];
-        d2 = red[1][warp][lane];
+        t1 = red[0][warp][lane].x;
+        e1 = red[0][warp][lane].y;
+        t2 = red[1][warp][lane].x;
+        e2 = red[1][warp][lane].y;
 #pragma unroll
-        for (int k = 1; k < 32; k *= 2) {
-            d1 += __shfl_xor_sync(0xffffffffu, d1, k);
-            d2 += __shfl_xor_sync(0xffffffffu, d2, k);
-        }
+        for (int k = 1; k < 32; k *= 2) merge(k);
+        const double d1 = static_cast<double>(t1) + e1, d2 = static_cast<double>(t2) + e2;
         const int cw = blockIdx.x * FIN_C + warp;
         if (lane == 0 && cw < C) {
             const double inv_n = 1.0 / static_cast<double>(npix);
