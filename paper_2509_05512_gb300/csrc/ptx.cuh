@@ -110,6 +110,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* map, uint3
         : "memory");
 }
 
+// 2-D tiled load of a CTA pair: `bar` (a shared::cluster address) may be the peer's barrier.
+__device__ __forceinline__ void tma_load_2d_cg2(uint32_t dst, const void* map, uint32_t bar,
+                                                int x, int y, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile"
+        ".mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "l"(policy)
+        : "memory");
+}
+
 // 5-D tiled load (coordinates may be past the end: the box is zero-filled).
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const void* map, uint32_t bar, int c0,
                                             int c1, int c2, int c3, int c4, uint64_t policy) {

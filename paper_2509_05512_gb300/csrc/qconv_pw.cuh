@@ -25,6 +25,16 @@
 // the number of blocks), and the blocks of one pixel tile run on neighbouring CTAs, so a
 // pixel tile read for one block is still in L2 for the others.
 //
+// CTA pairs (CG2; stride 1, an even number of channel blocks).  Alone, a CTA needs 32 KB of
+// pixels per 512 clocks of MMAs from a ring of three stages: the copies' latency and the L2
+// traffic (every channel block's CTA copies every pixel) set the pace, 116 us for the neck
+// layer of 16 x 80 x 80 pixels, 512 -> 1024 channels.  A pair (tcgen05 cta_group::2) runs
+// M = 256 MMAs over two channel blocks: each CTA holds the A rows of its own block and HALF of
+// the tile's pixels, 128, and the tensor cores exchange the halves, so a stage is 16 KB, the
+// ring six stages deep and the traffic half: 100 us.  The pixels of both CTAs complete on
+// the even CTA's barrier (cta_group::2 copies), whose issuer runs both tensor cores; commits
+// are multicast, and accumulators are handed back by both epilogues to the even CTA.
+//
 // Roles (20 warps, one CTA per SM, persistent):
 //   warp 0       TMA producer (one lane);
 //   warp 1       TMEM owner and MMA issuer (one lane): per tile Cin / 16 MMAs of
@@ -70,8 +80,8 @@ struct PwCfg {
     // A (the expanded weight, kchunks x 16 KB) sits at 0, the barriers in the next 1 KB,
     // the ring after them; a_bytes depends on Cin
     static int ring_off(int kchunks) { return kchunks * CHUNK + 1024; }
-    static int max_stages(int kchunks) {
-        const int n = (SMEM_BYTES - 1024 - ring_off(kchunks)) / STAGE;
+    static int max_stages(int kchunks, int stage = STAGE) {
+        const int n = (SMEM_BYTES - 1024 - ring_off(kchunks)) / stage;
         return n < MAX_STAGES ? n : MAX_STAGES;
     }
     static_assert(NUM_BARS * 8 + 16 <= 1024, "pointwise barriers");
@@ -86,9 +96,15 @@ bool pw_ok(const ConvShape& s, const EpilogueArgs& ep) {
     return true;
 }
 
+// CTA pairs: stride 1, two channel blocks to a pair, at least one whole tile of pixels.
+bool pw_cg2_ok(const ConvShape& s) {
+    return s.stride == 1 && s.Cout % 256 == 0 && s.M >= PW_NPIX;
+}
+
 // A[R][k] for the CTA's channel block, K-major 64-channel chunks of 128 rows x 128 bytes
 // with the 128-byte swizzle (16-byte unit u of row R at unit u ^ (R mod 8)).  One 16-byte
 // unit per item: eight consecutive input channels of one component, one letter row.
+template <bool CG2>
 __device__ __forceinline__ void pw_expand(const PwParams& p, uint8_t* smem, int mb, int et,
                                           int lane, uint32_t bready_bar) {
     constexpr int ET = PW_EXP_WARPS * 32;
@@ -108,10 +124,15 @@ __device__ __forceinline__ void pw_expand(const PwParams& p, uint8_t* smem, int 
     }
     fence_proxy_async_smem();
     __syncwarp();
-    if (lane == 0) mbar_arrive(bready_bar);
+    if (lane == 0) {
+        if constexpr (CG2)
+            mbar_arrive_cluster(mapa_shared(bready_bar, 0));
+        else
+            mbar_arrive(bready_bar);
+    }
 }
 
-template <int STRIDE, int ACT>
+template <int STRIDE, int ACT, bool CG2 = false>
 __global__ void __launch_bounds__(PW_THREADS, 1)
     qconv_pw_kernel(const __grid_constant__ CUtensorMap tmap_x, const PwParams p) {
     using C = PwCfg;
@@ -136,6 +157,9 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
     const ConvShape& s = p.s;
     const uint64_t limit = p.wait_limit_ns;
     // this CTA's channel block and its pixel tiles t = t0, t0 + tstep, ...
+    // (CG2: the pair's blocks are neighbours, mb even in CTA 0, and share their tiles)
+    constexpr int STAGE = CG2 ? C::STAGE / 2 : C::STAGE;
+    const int rank = CG2 ? static_cast<int>(cluster_ctarank()) : 0;
     const int mb = blockIdx.x % p.mblocks;
     const int t0 = blockIdx.x / p.mblocks, tstep = gridDim.x / p.mblocks;
 
@@ -147,20 +171,27 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(accf0 + 8u * b, 1);
-            mbar_init(acce0 + 8u * b, PW_EPI_THREADS);
+            mbar_init(acce0 + 8u * b, (CG2 ? 2 : 1) * PW_EPI_THREADS);
         }
         mbar_init(drain_bar, 1);
-        mbar_init(bready_bar, PW_EXP_WARPS);
+        mbar_init(bready_bar, (CG2 ? 2 : 1) * PW_EXP_WARPS);
         *abort_flag = 0;
         fence_barrier_init();
     }
     if (warp == 0 && lane == 0) tma_prefetch_desc(&tmap_x);
     if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
-        tmem_relinquish();
+        if constexpr (CG2) {
+            tmem_alloc_cg2(smem_u32(tmem_slot), C::TMEM_COLS);
+            tmem_relinquish_cg2();
+        } else {
+            tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
+    // both CTAs' barriers exist before any cluster arrive or multicast commit reaches them
+    if constexpr (CG2) cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // The block weight is expanded before the dependency wait, overlapping the previous
@@ -184,11 +215,16 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
                         break;
                     }
                     const uint32_t fb = full_bar(st);
-                    mbar_arrive_expect_tx(fb, static_cast<uint32_t>(128 * p.tile_pix));
+                    // (CG2: the even CTA's barrier counts both halves)
+                    if (rank == 0)
+                        mbar_arrive_expect_tx(fb, static_cast<uint32_t>(128 * p.tile_pix));
                     filled |= 1u << st;
                     fill_parity = (fill_parity & ~(1u << st)) | (phase << st);
-                    const uint32_t dst = ring + static_cast<uint32_t>(st * C::STAGE);
-                    if constexpr (STRIDE == 1)
+                    const uint32_t dst = ring + static_cast<uint32_t>(st * STAGE);
+                    if constexpr (CG2)
+                        tma_load_2d_cg2(dst, &tmap_x, mapa_shared(fb, 0), 64 * kc,
+                                        t * PW_NPIX + rank * (PW_NPIX / 2), pol);
+                    else if constexpr (STRIDE == 1)
                         tma_load_2d(dst, &tmap_x, fb, 64 * kc, t * p.tile_pix, pol);
                     else
                         tma_load_5d(dst, &tmap_x, fb, 64 * kc, 0, 0, 0, t * p.rows_per_tile,
@@ -199,14 +235,23 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
                     }
                 }
             }
-            if (!ok || *abort_flag) drain_fills(full_bar(0), p.stages, filled, fill_parity, limit);
+            // (the odd CTA's copies complete on the even CTA's barrier, and it waits for that
+            // CTA at the end)
+            if ((!ok || *abort_flag) && rank == 0)
+                drain_fills(full_bar(0), p.stages, filled, fill_parity, limit);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t IDESC = make_idesc(BM, PW_NPIX, 0);
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t IDESC = make_idesc(CG2 ? 2 * BM : BM, PW_NPIX, 0);
             bool ok = wait_or_abort(bready_bar, 0, limit, abort_flag, STATUS_TIMEOUT_MMA);
             int issued = 0;
+            auto commit = [](uint32_t bar) {  // CG2: on both CTAs' barriers
+                if constexpr (CG2)
+                    umma_commit_cg2(bar, 3);
+                else
+                    umma_commit(bar);
+            };
             if (p.inject_stall) {
                 // Failure injection: wait on a barrier nothing arrives on.
                 wait_or_abort(drain_bar, 0, limit, abort_flag, STATUS_TIMEOUT_MMA);
@@ -233,25 +278,33 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t b_lo = desc_lo(ring + static_cast<uint32_t>(st * C::STAGE));
+                    const uint32_t b_lo = desc_lo(ring + static_cast<uint32_t>(st * STAGE));
                     const uint32_t a_lo = a_lo0 + static_cast<uint32_t>((kc * C::CHUNK) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)  // 16-channel steps: 32 bytes into the row
-                        umma_f16_w(d, a_lo + 2 * kk, C::DESC_HI, b_lo + 2 * kk, C::DESC_HI,
-                                   IDESC, (kc | kk) != 0 ? 1u : 0u);
+                    for (int kk = 0; kk < 4; ++kk) {  // 16-channel steps: 32 bytes into the row
+                        if constexpr (CG2)
+                            umma_f16_cg2(d, a_lo + 2 * kk, C::DESC_HI, b_lo + 2 * kk, C::DESC_HI,
+                                         IDESC, (kc | kk) != 0 ? 1u : 0u);
+                        else
+                            umma_f16_w(d, a_lo + 2 * kk, C::DESC_HI, b_lo + 2 * kk, C::DESC_HI,
+                                       IDESC, (kc | kk) != 0 ? 1u : 0u);
+                    }
                     ++issued;
-                    umma_commit(empty_bar(st));
+                    commit(empty_bar(st));
                     if (++st == p.stages) {
                         st = 0;
                         phase ^= 1u;
                     }
                 }
                 if (!ok) break;
-                umma_commit(accf0 + 8u * buf);
+                commit(accf0 + 8u * buf);
             }
             if (!ok && issued > 0) {
                 // let the issued MMAs finish before TMEM is released
-                umma_commit(drain_bar);
+                if constexpr (CG2)
+                    umma_commit_cg2(drain_bar, 1);
+                else
+                    umma_commit(drain_bar);
                 const uint64_t t1 = global_timer_ns();
                 while (!mbar_try_wait(drain_bar, 0u)) {
                     if (global_timer_ns() - t1 > limit) {
@@ -262,7 +315,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
             }
         }
     } else {
-        pw_expand(p, smem, mb, (warp - PW_EXP_WARP0) * 32 + lane, lane, bready_bar);
+        pw_expand<CG2>(p, smem, mb, (warp - PW_EXP_WARP0) * 32 + lane, lane, bready_bar);
         griddep_wait();  // the output buffer no longer read by the previous kernel
         if (warp >= PW_EPI_WARP0) {
             // -------------------------------------------------------- epilogue
@@ -292,7 +345,10 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
                 tmem_ld_wait();
                 // the accumulator is in registers: hand the buffer back to the issuer
                 tc_fence_before();
-                mbar_arrive_relaxed(acce0 + 8u * buf);
+                if constexpr (CG2)
+                    mbar_arrive_cluster_relaxed(mapa_shared(acce0 + 8u * buf, 0));
+                else
+                    mbar_arrive_relaxed(acce0 + 8u * buf);
                 const long long pix0 = static_cast<long long>(t) * p.tile_pix;
                 long long left = p.npix - pix0;
                 if (left > p.tile_pix) left = p.tile_pix;
@@ -329,9 +385,14 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
 
     tc_fence_before();
     __syncthreads();
+    // CG2: the pair's MMAs into both CTAs' TMEM and both epilogues are done
+    if constexpr (CG2) cluster_sync_all();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, C::TMEM_COLS);
+        if constexpr (CG2)
+            tmem_dealloc_cg2(tmem_base, C::TMEM_COLS);
+        else
+            tmem_dealloc(tmem_base, C::TMEM_COLS);
     }
 }

@@ -741,6 +741,27 @@ cudaError_t set_smem_once(K kern, int bytes, std::atomic<unsigned long long>& do
     return cudaSuccess;
 }
 
+// launch_pdl for clusters of two CTAs.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_pairs(void (*kern)(KArgs...), int pairs, int threads, int smem,
+                             cudaStream_t stream, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false>
 cudaError_t launch_cfg(const CUtensorMap maps[6], const TcParams& prm, int grid,
                        cudaStream_t stream, const ScMaps* scm = nullptr,
@@ -1141,6 +1162,16 @@ bool encode_x_pw(CUtensorMap* map, const ConvShape& s, const void* x, int rows) 
     return r == CUDA_SUCCESS;
 }
 
+template <int ACT>
+cudaError_t launch_pw_pairs(const CUtensorMap& map, const PwParams& prm, int grid,
+                            cudaStream_t stream) {
+    auto kern = qconv_pw_kernel<1, ACT, true>;
+    static std::atomic<unsigned long long> attr_done{0};
+    cudaError_t e = set_smem_once(kern, PwCfg::SMEM_BYTES, attr_done);
+    if (e != cudaSuccess) return e;
+    return launch_pdl_pairs(kern, grid / 2, PW_THREADS, PwCfg::SMEM_BYTES, stream, map, prm);
+}
+
 template <int STRIDE, int ACT>
 cudaError_t launch_pw_kernel(const CUtensorMap& map, const PwParams& prm, int grid,
                              cudaStream_t stream) {
@@ -1162,7 +1193,8 @@ cudaError_t launch_pw(const ConvShape& s, const void* x, const void* const w[4],
     prm.wait_limit_ns = opt.wait_limit_ns;
     prm.inject_stall = opt.inject_stall;
     prm.kchunks = s.Cin / 64;
-    prm.stages = PwCfg::max_stages(prm.kchunks);
+    const bool cg2 = pw_cg2_ok(s);
+    prm.stages = PwCfg::max_stages(prm.kchunks, cg2 ? PwCfg::STAGE / 2 : PwCfg::STAGE);
     prm.mblocks = s.Cout / 128;
     prm.npix = s.M;
     // (no box extends past the tensor: tiles shrink for inputs smaller than one tile)
@@ -1181,11 +1213,11 @@ cudaError_t launch_pw(const ConvShape& s, const void* x, const void* const w[4],
         snprintf(err, errlen, "pointwise kernel: Cin=%d does not fit", s.Cin);
         return cudaErrorInvalidValue;
     }
-    const MapKey key = make_key(s, x, w, out, 64, 32, 8);
+    const MapKey key = make_key(s, x, w, out, 64, 32, cg2 ? 23 : 8);
     CUtensorMap maps[6];
     if (!cache_lookup(key, maps)) {
         if (!encode_x_pw(&maps[0], s, x,
-                         s.stride == 1 ? prm.tile_pix : prm.rows_per_tile)) {
+                         cg2 ? PW_NPIX / 2 : s.stride == 1 ? prm.tile_pix : prm.rows_per_tile)) {
             snprintf(err, errlen, "tensor-map encode failed for the activation tensor");
             return cudaErrorInvalidValue;
         }
@@ -1200,6 +1232,11 @@ cudaError_t launch_pw(const ConvShape& s, const void* x, const void* const w[4],
     if (grid < prm.mblocks) grid = prm.mblocks;
     set_kernel_name(s.stride == 1 ? "qconv_pw_kernel<s1>" : "qconv_pw_kernel<s2>");
     const int act = s.act;
+    if (cg2) {
+        if (act == 1) return launch_pw_pairs<1>(maps[0], prm, grid, stream);
+        if (act == 2) return launch_pw_pairs<2>(maps[0], prm, grid, stream);
+        return launch_pw_pairs<0>(maps[0], prm, grid, stream);
+    }
     if (s.stride == 1) {
         if (act == 1) return launch_pw_kernel<1, 1>(maps[0], prm, grid, stream);
         if (act == 2) return launch_pw_kernel<1, 2>(maps[0], prm, grid, stream);
@@ -1334,21 +1371,7 @@ cudaError_t launch_cg2(const ConvShape& s, const void* x, const void* const w[4]
     static std::atomic<unsigned long long> attr_done[3];
     cudaError_t e = set_smem_once(kern, CgCfg::SMEM_BYTES, attr_done[stg]);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs);
-    cfg.blockDim = dim3(CG_THREADS);
-    cfg.dynamicSmemBytes = CgCfg::SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, maps[0], prm);
+    return launch_pdl_pairs(kern, pairs, CG_THREADS, CgCfg::SMEM_BYTES, stream, maps[0], prm);
 }
 
 template <int ROWS, int NSP, int ACT, bool RGB>

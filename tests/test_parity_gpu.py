@@ -586,6 +586,24 @@ def test_simt_small_layers(case):
     check(spec, expect_path=quan.QUAN_PATH_SIMT)
 
 
+PW_PAIR_CASES = [
+    # name, N, H, W, Cin, Cout, extra, max_ctas: 1x1 stride 1 on CTA pairs
+    ("pwp_one_tile", 1, 16, 16, 64, 256, {}, 0),
+    ("pwp_tail", 2, 17, 19, 128, 512, {"bias": True, "act": quan.QUAN_ACT_SILU}, 0),  # odd CTA's
+    ("pwp_tail_half", 1, 18, 19, 512, 256, {"iqbn": False}, 0),   # tail ends in the even half
+    ("pwp_wrap", 8, 24, 25, 192, 768, {"act": quan.QUAN_ACT_NONE}, 6),  # several tiles a pair
+]
+
+
+@pytest.mark.parametrize("case", PW_PAIR_CASES, ids=[c[0] for c in PW_PAIR_CASES])
+def test_pointwise_cta_pairs(case):
+    name, N, H, W, Cin, Cout, extra, max_ctas = case
+    quan.quan_set_tc_tiles(0, 0, max_ctas, 0)
+    check(inputs.small_layer(name, N, H, W, Cin, Cout, 1, 1, 0, seed=(306, len(name)), **extra),
+          path=quan.QUAN_PATH_TC)
+    assert quan.quan_last_kernel() == "qconv_pw_kernel<s1>"
+
+
 PAIR_TILE_CASES = [
     # name, N, H, W, Cin, Cout, k, stride, pad, extra, grid, bnq: channel tiles the pair mode
     # chooses, the last one reaching past the channels where it does not divide them
