@@ -250,12 +250,13 @@ size_t quan_qconv2d_bwd_data_workspace_size_ex(int N, int H, int W, int Cin, int
  * conj(W) with its channel axes swapped and the filter rotated by 180 degrees into the
  * workspace, then the forward tensor-core kernel convolves dy with it (stride 1, padding
  * kh - 1 - pad).  A strided forward needs the larger workspace of
- * quan_qconv2d_bwd_data_workspace_size_ex.  For stride 2 (and no tile overrides) the pixels of
- * dx are computed in four classes by the parity of their row and column, each a stride-1
+ * quan_qconv2d_bwd_data_workspace_size_ex.  For stride 2 (and no tile overrides) the pixels
+ * of dx are computed in four classes by the parity of their row and column, each a stride-1
  * convolution of dy with its share of the filter taps; for other strides dy is first spread
  * out with zeros between its pixels (stride - 1 of them), which multiplies the MMAs by
- * stride^2 but keeps them on the tensor cores.  Other shapes, or a strided forward with the smaller workspace, run a
- * direct CUDA-core kernel.
+ * stride^2 but keeps them on the tensor cores.  Other shapes, or a strided forward with the
+ * smaller workspace, run without them: bf16 products of narrow layers on warp-level MMAs,
+ * the rest on the CUDA cores.
  * quan_set_path(QUAN_PATH_TC) makes a shape the tensor-core path cannot run fail with
  * QUAN_ERR_UNSUPPORTED.
  */

@@ -10,7 +10,7 @@
 //   MODE_QUAD  16 MMAs per 16-wide K step, one per (output q, input p):
 //                D_q += sign(q, p) * X_p * W_{q xor p}^T            (N = BNQ)
 //              the letter is chosen by the B descriptor and the sign by the
-//              instruction descriptor's negate bit.
+//              instruction descriptor's negate bit.  Runs on request only (tile mode 1).
 //   MODE_PAIR  8 MMAs per K step, each covering two output components:
 //                [D_r | D_i] and [D_j | D_k] += +-X_p * S^T         (N = 2 BNQ)
 //              where S is a stack of two letter blocks.  The four stacks Eq. 6 needs,
@@ -20,7 +20,8 @@
 //              so a stage holds 6 letter blocks; TMA loads the 4 letters and a helper
 //              warp writes the two negated copies.  The larger N keeps the tensor pipe
 //              busy (an M=128 MMA costs at least ~45 cycles on this part, a full N=64 one
-//              is 32 cycles of work, N=128 is 64).
+//              is 32 cycles of work, N=128 is 64).  Also the stride-2 input gradient, the
+//              parity classes of its pixels as tiles of one launch.
 //   MODE_SEP   the separable form of Eq. 7: 4 MMAs per K step, D_p += X_p * W_p^T
 //              (N = BNQ), one per input component; the epilogue mixes the four D_p
 //              with the signs of Eq. 7 (epilogue_direct_sep), so no negated letters.
