@@ -96,7 +96,25 @@ struct TcParams {
     int inject_stall;
     SplitK sk;        // K ranges split evenly over the CTAs (QUAD/PAIR modes, caller workspace)
     ScParams sc;      // the fused 1x1 shortcut (the SC form of the kernel)
+    int Wp;           // WALK form: positions per image row, W + pad
+    long long Mp;     //            N * Ho * Wp
 };
+
+// WALK form (pair mode, 16-channel K blocks, stride 1, filters wider than one column).  The input pixels of a tap
+// row are walked in rows of Wp = W + pad positions, the pad zero columns before each image row
+// also serving as the ones after the row above it.  The pixel at position m then reads
+// position m + dw for tap dw, so one box of 128 + kw - 1 positions serves all taps of a tap
+// row as row offsets of the A descriptor (the swizzle applies to absolute addresses, so any
+// row may start an operand).  Positions that are no output pixel (Wp - Wo per row) are
+// computed and not stored.  A box per tap instead copies a tap row's pixels kw times, and with
+// 32-byte rows the copies, at 1.6-1.9 clocks per row, take longer than the MMAs: 80 us, now
+// 67 us, for 320 -> 320 channels, 16 images of 40 x 40, 3x3; 32 and 25.5 us for 64 -> 256, 64 of
+// 28 x 28; 36 and 35 us for 448 -> 320, 32 of 14 x 14 (7% of its positions are padding).  K
+// blocks of 32 channels wait for the MMAs themselves: there the walk's padding and second
+// ring cost 2-8% (159 against 155 us for 256 -> 256, 64 of 56 x 56).
+// The pixel boxes and the letters have a ring each.
+constexpr int WALK_ROWS = 136;  // box rows: a multiple of 8 (whole swizzle patterns)
+constexpr int WALK_MAX_KW = WALK_ROWS - BM + 1;
 
 // The fused shortcut's four letter maps (SC form; unused otherwise).
 struct ScMaps {
@@ -136,6 +154,28 @@ __device__ __forceinline__ int par_class(const ParArgs& a, int tile) {
     return c;
 }
 
+struct WalkGeo {
+    static constexpr bool kScattered = true;
+    long long Mp;
+    int Wp, Wo, num_n;
+    __device__ __forceinline__ EpiTile operator()(int tile) const {
+        EpiTile g;
+        const int m_tile = tile / num_n;
+        g.n_tile = tile - m_tile * num_n;
+        g.m0 = static_cast<long long>(m_tile) * BM;
+        const long long left = Mp - g.m0;
+        g.rows = left < BM ? static_cast<int>(left) : BM;
+        return g;
+    }
+    __device__ __forceinline__ long long pixel(const EpiTile& g, int, int row) const {
+        if (row >= g.rows) return -1;
+        const int m = static_cast<int>(g.m0) + row;  // fewer than 2^31 positions
+        const int r = m / Wp, c = m - r * Wp;
+        return c < Wo ? static_cast<long long>(r) * Wo + c : -1;
+    }
+    __device__ __forceinline__ bool empty(int) const { return false; }
+};
+
 struct ParGeo {
     static constexpr bool kScattered = true;
     const ParArgs& a;
@@ -151,7 +191,7 @@ struct ParGeo {
         return g;
     }
     __device__ __forceinline__ long long pixel(const EpiTile& g, int tile, int row) const {
-        if (row >= g.rows) return 0;
+        if (row >= g.rows) return -1;
         const PixClass& c = a.cls[par_class(a, tile)];
         const int m = static_cast<int>(g.m0) + row;  // fewer than 2^31 pixels
         const int r = m / c.Wc, j = m - r * c.Wc;
@@ -163,26 +203,31 @@ struct ParGeo {
     }
 };
 
-template <int KAPPA, int BNQ, int MODE>
+template <int KAPPA, int BNQ, int MODE, bool WALK = false>
 struct Cfg {
     static constexpr int A_ROW_BYTES = KAPPA * 2;
-    static constexpr int A_TILE = BM * A_ROW_BYTES;  // one component of the pixel tile
+    // one component of the pixel tile
+    static constexpr int A_TILE = (WALK ? WALK_ROWS : BM) * A_ROW_BYTES;
     static constexpr int B_TILE = BNQ * KAPPA * 2;   // one letter block of the weight tile
     static constexpr int B_SLOTS = MODE == MODE_PAIR ? 6 : 4;
-    static constexpr int STAGE_BYTES = 4 * A_TILE + B_SLOTS * B_TILE;
+    // WALK: the letters' ring (STAGE_BYTES, STAGES) after the pixel boxes' (XSTAGES)
+    static constexpr int XSTAGES = WALK ? 5 : 0;
+    static constexpr int X_BYTES = XSTAGES * 4 * A_TILE;
+    static constexpr int STAGE_BYTES = (WALK ? 0 : 4 * A_TILE) + B_SLOTS * B_TILE;
     static constexpr int TX_A = 4 * A_TILE;          // bytes TMA writes per stage: pixels
     static constexpr int TX_W = 4 * B_TILE;          //                               letters
     // 1024 bytes of alignment slack, then the stage ring and the barrier area (the
     // epilogue needs no shared memory)
     static constexpr int FIXED_BYTES = 1024 + 384;
-    static constexpr int STAGES_RAW = (227 * 1024 - FIXED_BYTES) / STAGE_BYTES;
+    static constexpr int STAGES_RAW = (227 * 1024 - FIXED_BYTES - X_BYTES) / STAGE_BYTES;
     static constexpr int STAGES =
         STAGES_RAW > MAX_STAGES ? MAX_STAGES : (STAGES_RAW < 2 ? 2 : STAGES_RAW);
-    static constexpr int TILES_BYTES = STAGES * STAGE_BYTES;
+    static constexpr int TILES_BYTES = X_BYTES + STAGES * STAGE_BYTES;
     static constexpr int BAR_OFF = TILES_BYTES;
-    // full (pixels), empty, full (letters), acc_full[2], acc_empty[2], drain; then the
-    // TMEM address, the abort flag and one ready sequence word per stage
-    static constexpr int NUM_BARS = 3 * STAGES + 5;
+    // full (pixels), empty, full (letters), acc_full[2], acc_empty[2], drain (WALK: full and
+    // empty of the pixel boxes); then the TMEM address, the abort flag and one ready sequence
+    // word per stage
+    static constexpr int NUM_BARS = 3 * STAGES + 5 + 2 * XSTAGES;
     static constexpr int SMEM_BYTES = 1024 + BAR_OFF + NUM_BARS * 8 + 16 + 4 * STAGES;
     static_assert(NUM_BARS * 8 + 16 + 4 * STAGES <= FIXED_BYTES - 1024, "barrier area");
     static constexpr bool FITS = SMEM_BYTES <= 227 * 1024;
@@ -192,7 +237,12 @@ struct Cfg {
     static constexpr uint32_t DESC_HI = desc_hi(8 * A_ROW_BYTES, desc_layout(A_ROW_BYTES));
     static_assert(KAPPA == 16 || KAPPA == 32 || KAPPA == 64, "KAPPA");
     static_assert(BNQ == 16 || BNQ == 32 || BNQ == 64 || (BNQ == 48 && MODE == MODE_PAIR), "BNQ");
-    static_assert(STAGE_BYTES % 1024 == 0, "stages start on swizzle patterns");
+    // (a pattern is 8 rows: 1024, 512 or 256 bytes)
+    static_assert(STAGE_BYTES % (8 * A_ROW_BYTES) == 0 && A_TILE % (8 * A_ROW_BYTES) == 0 &&
+                      X_BYTES % 1024 == 0,
+                  "stages start on swizzle patterns");
+    static_assert(TILES_BYTES % 16 == 0 && (!WALK || (MODE == MODE_PAIR && KAPPA == 16)),
+                  "WALK");
 };
 
 // SC: N tiles from p.sc.n_conv on belong to a 1x1 shortcut on the same input, fused into
@@ -200,7 +250,8 @@ struct Cfg {
 // come from `scm`, and the epilogue writes them to the shortcut's output.
 // PAR: the pixel classes of `par` (tmap_x unused).  PAD: the last channel tile may reach past
 // Qout (an instance of its own: the epilogue's checks cost the epilogue-bound layers 15%).
-template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false>
+template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false,
+          bool WALK = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     qconv_tc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                     const __grid_constant__ CUtensorMap tmap_wr,
@@ -210,7 +261,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     const __grid_constant__ ScMaps scm, const __grid_constant__ ParOf<PAR> par) {
     static_assert(!PAR || (!SC && (MODE == MODE_PAIR || MODE == MODE_SEPT)), "class modes");
     static_assert(!SC || MODE == MODE_PAIR || MODE == MODE_QUAD, "fused shortcut modes");
-    using C = Cfg<KAPPA, BNQ, MODE>;
+    static_assert(!WALK || (!SC && !PAR), "walk forms");
+    using C = Cfg<KAPPA, BNQ, MODE, WALK>;
     constexpr int STAGES = C::STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -228,6 +280,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const uint32_t accf0 = bar0 + 8u * (3 * STAGES);
     const uint32_t acce0 = bar0 + 8u * (3 * STAGES + 2);
     const uint32_t drain_bar = bar0 + 8u * (3 * STAGES + 4);
+    // WALK: the pixel boxes' barriers
+    auto xfull_bar = [&](int x) { return bar0 + 8u * (3 * STAGES + 5 + x); };
+    auto xempty_bar = [&](int x) { return bar0 + 8u * (3 * STAGES + 5 + C::XSTAGES + x); };
+    // a stage's letters
+    auto letters = [&](int st) {
+        return C::X_BYTES + st * C::STAGE_BYTES + (WALK ? 0 : 4 * C::A_TILE);
+    };
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const ConvShape& s = p.s;
@@ -240,6 +299,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             mbar_init(fullw_bar(i), 1);
             mbar_init(empty_bar(i), 1);
             ready_seq[i] = 0;
+        }
+        for (int i = 0; i < C::XSTAGES; ++i) {
+            mbar_init(xfull_bar(i), 1);
+            mbar_init(xempty_bar(i), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(accf0 + 8u * b, 1);
@@ -272,7 +335,78 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int hw = s.Ho * s.Wo;
     griddep_wait();  // the previous kernel's output (this layer's input) is complete
 
-    if (warp == 0 || warp == 3) {
+    if (WALK && (warp == 0 || warp == 3)) {
+        // ------------------------------------------------------------ TMA producers, WALK
+        // K block kt = (dh, chunk, dw), dw fastest; a unit starts with a box of its own
+        if (lane == 0) {
+            const bool pixels = warp == 0;
+            const uint64_t pol = pixels ? l2_policy_evict_normal() : l2_policy_evict_last();
+            const uint32_t x_tx = 4u * static_cast<uint32_t>((BM + s.kw - 1) * C::A_ROW_BYTES);
+            const int ring = pixels ? C::XSTAGES : STAGES;
+            int stage = 0;
+            uint32_t phase = 0;
+            uint32_t filled = 0, fill_parity = 0;
+            bool ok = true;
+            UnitIter units(p.sk.on, p.num_tiles, p.ktiles);
+            Unit unit;
+            while (ok && units.next(unit)) {
+                const int m_tile = unit.tile / p.num_n_tiles;
+                const int wrow = (unit.tile - m_tile * p.num_n_tiles) * BNQ;
+                const int m0 = m_tile * BM;  // (fewer than 2^31 positions)
+                const int r = m0 / p.Wp, img = r / s.Ho;
+                const int wbase = m0 - r * p.Wp - s.pad, hbase = r - img * s.Ho - s.pad;
+                int t = unit.k0 / s.kw;
+                int dw = unit.k0 - t * s.kw;
+                int dh = t / p.kchunks;
+                int chunk = t - dh * p.kchunks;
+                for (int kt = unit.k0; kt < unit.k1; ++kt) {
+                    if (!pixels || dw == 0 || kt == unit.k0) {
+                        const uint32_t fb = pixels ? xfull_bar(stage) : fullw_bar(stage);
+                        if (!wait_or_abort(pixels ? xempty_bar(stage) : empty_bar(stage),
+                                           phase ^ 1u, limit, abort_flag,
+                                           STATUS_TIMEOUT_PRODUCER)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_arrive_expect_tx(fb, pixels ? x_tx : C::TX_W);
+                        filled |= 1u << stage;
+                        fill_parity = (fill_parity & ~(1u << stage)) | (phase << stage);
+                        const int cin0 = chunk * KAPPA;
+                        if (pixels) {
+                            const uint32_t a0 = sbase + stage * (4 * C::A_TILE);
+#pragma unroll
+                            for (int comp = 0; comp < 4; ++comp)
+                                tma_load_im2col_4d(a0 + comp * C::A_TILE, &tmap_x, fb,
+                                                   comp * s.Qin + cin0, wbase, hbase, img,
+                                                   static_cast<uint16_t>(0),
+                                                   static_cast<uint16_t>(dh), pol);
+                        } else {
+                            const int wcol = (dh * s.kw + dw) * s.Qin + cin0;
+                            const uint32_t b0 = sbase + letters(stage);
+                            tma_load_2d(b0 + 1 * C::B_TILE, &tmap_wr, fb, wcol, wrow, pol);
+                            tma_load_2d(b0 + 2 * C::B_TILE, &tmap_wi, fb, wcol, wrow, pol);
+                            tma_load_2d(b0 + 3 * C::B_TILE, &tmap_wj, fb, wcol, wrow, pol);
+                            tma_load_2d(b0 + 4 * C::B_TILE, &tmap_wk, fb, wcol, wrow, pol);
+                        }
+                        if (++stage == ring) {
+                            stage = 0;
+                            phase ^= 1u;
+                        }
+                    }
+                    if (++dw == s.kw) {
+                        dw = 0;
+                        if (++chunk == p.kchunks) {
+                            chunk = 0;
+                            ++dh;
+                        }
+                    }
+                }
+            }
+            if (!ok || *abort_flag)
+                drain_fills(pixels ? xfull_bar(0) : fullw_bar(0), ring, filled, fill_parity,
+                            limit);
+        }
+    } else if (warp == 0 || warp == 3) {
         // ------------------------------------------------------------ TMA producers
         if (lane == 0) {
             const int role = warp == 0 ? 0 : 1;  // 0: pixels, 1: letters
@@ -416,6 +550,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             constexpr uint32_t IDESC_NEG = make_idesc(BM, NMMA, 1);
             int stage = 0;
             uint32_t round = 0;  // completed passes over the stage ring
+            [[maybe_unused]] int xs = 0, dw = 0;  // WALK: pixel box, tap column
             bool ok = true;
             int issued = 0;
             if (p.inject_stall) {
@@ -442,6 +577,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 if constexpr (SC)
                     if (unit.tile % p.num_n_tiles >= p.sc.n_conv) k1 = p.sc.ktiles;
                 if constexpr (PAR) k1 = par.cls[par_class(par, unit.tile)].ktiles;
+                if constexpr (WALK) dw = unit.k0 % s.kw;
                 for (int kt = unit.k0; kt < k1; ++kt) {
                     // pixels and letter tiles landed (pair mode: with the negated copies)
                     if (!flag_wait_or_abort(ready_word(stage), round + 1u, limit, abort_flag,
@@ -452,8 +588,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     tc_fence_after();
                     // descriptor low words of this stage's first X_p and W_L tiles; every
                     // sub-MMA below only adds a compile-time offset to them
-                    const uint32_t a_lo0 = desc_lo(sbase + stage * C::STAGE_BYTES);
-                    const uint32_t b_lo0 = a_lo0 + (4 * C::A_TILE >> 4);
+                    const uint32_t a_lo0 =
+                        desc_lo(sbase + (WALK ? xs * (4 * C::A_TILE) + dw * C::A_ROW_BYTES
+                                              : stage * C::STAGE_BYTES));
+                    const uint32_t b_lo0 = desc_lo(sbase + letters(stage));
                     const uint32_t first = kt != unit.k0 ? 1u : 0u;
 #pragma unroll
                     for (int pc = 0; pc < 4; ++pc) {
@@ -499,6 +637,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
                     ++issued;
                     umma_commit(empty_bar(stage));  // frees the stage when these MMAs finish
+                    if constexpr (WALK) {
+                        if (++dw == s.kw || kt + 1 == k1) {  // the box's last tap
+                            dw = 0;
+                            umma_commit(xempty_bar(xs));
+                            if (++xs == C::XSTAGES) xs = 0;
+                        }
+                    }
                     if (++stage == STAGES) {
                         stage = 0;
                         ++round;
@@ -530,11 +675,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         constexpr int WORDS = C::B_TILE / 16;  // uint4 per slot
         int stage = 0;
         uint32_t phase = 0, round = 0;
+        [[maybe_unused]] int xs = 0, dw = 0;
+        [[maybe_unused]] uint32_t xphase = 0;
         bool ok = true;
         UnitIter units(p.sk.on, p.num_tiles, p.ktiles);
         Unit unit;
         while (ok && units.next(unit)) {
             int k1 = unit.k1;
+            if constexpr (WALK) dw = unit.k0 % s.kw;
             if constexpr (SC)
                 if (unit.tile % p.num_n_tiles >= p.sc.n_conv) k1 = p.sc.ktiles;
             if constexpr (PAR) k1 = par.cls[par_class(par, unit.tile)].ktiles;
@@ -545,7 +693,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     break;
                 }
                 if constexpr (MODE == MODE_PAIR) {
-                    uint8_t* b0 = smem + stage * C::STAGE_BYTES + 4 * C::A_TILE;
+                    uint8_t* b0 = smem + letters(stage);
                     const uint4* s2 = reinterpret_cast<const uint4*>(b0 + 2 * C::B_TILE);
                     const uint4* s3 = reinterpret_cast<const uint4*>(b0 + 3 * C::B_TILE);
                     uint4* s0 = reinterpret_cast<uint4*>(b0);
@@ -558,8 +706,23 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     // make the generic-proxy writes visible to the tensor core (async proxy)
                     fence_proxy_async_smem();
                 }
-                if (!wait_or_abort(full_bar(stage), phase, limit, abort_flag,
-                                   STATUS_TIMEOUT_PRODUCER)) {
+                if constexpr (WALK) {
+                    // (a box is waited for with its first tap)
+                    if ((dw == 0 || kt == unit.k0) &&
+                        !wait_or_abort(xfull_bar(xs), xphase, limit, abort_flag,
+                                       STATUS_TIMEOUT_PRODUCER)) {
+                        ok = false;
+                        break;
+                    }
+                    if (++dw == s.kw || kt + 1 == k1) {
+                        dw = 0;
+                        if (++xs == C::XSTAGES) {
+                            xs = 0;
+                            xphase ^= 1u;
+                        }
+                    }
+                } else if (!wait_or_abort(full_bar(stage), phase, limit, abort_flag,
+                                          STATUS_TIMEOUT_PRODUCER)) {
                     ok = false;
                     break;
                 }
@@ -595,6 +758,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             epilogue_direct_pair<BNQ, PAD>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
                                            p.ktiles, p.sk, limit, abort_flag,
                                            ParGeo{par, p.num_n_tiles});
+        else if constexpr (WALK)
+            epilogue_direct_pair<BNQ, PAD>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
+                                           p.ktiles, p.sk, limit, abort_flag,
+                                           WalkGeo{p.Mp, p.Wp, s.Wo, p.num_n_tiles});
         else
             epilogue_direct_pair<BNQ, PAD>(s, p.ep, p.y, tmem_base, accf0, acce0, p.num_tiles,
                                            p.ktiles, p.sk, limit, abort_flag, linear_geo(geo));
@@ -645,10 +812,10 @@ CUtensorMapSwizzle swizzle_for_row(int row_bytes) {
                                                : CU_TENSOR_MAP_SWIZZLE_32B);
 }
 
-// im2col map over x: boxes of BM pixels x `channels` channels, walking the filter origins
+// im2col map over x: boxes of `pixels` pixels x `channels` channels, walking the filter origins
 // from (lower) to (dim - 1 + upper) of each spatial dimension, innermost (W) first.
 bool encode_im2col(CUtensorMap* map, const ConvShape& s, const void* x, int channels,
-                   const int lower[2], const int upper[2]) {
+                   const int lower[2], const int upper[2], int pixels = BM) {
     const cuuint64_t dims[4] = {static_cast<cuuint64_t>(s.Cin), static_cast<cuuint64_t>(s.W),
                                 static_cast<cuuint64_t>(s.H), static_cast<cuuint64_t>(s.N)};
     const cuuint64_t strides[3] = {static_cast<cuuint64_t>(s.Cin) * 2,
@@ -658,9 +825,9 @@ bool encode_im2col(CUtensorMap* map, const ConvShape& s, const void* x, int chan
                                 static_cast<cuuint32_t>(s.stride), 1};
     const CUresult r = g_encode_im2col(
         map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, lower,
-        upper, static_cast<cuuint32_t>(channels), BM, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-        swizzle_for_row(channels * 2), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        upper, static_cast<cuuint32_t>(channels), static_cast<cuuint32_t>(pixels), estr,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for_row(channels * 2),
+        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 
@@ -763,15 +930,16 @@ cudaError_t launch_pdl_pairs(void (*kern)(KArgs...), int pairs, int threads, int
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false>
+template <int KAPPA, int BNQ, int MODE, bool SC = false, bool PAR = false, bool PAD = false,
+          bool WALK = false>
 cudaError_t launch_cfg(const CUtensorMap maps[6], const TcParams& prm, int grid,
                        cudaStream_t stream, const ScMaps* scm = nullptr,
                        const ParOf<PAR>& par = {}) {
-    using C = Cfg<KAPPA, BNQ, MODE>;
+    using C = Cfg<KAPPA, BNQ, MODE, WALK>;
     if constexpr (!C::FITS || (SC && MODE != MODE_PAIR && MODE != MODE_QUAD)) {
         return cudaErrorInvalidValue;
     } else {
-        auto kern = qconv_tc_kernel<KAPPA, BNQ, MODE, SC, PAR, PAD>;
+        auto kern = qconv_tc_kernel<KAPPA, BNQ, MODE, SC, PAR, PAD, WALK>;
         static std::atomic<unsigned long long> attr_done{0};
         cudaError_t e = set_smem_once(kern, C::SMEM_BYTES, attr_done);
         if (e != cudaSuccess) return e;
@@ -869,22 +1037,32 @@ int grid_for(const TcOptions& opt, int num_sms, int num_tiles) {
 // tiles of 48 and not five of 16, which copy the pixels five times (145 us against 80 us for
 // 320 -> 320 channels, 16 images of 40 x 40, 3x3).  split: K ranges split evenly between one
 // and two waves.
-int pair_pick_bnq(int Qout, long long m_tiles, int grid, bool split) {
+// x_rows: pixel rows copied per K block.  narrowest: the smallest tile.  *cost: the estimate.
+int pair_pick_bnq(int Qout, long long m_tiles, int grid, bool split, int x_rows = 4 * BM,
+                  int narrowest = 16, double* cost = nullptr) {
     int best = 64;
     double best_t = 1e30;
-    for (int b = 64; b >= 16; b -= 16) {
+    for (int b = 64; b >= narrowest; b -= 16) {
         if (Qout % b != 0 && (Qout % 64 == 0 || b < 48)) continue;
         const long long tiles = m_tiles * ((Qout + b - 1) / b);
         double waves = static_cast<double>((tiles + grid - 1) / grid);
         if (split && tiles > grid && tiles < 2LL * grid)
             waves = static_cast<double>(tiles) / grid;
-        const double t = waves * (512 + 4 * b);
+        const double t = waves * (x_rows + 4 * b);
         if (t < best_t) {
             best_t = t;
             best = b;
         }
     }
+    if (cost != nullptr) *cost = best_t;
     return best;
+}
+
+// WALK form: filters of 2 to WALK_MAX_KW columns whose padding is less than their width, the
+// walk's corner offsets within the im2col encoding (those of tc_supported).
+bool walk_ok(const ConvShape& s) {
+    return s.stride == 1 && s.kw > 1 && s.kw <= WALK_MAX_KW && s.pad < s.kw && s.pad < s.kh &&
+           static_cast<long long>(s.N) * s.Ho * (s.W + s.pad) < 0x7fffffffLL - BM;
 }
 
 template <bool HALO, int KH, int NI, bool SEP>
@@ -1733,10 +1911,28 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
                  opt.kappa, opt.bnq, s.Qin, s.Qout);
         return cudaErrorInvalidValue;
     }
-    const long long m_tiles = (s.M + BM - 1) / BM;
-    if (mode == MODE_PAIR && opt.mode == 0 && opt.bnq == 0 && opt.kappa == 0)
-        bnq = pair_pick_bnq(s.Qout, m_tiles, opt.max_ctas > 0 ? opt.max_ctas : num_sms,
-                            opt.sk_ws != nullptr);
+    long long m_tiles = (s.M + BM - 1) / BM;
+    bool walk = false;
+    if (mode == MODE_PAIR && opt.mode == 0 && opt.bnq == 0 && opt.kappa == 0) {
+        const int ctas = opt.max_ctas > 0 ? opt.max_ctas : num_sms;
+        const bool split = opt.sk_ws != nullptr;
+        double cost = 0, walk_cost = 0;
+        bnq = pair_pick_bnq(s.Qout, m_tiles, ctas, split, 4 * BM, 16, &cost);
+        // The walk where it copies fewer rows, its padding included, in channel tiles of 48 or
+        // 64 (in tiles of 16 its 8 short MMAs per K block set the pace: 57 against 53 us for
+        // 320 -> 192 channels, 8 images of 20 x 20, 5x5).
+        if (kappa == 16 && s.Qout >= 48 && walk_ok(s)) {
+            const long long Mp = static_cast<long long>(s.N) * s.Ho * (s.W + s.pad);
+            const long long wm_tiles = (Mp + BM - 1) / BM;
+            const int wbnq = pair_pick_bnq(s.Qout, wm_tiles, ctas, split,
+                                           4 * (BM + s.kw - 1) / s.kw, 48, &walk_cost);
+            if (walk_cost < cost) {
+                walk = true;
+                m_tiles = wm_tiles;
+                bnq = wbnq;
+            }
+        }
+    }
     // Only two 6-slot stages of 64 x 64 letter blocks plus 64-channel pixel tiles fit in
     // shared memory; 32-channel K blocks give four.
     if (mode == MODE_PAIR && kappa == 64 && bnq == 64 && opt.kappa == 0) kappa = 32;
@@ -1758,10 +1954,13 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
             return cudaErrorInvalidValue;
         }
     }
-    const MapKey key = make_key(s, x, w, out, kappa, bnq, 0);
+    const MapKey key = make_key(s, x, w, out, kappa, bnq, walk ? 24 : 0);
     CUtensorMap maps[6];
     if (!cache_lookup(key, maps)) {
-        if (!encode_x_im2col(&maps[0], s, x, kappa)) {
+        const int lower[2] = {-s.pad, -s.pad};
+        const int upper[2] = {0, s.pad - (s.kh - 1)};
+        if (walk ? !encode_im2col(&maps[0], s, x, kappa, lower, upper, BM + s.kw - 1)
+                 : !encode_x_im2col(&maps[0], s, x, kappa)) {
             snprintf(err, errlen, "cuTensorMapEncodeIm2col failed for the activation tensor");
             return cudaErrorInvalidValue;
         }
@@ -1780,6 +1979,8 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     prm.ktiles = s.kh * s.kw * prm.kchunks;
     prm.num_n_tiles = (s.Qout + bnq - 1) / bnq;
     prm.y = out;
+    prm.Wp = s.W + s.pad;
+    prm.Mp = static_cast<long long>(s.N) * s.Ho * prm.Wp;
     const long long tiles = m_tiles * prm.num_n_tiles;
     if (tiles > 0x7fffffffLL) {
         snprintf(err, errlen, "too many tiles");
@@ -1809,7 +2010,8 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
         prm.sk.flags = reinterpret_cast<unsigned*>(static_cast<char*>(opt.sk_ws) +
                                                    static_cast<size_t>(grid) * slot_bytes);
     }
-    set_kernel_name(mode == MODE_PAIR   ? "qconv_tc_kernel<pair,kappa=%d,bnq=%d>"
+    set_kernel_name(walk                ? "qconv_tc_kernel<pair,walk,kappa=%d,bnq=%d>"
+                    : mode == MODE_PAIR ? "qconv_tc_kernel<pair,kappa=%d,bnq=%d>"
                     : mode == MODE_SEP  ? "qconv_tc_kernel<sep,kappa=%d,bnq=%d>"
                     : mode == MODE_SEPT ? "qconv_tc_kernel<sep_t,kappa=%d,bnq=%d>"
                                         : "qconv_tc_kernel<quad,kappa=%d,bnq=%d>",
@@ -1822,6 +2024,13 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
         }
     }
 
+#define QUAN_WALK_CASE(B, PAD)                                                          \
+    if (walk && bnq == B && ((B == 48 || s.Qout % B != 0) == PAD))                      \
+        return launch_cfg<16, B, MODE_PAIR, false, false, PAD, true>(maps, prm, grid, stream);
+    QUAN_WALK_CASE(48, true)
+    QUAN_WALK_CASE(64, false)
+    QUAN_WALK_CASE(64, true)
+#undef QUAN_WALK_CASE
 #define QUAN_PAD_CASE(K, B)                                     \
     if (kappa == K && bnq == B && (B == 48 || s.Qout % B != 0)) \
         return launch_cfg<K, B, MODE_PAIR, false, false, true>(maps, prm, grid, stream);

@@ -177,7 +177,7 @@ struct EpiTile {
 };
 
 // Tile geometry functors of the QUAD/PAIR kernel's epilogue: tile index -> EpiTile, the output
-// pixel of a tile's row (kScattered; else consecutive pixels from m0), and whether a tile has
+// pixel of a tile's row (kScattered, negative for none; else consecutive from m0), and whether a tile has
 // no K blocks (its accumulator is never written and the output is zero).
 template <typename TileOf>
 struct LinearGeo {  // tiles of consecutive output pixels
@@ -484,6 +484,10 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
             if constexpr (Geo::kScattered) return pixels[k];
             return g.m0 + row0 + k;
         };
+        auto row_ok = [&](int k) {
+            if constexpr (Geo::kScattered) return pixels[k] >= 0;
+            return row0 + k < g.rows;
+        };
         const int c_tile = g.n_tile * BNQ + 8 * ci;  // + q Qout + slice offset: lane's channel
         // block b's first channel in this lane's chunk (past Qout: channel 0's vectors stand in)
         auto chan_ok = [&](int b) { return !PAD || c_tile + (b % SLICES) * CH < s.Qout; };
@@ -547,7 +551,7 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
 #pragma unroll
                 for (int k = 0; k < NCH; ++k) {
                     r4[k] = make_uint4(0u, 0u, 0u, 0u);
-                    if (store && row0 + k < g.rows)
+                    if (store && row_ok(k))
                         r4[k] = ld_global_na(res + pix(k) * Cout + cb);
                 }
             }
@@ -586,7 +590,7 @@ __device__ __forceinline__ void epilogue_direct_pair(const ConvShape& s, const E
                         fmaf(sc[2 * t + 1], E[k][2 * t + 1], sh[2 * t + 1]) + rz[2 * t + 1];
                     w[t] = pack_bf16x2(activate(z0, s.act), activate(z1, s.act));
                 }
-                if (store && row0 + k < g.rows)
+                if (store && row_ok(k))
                     st_global_na(out + pix(k) * Cout + cb,
                                  make_uint4(w[0], w[1], w[2], w[3]));
             }

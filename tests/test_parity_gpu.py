@@ -625,6 +625,32 @@ def test_pair_channel_tiles(case):
     assert quan.quan_last_kernel().endswith("bnq=%d>" % bnq), quan.quan_last_kernel()
 
 
+WALK_CASES = [
+    # name, N, H, W, Cin, Cout, k, pad, extra, walk: layers of 16-channel K blocks with one
+    # pixel box per tap row; paddings, images of one column or row, boxes across images, the
+    # widest filter and one past it (split K ranges: sk_5x5 above)
+    ("wk_3x3", 3, 13, 11, 64, 256, 3, 1, {"residual": True, "bias": True}, True),
+    ("wk_pad0", 2, 12, 10, 192, 256, 3, 0, {}, True),
+    ("wk_pad2", 2, 9, 8, 64, 320, 3, 2, {"act": quan.QUAN_ACT_SILU}, True),
+    ("wk_2x2", 3, 15, 14, 64, 192, 2, 0, {}, True),
+    ("wk_2x2_pad", 2, 15, 14, 64, 448, 2, 1, {}, True),
+    ("wk_9x9", 2, 14, 12, 64, 256, 9, 4, {}, True),
+    ("wk_11x11", 1, 14, 12, 64, 256, 11, 5, {}, False),
+    ("wk_row", 5, 1, 140, 64, 256, 3, 1, {}, True),
+    ("wk_col", 3, 140, 1, 64, 256, 3, 1, {}, True),
+]
+
+
+@pytest.mark.parametrize("case", WALK_CASES, ids=[c[0] for c in WALK_CASES])
+def test_pair_walk(case):
+    name, N, H, W, Cin, Cout, k, p, extra, walk = case
+    quan.quan_set_tc_tiles(0, 0, 3, 0)
+    check(inputs.small_layer(name, N, H, W, Cin, Cout, k, 1, p, seed=(306, len(name)), **extra),
+          path=quan.QUAN_PATH_TC)
+    assert quan.quan_last_kernel().startswith(
+        "qconv_tc_kernel<pair,walk," if walk else "qconv_tc_kernel<pair,kappa")
+
+
 NARROW_CASES = [
     # name, N, H, W, Cin, Cout, k, stride, pad, extra: bf16 layers off the tcgen05 channel
     # grid on warp-level MMAs: K tails, channel tiles past 64, one pixel buffer, few pixels
