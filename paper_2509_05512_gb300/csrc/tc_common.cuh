@@ -92,10 +92,14 @@ __host__ __device__ constexpr uint32_t make_idesc(int M, int N, int negate) {
 __device__ __forceinline__ float activate(float z, int act) {
     if (act == 1) return fmaxf(z, 0.0f);
     if (act == 2) {
-        // SiLU z / (1 + e^-z) with the fast exponential and division (a few ulp of fp32,
-        // far below the bf16 output's rounding); z >= -80 keeps the divisor below 2^126,
-        // where the fast division is exact enough (below that the value is ~0 anyway)
-        return __fdividef(z, 1.0f + __expf(-fmaxf(z, -80.0f)));
+        // SiLU z / (1 + e^-z), e^-z = 2^(-z log2 e), with the hardware's approximate 2^x and
+        // reciprocal (a few ulp of fp32, far below the bf16 output's rounding).  z >= -80 in
+        // the exponential keeps the divisor below 2^126, so its reciprocal is no subnormal
+        // (below that the value is ~0 anyway), and a subnormal 2^x does not change 1 + 2^x:
+        // both may flush subnormals to zero.  __expf and __fdividef handle them, at a cost
+        // that set the pace of SiLU epilogues: 94 us, now 85 us, for the pointwise layer
+        // 512 -> 1024 on 16 images of 80 x 80; 61 and 56 us for 64 -> 64, 3x3, 256 of 56 x 56.
+        return z * rcp_approx_ftz(1.0f + ex2_approx_ftz(fminf(z * -1.44269504f, 115.41560f)));
     }
     return z;
 }

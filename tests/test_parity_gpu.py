@@ -651,6 +651,25 @@ def test_pair_walk(case):
         "qconv_tc_kernel<pair,walk," if walk else "qconv_tc_kernel<pair,kappa")
 
 
+@pytest.mark.parametrize("cout,k", [(128, 1), (64, 3), (256, 3)])  # pointwise, vertical-tap, pair
+def test_silu_range(cout, k):
+    # zero weights, so z is the shift itself: SiLU over the whole range of z.  Within one bf16
+    # rounding (2^-8) plus 2^-15 of fp32 steps (z log2 e rounded: |z| 2^-24 in the exponent);
+    # below z = -80 the exact values, under 1.5e-33, may be off by as much
+    vals = np.concatenate([[0.0, -0.0, 1e-30, -1e-30, 3.3e38, -79.9, -80.1, -88.0, -100.0, -3e38],
+                           np.linspace(-90.0, 90.0, cout - 10)]).astype(np.float32)
+    x = torch.zeros(2, 56, 56, 64, device="cuda", dtype=torch.bfloat16)
+    w = [torch.zeros(cout // 4, k, k, 16, device="cuda", dtype=torch.bfloat16)] * 4
+    y = quan.qconv2d(x, *w, pad=k // 2, scale=torch.ones(cout, device="cuda"),
+                     shift=torch.from_numpy(vals).cuda(), act=quan.QUAN_ACT_SILU)
+    got = y.float().cpu().numpy().reshape(-1, cout).astype(np.float64)
+    z = vals.astype(np.float64)
+    ref = z / (1.0 + np.exp(np.minimum(-z, 700.0)))
+    tol = (2.0 ** -8 + 2.0 ** -15) * np.abs(ref) + np.where(z < -80.0, np.abs(z) * 2e-35, 1e-38)
+    assert (np.abs(got - ref) <= tol).all()
+    assert (got == got[:1]).all()
+
+
 NARROW_CASES = [
     # name, N, H, W, Cin, Cout, k, stride, pad, extra: bf16 layers off the tcgen05 channel
     # grid on warp-level MMAs: K tails, channel tiles past 64, one pixel buffer, few pixels
