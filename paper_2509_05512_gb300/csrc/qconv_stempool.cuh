@@ -260,7 +260,9 @@ __device__ __forceinline__ uint4 sp_poincare_pair(float2 a, float2 b, float2 c) 
     for (int e = 0; e < 2; ++e) {
         const float rr = px[e][0], gg = px[e][1], bb = px[e][2];
         const float n2 = fmaf(rr, rr, fmaf(gg, gg, bb * bb));
-        const float inv = __fdividef(1.0f, 1.0f + n2);
+        // (the divisor is at least 1: poincare.cu's __fdividef to the bit, which also handles
+        // subnormal divisors)
+        const float inv = rcp_approx_ftz(1.0f + n2);
         const float two_inv = 2.0f * inv;
         w[2 * e] = pack_bf16x2((1.0f - n2) * inv, rr * two_inv);
         w[2 * e + 1] = pack_bf16x2(gg * two_inv, bb * two_inv);
