@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace quan {
 namespace {
@@ -212,7 +213,14 @@ __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16
 
 __device__ __forceinline__ float act_fn(float z, int act) {
     if (act == 1) return fmaxf(z, 0.0f);
-    if (act == 2) return z / (1.0f + __expf(-z));
+    // SiLU z / (1 + e^-z), e^-z = 2^(-z log2 e), as (z / 16) (16 / (1 + 2^x)): the sixteenth of
+    // the divisor stays below 2^126 for every finite 2^x, so its approximate reciprocal is no
+    // subnormal, and a subnormal 2^x does not change 1 + 2^x: both may flush subnormals.  With
+    // an exact division SiLU took the pass over its memory time: 74 us for the statistics
+    // and this kernel at 64 x 56 x 56 x 256, now 61 (ReLU: 57).
+    if (act == 2)
+        return (z * 0.0625f) *
+               rcp_approx_ftz(fmaf(ex2_approx_ftz(z * -1.44269504f), 0.0625f, 0.0625f));
     return z;
 }
 

@@ -129,6 +129,23 @@ def test_train_forward(act, C):
     check_train(_dev(bits), x64, gamma, beta, 1e-5, act)
 
 
+@pytest.mark.parametrize("C", [64, 44, 32 + 28])
+def test_silu_range(C):
+    # gamma = 0, so z is beta itself: SiLU over the whole range of z, within one bf16 rounding
+    # (2^-8) plus 2^-15 of fp32 steps (z log2 e rounded: |z| 2^-24 in the exponent); 2^x
+    # overflows below z = -88.7, where the exact values are under 3e-37
+    beta = np.concatenate([[0.0, -0.0, 1e-30, -1e-30, 3.3e38, -88.0, -89.0, -100.0],
+                           np.linspace(-87.5, 90.0, C - 8)]).astype(np.float32)
+    x = torch.ones(3, 5, 7, C, device="cuda", dtype=torch.bfloat16)
+    y, _, _ = quan.iqbn_train(x, torch.zeros(C, device="cuda"), torch.from_numpy(beta).cuda(),
+                              act=quan.QUAN_ACT_SILU)
+    got = y.float().cpu().numpy().reshape(-1, C).astype(np.float64)
+    z = beta.astype(np.float64)
+    ref = z / (1.0 + np.exp(-z))
+    tol = (2.0 ** -8 + 2.0 ** -15) * np.abs(ref) + np.where(z < -88.0, 3e-37, 1e-38)
+    assert (np.abs(got - ref) <= tol).all()
+
+
 def test_train_forward_in_place_and_defaults():
     rng = np.random.default_rng(830)
     bits, x64 = _bf16(rng, (2, 8, 8, 128), scale=2.0, offset=-1.0)
