@@ -133,9 +133,11 @@ quan_status_t quan_qconv2d_fwd_res(const void* x, const void* wr, const void* wi
  * not bit for bit.
  *   workspace        device memory of at least quan_qconv2d_fwd_workspace_size() bytes,
  *                    256-byte aligned, owned by the caller, overlapping no tensor of the
- *                    call; ZERO-FILLED before its first use: every call leaves it as zero
- *                    again (after a QUAN_ERR_DEVICE_TIMEOUT, zero it once more).  Calls that
- *                    may run at the same time on the GPU need separate workspaces.  NULL
+ *                    call; ZERO-FILLED before its first use: every call leaves its flags
+ *                    (at the end) zero again, the partial sums before them as they are, so
+ *                    calls of any shapes may share it one after another on one device (after a
+ *                    QUAN_ERR_DEVICE_TIMEOUT, zero it once more).  Calls that may run at the
+ *                    same time on the GPU need separate workspaces.  NULL
  *                    (with workspace_bytes 0) or a smaller workspace: no split, the call runs
  *                    as quan_qconv2d_fwd / quan_qconv2d_fwd_res.
  * Errors as quan_qconv2d_fwd; a NULL workspace with workspace_bytes > 0 or a workspace not

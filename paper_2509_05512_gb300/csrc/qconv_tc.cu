@@ -1799,13 +1799,19 @@ bool encode_dw_map(CUtensorMap* map, const void* t, int C, int W, int H, int N, 
     return r == CUDA_SUCCESS;
 }
 
+// The split-K workspace: a partial tile of the widest channel tile (bnq = 64: 4 x 64 fp32
+// columns x 128 rows) for every SM, then a flag per SM.  The flags' place depends on the device
+// alone: calls of any channel tile and grid share a workspace, partial tiles are never cleared,
+// and a flag that lay where another call's partial tile had been would read as ready.
+size_t split_flags_offset(int num_sms) {
+    return static_cast<size_t>(num_sms) * 512 * 64 * sizeof(float);
+}
+
 }  // namespace
 
 size_t tc_split_workspace_bytes(int num_sms) {
-    // a partial tile of the widest tile (bnq = 64: 4 x 64 fp32 columns x 128 rows) and a
-    // flag per CTA of a full-width grid
-    const size_t n = num_sms > 0 ? static_cast<size_t>(num_sms) : 0;
-    return (n * 512 * 64 * sizeof(float) + n * 4 + 255) / 256 * 256;
+    const int n = num_sms > 0 ? num_sms : 0;
+    return (split_flags_offset(n) + static_cast<size_t>(n) * 4 + 255) / 256 * 256;
 }
 
 bool tc_supported(const ConvShape& s, const void* x, const void* const w[4], const void* out,
@@ -2000,15 +2006,14 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     prm.sk.on = 0;
     prm.sk.partial = nullptr;
     prm.sk.flags = nullptr;
-    const size_t slot_bytes = static_cast<size_t>(512) * bnq * sizeof(float);
-    const size_t sk_need = static_cast<size_t>(grid) * slot_bytes + static_cast<size_t>(grid) * 4;
-    if (opt.sk_ws != nullptr && opt.sk_ws_bytes >= sk_need &&
-        (mode == MODE_PAIR || mode == MODE_QUAD) && prm.num_tiles > grid &&
+    // (a CTA waits for its neighbour's flag: all of them resident, so no more than the SMs)
+    if (opt.sk_ws != nullptr && opt.sk_ws_bytes >= tc_split_workspace_bytes(num_sms) &&
+        grid <= num_sms && (mode == MODE_PAIR || mode == MODE_QUAD) && prm.num_tiles > grid &&
         prm.num_tiles < 2 * grid) {
         prm.sk.on = 1;
         prm.sk.partial = static_cast<float*>(opt.sk_ws);
         prm.sk.flags = reinterpret_cast<unsigned*>(static_cast<char*>(opt.sk_ws) +
-                                                   static_cast<size_t>(grid) * slot_bytes);
+                                                   split_flags_offset(num_sms));
     }
     set_kernel_name(walk                ? "qconv_tc_kernel<pair,walk,kappa=%d,bnq=%d>"
                     : mode == MODE_PAIR ? "qconv_tc_kernel<pair,kappa=%d,bnq=%d>"

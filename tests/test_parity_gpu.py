@@ -235,6 +235,12 @@ SPLITK_CASES = [
 ]
 
 
+def split_flags(ws):
+    # a flag per SM after a partial tile of 512 x 64 floats per SM, for every tile and grid
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return ws.view(torch.uint8)[sms * 512 * 64 * 4:sms * (512 * 64 * 4 + 4)]
+
+
 def run_split(d, ws, grid, tiles):
     kappa, bnq, mode = tiles
     quan.quan_set_tc_tiles(kappa, bnq, grid, mode)
@@ -265,12 +271,39 @@ def test_tc_split_k_layers(case):
     # every flag is clear again afterwards
     y2, _ = run_split(d, ws, grid, tiles)
     assert torch.equal(y1, y2)
-    flags = ws.view(torch.uint8)[grid * 512 * (tiles[1] or 64) * 4:]
-    assert int(flags[:grid * 4].count_nonzero()) == 0
+    assert int(split_flags(ws).count_nonzero()) == 0
     # no workspace: the unsplit kernel, within rounding of the split one
     y0, kernel0 = run_split(d, None, grid, tiles)
     assert not kernel0.endswith(",splitk>")
     assert_bf16_close(out_f64(y0), ref, name + "-unsplit")
+
+
+SPLITK_SHARED_CASES = [
+    # name, N, H, W, Cout, extra, grid, bnq: 3x3 layers of 128 input channels whose channel
+    # tiles and grids differ, in turn on one workspace that is not cleared between them
+    ("skw_64", 5, 15, 17, 256, {}, 6, 64),                     # 10 tiles
+    ("skw_32", 4, 12, 12, 256, {"residual": True}, 9, 32),     # 10
+    ("skw_48", 2, 13, 11, 320, {}, 5, 48),                     # 6
+    ("skw_16", 2, 13, 11, 256, {}, 11, 16),                    # 12
+    ("skw_64_grid3", 4, 12, 12, 256, {"bias": True}, 3, 64),   # 5
+]
+
+
+def test_tc_split_k_shared_workspace():
+    ws = quan.fwd_workspace()
+    first = {}
+    for rep in range(2):
+        for name, N, H, W, Cout, extra, grid, bnq in SPLITK_SHARED_CASES:
+            d = inputs.layer_inputs(inputs.small_layer(name, N, H, W, 128, Cout, 3, 1, 1,
+                                                       seed=(213, len(name)), **extra))
+            y, kernel = run_split(d, ws, grid, (0, 0, 0))
+            assert kernel == "qconv_tc_kernel<pair,kappa=32,bnq=%d,splitk>" % bnq, kernel
+            assert int(split_flags(ws).count_nonzero()) == 0, name
+            if rep == 0:
+                assert_bf16_close(out_f64(y), oracle_full(d), name)
+                first[name] = y
+            else:
+                assert torch.equal(y, first[name]), name
 
 
 def test_tc_split_k_full_size_stage4():
