@@ -175,26 +175,6 @@ __device__ __forceinline__ void cg2_expand(const Cg2Params& p, uint32_t sbase, u
     }
 }
 
-// Bounded wait with cluster-scope acquire (arrivals from the peer CTA); otherwise as
-// wait_or_abort.
-__device__ __forceinline__ bool wait_cluster_or_abort(uint32_t bar, uint32_t parity,
-                                                      uint64_t limit, volatile int* abort_flag,
-                                                      unsigned code) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
-    while (true) {
-        if (mbar_try_wait_sleep(bar, parity, WAIT_SUSPEND_NS) &&
-            mbar_try_wait_cluster(bar, parity))
-            return true;
-        if (*abort_flag) return false;
-        if (global_timer_ns() - t0 > limit) {
-            atomicOr(&g_status, code);
-            *abort_flag = 1;
-            return false;
-        }
-    }
-}
-
 // One expansion warp: wait for the staged letters, expand this CTA's share, make the stores
 // visible to the tensor cores, then tell the producer (the letters may be overwritten) and
 // the even CTA's issuers (this part of the B half is ready).

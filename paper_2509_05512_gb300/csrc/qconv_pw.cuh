@@ -33,7 +33,8 @@
 // the tile's pixels, 128, and the tensor cores exchange the halves, so a stage is 16 KB, the
 // ring six stages deep and the traffic half: 100 us.  The pixels of both CTAs complete on
 // the even CTA's barrier (cta_group::2 copies), whose issuer runs both tensor cores; commits
-// are multicast, and accumulators are handed back by both epilogues to the even CTA.
+// are multicast, and accumulators are handed back by both epilogues to the even CTA.  Waits
+// that the peer's arrivals, copies or multicast commits end acquire at cluster scope.
 //
 // Roles (20 warps, one CTA per SM, persistent):
 //   warp 0       TMA producer (one lane);
@@ -156,6 +157,12 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const ConvShape& s = p.s;
     const uint64_t limit = p.wait_limit_ns;
+    auto wait = [&](uint32_t bar, uint32_t parity, unsigned code) {
+        if constexpr (CG2)
+            return wait_cluster_or_abort(bar, parity, limit, abort_flag, code);
+        else
+            return wait_or_abort(bar, parity, limit, abort_flag, code);
+    };
     // this CTA's channel block and its pixel tiles t = t0, t0 + tstep, ...
     // (CG2: the pair's blocks are neighbours, mb even in CTA 0, and share their tiles)
     constexpr int STAGE = CG2 ? C::STAGE / 2 : C::STAGE;
@@ -209,8 +216,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
             uint32_t phase = 0;
             for (int t = t0; ok && t < p.num_tiles; t += tstep) {
                 for (int kc = 0; kc < p.kchunks; ++kc) {
-                    if (!wait_or_abort(empty_bar(st), phase ^ 1u, limit, abort_flag,
-                                       STATUS_TIMEOUT_PRODUCER)) {
+                    if (!wait(empty_bar(st), phase ^ 1u, STATUS_TIMEOUT_PRODUCER)) {
                         ok = false;
                         break;
                     }
@@ -244,7 +250,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0 && rank == 0) {
             constexpr uint32_t IDESC = make_idesc(CG2 ? 2 * BM : BM, PW_NPIX, 0);
-            bool ok = wait_or_abort(bready_bar, 0, limit, abort_flag, STATUS_TIMEOUT_MMA);
+            bool ok = wait(bready_bar, 0, STATUS_TIMEOUT_MMA);
             int issued = 0;
             auto commit = [](uint32_t bar) {  // CG2: on both CTAs' barriers
                 if constexpr (CG2)
@@ -264,16 +270,14 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
             for (int t = t0; ok && t < p.num_tiles; t += tstep, ++local) {
                 const int buf = local & 1;
                 const uint32_t use = static_cast<uint32_t>(local >> 1) & 1u;
-                if (!wait_or_abort(acce0 + 8u * buf, use ^ 1u, limit, abort_flag,
-                                   STATUS_TIMEOUT_MMA)) {
+                if (!wait(acce0 + 8u * buf, use ^ 1u, STATUS_TIMEOUT_MMA)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t d = tmem_base + static_cast<uint32_t>(buf * PW_NPIX);
                 for (int kc = 0; kc < p.kchunks; ++kc) {
-                    if (!wait_or_abort(full_bar(st), phase, limit, abort_flag,
-                                       STATUS_TIMEOUT_MMA)) {
+                    if (!wait(full_bar(st), phase, STATUS_TIMEOUT_MMA)) {
                         ok = false;
                         break;
                     }
@@ -332,9 +336,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
                 const int buf = local & 1;
                 const uint32_t use = static_cast<uint32_t>(local >> 1) & 1u;
                 bool ok = true;
-                if (lane == 0)
-                    ok = wait_or_abort(accf0 + 8u * buf, use, limit, abort_flag,
-                                       STATUS_TIMEOUT_EPILOGUE);
+                if (lane == 0) ok = wait(accf0 + 8u * buf, use, STATUS_TIMEOUT_EPILOGUE);
                 if (__shfl_sync(0xffffffffu, ok ? 1 : 0, 0) == 0) break;
                 tc_fence_after();
                 const uint32_t taddr = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) +

@@ -138,6 +138,26 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, uin
     }
 }
 
+// Bounded wait with cluster-scope acquire (arrivals from the peer CTA); otherwise as
+// wait_or_abort.
+__device__ __forceinline__ bool wait_cluster_or_abort(uint32_t bar, uint32_t parity,
+                                                      uint64_t limit, volatile int* abort_flag,
+                                                      unsigned code) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    const uint64_t t0 = global_timer_ns();
+    while (true) {
+        if (mbar_try_wait_sleep(bar, parity, WAIT_SUSPEND_NS) &&
+            mbar_try_wait_cluster(bar, parity))
+            return true;
+        if (*abort_flag) return false;
+        if (global_timer_ns() - t0 > limit) {
+            atomicOr(&g_status, code);
+            *abort_flag = 1;
+            return false;
+        }
+    }
+}
+
 // Bounded wait for a sequence word in shared memory (written with st_release_shared) to
 // reach `target` (wrap-safe comparison).  Same failure handling as wait_or_abort.
 __device__ __forceinline__ bool flag_wait_or_abort(uint32_t addr, uint32_t target,

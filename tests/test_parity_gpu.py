@@ -901,16 +901,18 @@ def test_maxpool(shape):
 
 # ------------------------------------------------------------------ failure detection
 
-@pytest.mark.parametrize("mode,issuers", [(2, 0), (3, 2), (3, 3), (4, 0), (5, 0), (6, 0),
-                                          (6, 1), (6, 2), (7, 0)])
+@pytest.mark.parametrize("mode,issuers", [(2, 0), (3, 2), (3, 3), (4, 0), (5, 0), (5, 1),
+                                          (6, 0), (6, 1), (6, 2), (7, 0)])
 def test_bounded_wait_timeout_every_kernel(mode, issuers):
     # the failure-injection path of the pair-mode, weight-stationary (two and three
-    # issuers), gather, pointwise and CTA-pair kernels (the CTA-pair kernel ignores the
-    # issuer count, which selects its staging here: halo, stride-2 halo, per tap)
+    # issuers), gather, pointwise and CTA-pair kernels (the last two ignore the issuer count,
+    # which selects the form here: one CTA or pairs; halo, stride-2 halo or per-tap staging)
     if mode == 4:
         spec = inputs.small_layer("inject_m", 2, 32, 32, 4, 64, 7, 2, 3, seed=(401, mode))
     elif mode == 5:
-        spec = inputs.small_layer("inject_m", 2, 16, 16, 64, 128, 1, 1, 0, seed=(401, mode))
+        spec = inputs.small_layer("inject_m", 2, 16, 16, 64, 256 if issuers else 128, 1, 1, 0,
+                                  seed=(401, mode))
+        issuers = 0
     elif mode == 6:
         spec = inputs.small_layer("inject_m", 2, 16, 16, 128 if issuers == 2 else 64, 128, 3,
                                   1 if issuers == 0 else 2, 1, seed=(401, mode))
