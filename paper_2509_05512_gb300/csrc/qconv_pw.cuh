@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + a_bytes);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::NUM_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile uint32_t* fills = tmem_slot + 2;  // CG2: stages each CTA of the pair filled
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int st) { return bar0 + 8u * st; };
     auto empty_bar = [&](int st) { return bar0 + 8u * (C::MAX_STAGES + st); };
@@ -183,6 +184,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
         mbar_init(drain_bar, 1);
         mbar_init(bready_bar, (CG2 ? 2 : 1) * PW_EXP_WARPS);
         *abort_flag = 0;
+        fills[0] = fills[1] = 0;
         fence_barrier_init();
     }
     if (warp == 0 && lane == 0) tma_prefetch_desc(&tmap_x);
@@ -211,6 +213,7 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
             griddep_wait();  // the previous kernel's output (this layer's input) is complete
             const uint64_t pol = l2_policy_evict_normal();
             uint32_t filled = 0, fill_parity = 0;
+            [[maybe_unused]] uint32_t nfills = 0;
             bool ok = true;
             int st = 0;
             uint32_t phase = 0;
@@ -235,14 +238,17 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
                     else
                         tma_load_5d(dst, &tmap_x, fb, 64 * kc, 0, 0, 0, t * p.rows_per_tile,
                                     pol);
+                    ++nfills;
                     if (++st == p.stages) {
                         st = 0;
                         phase ^= 1u;
                     }
                 }
             }
-            // (the odd CTA's copies complete on the even CTA's barrier, and it waits for that
-            // CTA at the end)
+            if constexpr (CG2)  // (read by both CTAs after the last cluster barrier)
+                for (uint32_t r = 0; r < 2; ++r)
+                    st_shared_cluster(mapa_shared(smem_u32(tmem_slot + 2 + rank), r), nfills);
+            // (the odd CTA's copies complete on the even CTA's barrier)
             if ((!ok || *abort_flag) && rank == 0)
                 drain_fills(full_bar(0), p.stages, filled, fill_parity, limit);
         }
@@ -388,7 +394,22 @@ __global__ void __launch_bounds__(PW_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     // CG2: the pair's MMAs into both CTAs' TMEM and both epilogues are done
-    if constexpr (CG2) cluster_sync_all();
+    if constexpr (CG2) {
+        cluster_sync_all();
+        // After an abort the odd CTA may have filled stages that the even one did not: they are
+        // counted on the even CTA's barriers, which it arms here, so that no copy still targets
+        // the odd CTA's shared memory when it exits.
+        if (fills[1] > fills[0]) {
+            if (rank == 0 && threadIdx.x == 0)
+                for (uint32_t k = fills[0]; k < fills[1]; ++k) {
+                    const uint32_t st = k % p.stages;
+                    mbar_arrive_expect_tx(full_bar(st), static_cast<uint32_t>(STAGE));
+                    drain_fills(full_bar(st), 1, 1u, (k / p.stages) & 1u, limit);
+                }
+            __syncwarp();
+            cluster_sync_all();
+        }
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
