@@ -24,6 +24,10 @@
  *               [Q_out][kh][kw][Q_in], contiguous.  Ho = (H + 2 pad - kh) / stride + 1
  *               (floor), likewise Wo.
  *   Convolution "convolution" is a cross-correlation (no kernel flip) with zero padding.
+ *               Infinite and NaN values: the kernels without tcgen05 leave the padding out of
+ *               the sums.  The tcgen05 kernels multiply it as zeros, so there an infinite or
+ *               NaN weight (in a weight gradient: dy, or x in the columns next to the image's
+ *               edge) makes NaN of border results that read it in the padding only.
  *   Epilogue    out = act(scale[c] * (acc + bias[c]) + shift[c] (+ residual)), every
  *               per-channel vector fp32 [C_out]; a NULL bias is 0, a NULL scale/shift pair
  *               is the identity (scale and shift must both be NULL or both non-NULL).

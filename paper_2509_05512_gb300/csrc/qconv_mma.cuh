@@ -128,6 +128,35 @@ __device__ __forceinline__ float activate(float z, int act) {
     return z;
 }
 
+__device__ __forceinline__ bool not_finite(float v) { return !(fabsf(v) <= 3.402823466e+38f); }
+
+// The taps of a pixel inside the source only: the MMAs multiply the zeros that stand for the
+// padding as well, which makes NaN of an infinite or NaN weight.  False where no tap is
+// outside (the MMAs' sum stands), else the sum without them.  m: the pixel's index in its
+// class; brow: its channel's row of the block weight.
+__device__ __forceinline__ bool sum_inside(const Params& p, const Class& c,
+                                           const __nv_bfloat16* brow, unsigned m, float& sum) {
+    const unsigned row = m / static_cast<unsigned>(c.Wc), n = row / static_cast<unsigned>(c.Hc);
+    const int hb = static_cast<int>(row - n * c.Hc) * p.istep + c.h0;
+    const int wb = static_cast<int>(m - row * c.Wc) * p.istep + c.w0;
+    const __nv_bfloat16* img = p.src + static_cast<long long>(n) * p.Hs * p.Ws * p.C;
+    bool outside = false;
+    sum = 0.f;
+#pragma unroll 1
+    for (int t = 0; t < c.th * c.tw; ++t) {
+        const int u = t / c.tw, h = hb + p.tdir * u, w = wb + p.tdir * (t - u * c.tw);
+        if (h < 0 || h >= p.Hs || w < 0 || w >= p.Ws) {
+            outside = true;
+            continue;
+        }
+        const __nv_bfloat16* g = img + (static_cast<long long>(h) * p.Ws + w) * p.C;
+#pragma unroll 1
+        for (int k = 0; k < p.C; ++k)
+            sum = fmaf(__bfloat162float(brow[t * p.C + k]), __bfloat162float(g[k]), sum);
+    }
+    return outside;
+}
+
 template <int OP, bool SEP>
 __global__ void __launch_bounds__(THREADS) qconv_mma_kernel(const __grid_constant__ Params p) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -296,26 +325,31 @@ __global__ void __launch_bounds__(THREADS) qconv_mma_kernel(const __grid_constan
                         mma(acc[3], a, b[2], b[3]);
                     }
                 }
+                // output pixel of the class's pixel m
+                auto pixel = [&](long long m) {
+                    if constexpr (OP == FWD) return m;
+                    const unsigned mm = static_cast<unsigned>(m);
+                    const unsigned row = mm / static_cast<unsigned>(c.Wc);
+                    const int j = static_cast<int>(mm - row * c.Wc);
+                    const unsigned n = row / static_cast<unsigned>(c.Hc);
+                    const int i = static_cast<int>(row - n * c.Hc);
+                    return (static_cast<long long>(n) * p.Hd + i * p.ostep + c.oh) * p.Wd +
+                           j * p.ostep + c.ow;
+                };
                 // rows m0 + lane / 4 (+ 8), channels nb + 8 t + 2 (lane % 4), + 1
+                const long long mrow = static_cast<long long>(tile - c.tile0) * PX + m0 + lane / 4;
+                float check = 0.f;  // NaN when one of the sums is not finite
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const long long m = static_cast<long long>(tile - c.tile0) * PX + m0 +
-                                        lane / 4 + 8 * h;
+                    const long long m = mrow + 8 * h;
                     if (m >= c.M) continue;
-                    long long o = m;
-                    if constexpr (OP == DGRAD) {
-                        const unsigned mm = static_cast<unsigned>(m);
-                        const unsigned row = mm / static_cast<unsigned>(c.Wc);
-                        const int j = static_cast<int>(mm - row * c.Wc);
-                        const unsigned n = row / static_cast<unsigned>(c.Hc);
-                        const int i = static_cast<int>(row - n * c.Hc);
-                        o = (static_cast<long long>(n) * p.Hd + i * p.ostep + c.oh) * p.Wd + j * p.ostep + c.ow;
-                    }
+                    const long long o = pixel(m);
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
                         const int ch = n0 + nb + 8 * t + 2 * (lane & 3);
                         if (ch >= n0 + nn) continue;  // (nn is even)
                         float z[2] = {acc[t][2 * h], acc[t][2 * h + 1]};
+                        check = fmaf(z[0], 0.f, fmaf(z[1], 0.f, check));
                         if constexpr (OP == FWD) {
                             const float2 f0 = affine[ch - n0], f1 = affine[ch - n0 + 1];
                             z[0] = fmaf(f0.x, z[0], f0.y);
@@ -333,6 +367,27 @@ __global__ void __launch_bounds__(THREADS) qconv_mma_kernel(const __grid_constan
                         }
                         *reinterpret_cast<__nv_bfloat162*>(p.out + o * p.Cd + ch) =
                             __floats2bfloat162_rn(z[0], z[1]);
+                    }
+                }
+                if (check != 0.f) {  // rare: the thread's sixteen sums once more
+#pragma unroll 1
+                    for (int e = 0; e < 16; ++e) {
+                        const long long m = mrow + 8 * (e & 1);
+                        const int row = nb + 8 * (e >> 2) + 2 * (lane & 3) + ((e >> 1) & 1);
+                        float z;
+                        if (m >= c.M || row >= nn ||
+                            !sum_inside(p, c, sB + row * ld, static_cast<unsigned>(m), z))
+                            continue;
+                        const long long o = pixel(m);
+                        const long long at = o * p.Cd + n0 + row;
+                        if constexpr (OP == FWD) {
+                            z = fmaf(affine[row].x, z, affine[row].y);
+                            if (p.ep.residual)
+                                z += __bfloat162float(
+                                    static_cast<const __nv_bfloat16*>(p.ep.residual)[at]);
+                            z = activate(z, s.act);
+                        }
+                        p.out[at] = __float2bfloat16_rn(z);
                     }
                 }
             }
@@ -477,6 +532,7 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
     // G to shared memory, then every letter element adds its four blocks and goes out once
     float* sG = reinterpret_cast<float*>(smem);
     const int ldg = p.cols + 1;
+    float check = 0.f;  // NaN when one of the sums is not finite
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
         if (16 * a >= p.rows) break;
@@ -485,8 +541,35 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
             const int n = 16 * (warp + 8 * (t >> 1)) + 8 * (t & 1) + 2 * (lane & 3);
             if (n >= p.cols) continue;
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
+            for (int e = 0; e < 4; ++e) {
                 sG[(16 * a + lane / 4 + 8 * (e >> 1)) * ldg + n + (e & 1)] = acc[a][t][e];
+                check = fmaf(acc[a][t][e], 0.f, check);
+            }
+        }
+    }
+    // Rare: the thread's sums that are not finite once more, over the pixels whose tap is inside
+    // the image (the MMAs multiply dy by the zeros that stand for the padding).
+    if (check != 0.f) {
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i) {
+            const int r = 16 * (i >> 4) + lane / 4 + 8 * ((i >> 1) & 1);
+            const int n = 16 * (warp + 8 * ((i >> 3) & 1)) + 8 * ((i >> 2) & 1) + 2 * (lane & 3) + (i & 1);
+            if (r >= rn || n >= cn || !not_finite(sG[r * ldg + n])) continue;
+            const int t = n / s.Cin, dh = (tap0 + t) / s.kw, dw = tap0 + t - dh * s.kw;
+            float g = 0.f;
+#pragma unroll 1
+            for (long long m = beg; m < end; ++m) {
+                const unsigned row = static_cast<unsigned>(m) / static_cast<unsigned>(s.Wo);
+                const unsigned img = row / static_cast<unsigned>(s.Ho);
+                const int h = static_cast<int>(row - img * s.Ho) * s.stride - s.pad + dh;
+                const int w = static_cast<int>(static_cast<unsigned>(m) - row * s.Wo) * s.stride -
+                              s.pad + dw;
+                if (h < 0 || h >= s.H || w < 0 || w >= s.W) continue;
+                const long long px = (static_cast<long long>(img) * s.H + h) * s.W + w;
+                g = fmaf(__bfloat162float(p.dy[m * s.Cout + r0 + r]),
+                         __bfloat162float(p.x[px * s.Cin + n - t * s.Cin]), g);
+            }
+            sG[r * ldg + n] = g;
         }
     }
     __syncthreads();

@@ -114,6 +114,109 @@ __device__ __forceinline__ void product(float4& c, const float4& a, const float4
     }
 }
 
+__device__ __forceinline__ bool not_finite(const float4& v) {
+    // (NaN when one of them is not finite)
+    return fmaf(v.x, 0.f, fmaf(v.y, 0.f, fmaf(v.z, 0.f, v.w * 0.f))) != 0.f;
+}
+
+// One output quaternion from the taps inside the image (WGRAD: the pixels whose tap is) only:
+// the tiles multiply the zeros that stand for the padding as well, which makes NaN of an
+// infinite or NaN factor.  False where nothing is outside: the tile's sum stands.
+// FWD: channel i, output pixel (n, h, w) by the input pixel of its first tap; DGRAD: channel i,
+// dx pixel (n, h, w); WGRAD: channel i, input channel n, tap (h, w), pixels k0 .. k1 - 1.
+template <typename T, int OP, bool SEP>
+__device__ __forceinline__ bool sum_inside(const Params& p, int i, int n, int h, int w,
+                                           long long k0, long long k1, float4& acc) {
+    const ConvShape& s = p.s;
+    const T* b = static_cast<const T*>(p.b);
+    acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool outside = false;
+    if constexpr (OP == WGRAD) {
+        const T* dy = static_cast<const T*>(p.a[0]);
+#pragma unroll 1
+        for (long long k = k0; k < k1; ++k) {
+            const long long r = k / s.Wo, img = r / s.Ho;
+            const int y = static_cast<int>(r - img * s.Ho) * s.stride - s.pad + h;
+            const int x = static_cast<int>(k - r * s.Wo) * s.stride - s.pad + w;
+            if (y < 0 || y >= s.H || x < 0 || x >= s.W) {
+                outside = true;
+                continue;
+            }
+            const float4 g = quat(dy + k * s.Cout + i, s.Qout);
+            const float4 q = quat(b + ((img * s.H + y) * s.W + x) * s.Cin + n, s.Qin);
+            product<SEP>(acc, SEP ? mix_eq9(g) : g, SEP ? q : conj(q));
+        }
+    } else {
+        const int C = OP == FWD ? s.Qin : s.Qout;
+        const int hs = OP == FWD ? s.H : s.Ho, ws = OP == FWD ? s.W : s.Wo;
+#pragma unroll 1
+        for (int t = 0; t < s.kh * s.kw; ++t) {
+            const int dh = t / s.kw, dw = t - dh * s.kw;
+            int y = h + dh, x = w + dw;
+            if constexpr (OP == DGRAD) {  // the output pixel this tap reads for dx (h, w)
+                y = h + s.pad - dh;
+                x = w + s.pad - dw;
+                if (y % s.stride != 0 || x % s.stride != 0) continue;
+                y /= s.stride;
+                x /= s.stride;
+            }
+            if (y < 0 || y >= hs || x < 0 || x >= ws) {
+                outside = true;
+                continue;
+            }
+            const T* px = b + ((static_cast<long long>(n) * hs + y) * ws + x) * (4LL * C);
+#pragma unroll 1
+            for (int c = 0; c < C; ++c) {
+                const long long row = OP == FWD ? i : c, col = OP == FWD ? c : i;
+                const float4 q = letters<T>(p, (row * s.kh * s.kw + t) * s.Qin + col);
+                const float4 g = quat(px + c, C);
+                product<SEP>(acc, OP == DGRAD && !SEP ? conj(q) : q,
+                             OP == DGRAD && SEP ? mix_eq9(g) : g);
+            }
+        }
+    }
+    return outside;
+}
+
+// One output quaternion of FWD at offset o (component q at o + q Qout): Eq. 7's mix of the
+// separable form, then act(scale (y + bias) + shift + residual).
+template <typename T, bool SEP>
+__device__ __forceinline__ void finish(const Params& p, const float4& v, const float (&bi)[4],
+                                       const float (&sc)[4], const float (&sh)[4], long long o) {
+    const ConvShape& s = p.s;
+    const T* res = static_cast<const T*>(p.ep.residual);
+    T* out = static_cast<T*>(p.out);
+    float z[4] = {v.x, v.y, v.z, v.w};
+    if constexpr (SEP) {
+        z[0] = v.x - v.y - v.z - v.w;
+        z[1] = v.x + v.y + v.z - v.w;
+        z[2] = v.x - v.y + v.z + v.w;
+        z[3] = v.x + v.y - v.z + v.w;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float y = z[q] + bi[q];
+        if (p.ep.scale) y = fmaf(sc[q], y, sh[q]);
+        if (res) y += to_f32(res[o + q * s.Qout]);
+        store(out + o + q * s.Qout, activate(y, s.act));
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void store4(T* o, int step, const float4& v) {
+    store(o, v.x);
+    store(o + step, v.y);
+    store(o + 2 * step, v.z);
+    store(o + 3 * step, v.w);
+}
+
+__device__ __forceinline__ void add4(float* const (&dw)[4], long long o, const float4& v) {
+    atomicAdd(dw[0] + o, v.x);
+    atomicAdd(dw[1] + o, v.y);
+    atomicAdd(dw[2] + o, v.z);
+    atomicAdd(dw[3] + o, v.w);
+}
+
 template <typename T, int OP, bool SEP, int TI, int TJ>
 __global__ void __launch_bounds__(THREADS, 1) qgemm_kernel(const __grid_constant__ Params p) {
     __shared__ float4 sa[KC][MAX_I + 1];
@@ -349,70 +452,73 @@ __global__ void __launch_bounds__(THREADS, 1) qgemm_kernel(const __grid_constant
     }
     if (!active || grp != 0) return;
 
+    // output channel i's vectors (FWD)
+    float bi[4], sc[4], sh[4];
+    auto vectors = [&](int i) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = q * s.Qout + i;
+            bi[q] = p.ep.bias ? __ldg(p.ep.bias + c) : 0.f;
+            sc[q] = p.ep.scale ? __ldg(p.ep.scale + c) : 1.f;
+            sh[q] = p.ep.scale ? __ldg(p.ep.shift + c) : 0.f;
+        }
+    };
+    // DGRAD: dx pixel (n, h, w) of the class's pixel m
+    auto dx_pixel = [&](long long m, long long& n, int& h, int& w) {
+        const long long rr = m / Wc;
+        w = static_cast<int>(m - rr * Wc) * s.stride + cb;
+        n = rr / Hc;
+        h = static_cast<int>(rr - n * Hc) * s.stride + ca;
+    };
+    T* out = static_cast<T*>(p.out);
+    unsigned odd = 0;  // the quaternions that are not finite
 #pragma unroll
     for (int r = 0; r < TI; ++r) {
         const int i = i0 + ti + r * p.ni;
         if (i >= p.I) continue;
+        if constexpr (OP == FWD) vectors(i);
+#pragma unroll
+        for (int c = 0; c < TJ; ++c) {
+            const long long m = j0 + tj + c * p.nj;
+            if (m >= J) continue;
+            const float4& v = acc[r][c];
+            const bool bad = not_finite(v);
+            if (bad) odd |= 1u << (r * TJ + c);
+            if constexpr (OP == FWD) {
+                finish<T, SEP>(p, v, bi, sc, sh, m * s.Cout + i);
+            } else if constexpr (OP == DGRAD) {
+                long long n;
+                int h, w;
+                dx_pixel(m, n, h, w);
+                store4(out + ((n * s.H + h) * s.W + w) * s.Cin + i, s.Qin, v);
+            } else if (!bad) {
+                add4(p.dw, static_cast<long long>(i) * J + m, v);
+            }
+        }
+    }
+    // rare: those once more without the padding
+#pragma unroll 1
+    for (; odd != 0; odd &= odd - 1) {
+        const int e = __ffs(odd) - 1;
+        const int i = i0 + ti + e / TJ * p.ni, jl = tj + e % TJ * p.nj;
+        const long long m = j0 + jl;
+        float4 v;
         if constexpr (OP == FWD) {
-            float bi[4], sc[4], sh[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = q * s.Qout + i;
-                bi[q] = p.ep.bias ? __ldg(p.ep.bias + c) : 0.f;
-                sc[q] = p.ep.scale ? __ldg(p.ep.scale + c) : 1.f;
-                sh[q] = p.ep.scale ? __ldg(p.ep.shift + c) : 0.f;
-            }
-            const T* res = static_cast<const T*>(p.ep.residual);
-            T* out = static_cast<T*>(p.out);
-#pragma unroll
-            for (int c = 0; c < TJ; ++c) {
-                const long long m = j0 + tj + c * p.nj;
-                if (m >= J) continue;
-                const float4 v = acc[r][c];
-                float z[4] = {v.x, v.y, v.z, v.w};
-                if constexpr (SEP) {  // Eq. 7
-                    z[0] = v.x - v.y - v.z - v.w;
-                    z[1] = v.x + v.y + v.z - v.w;
-                    z[2] = v.x - v.y + v.z + v.w;
-                    z[3] = v.x + v.y - v.z + v.w;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const long long o = m * s.Cout + q * s.Qout + i;
-                    float y = z[q] + bi[q];
-                    if (p.ep.scale) y = fmaf(sc[q], y, sh[q]);
-                    if (res) y += to_f32(res[o]);
-                    store(out + o, activate(y, s.act));
-                }
-            }
+            const int4 px = tab[jl];
+            if (!sum_inside<T, OP, SEP>(p, i, px.x, px.y, px.z, 0, 0, v)) continue;
+            vectors(i);
+            finish<T, SEP>(p, v, bi, sc, sh, m * s.Cout + i);
         } else if constexpr (OP == DGRAD) {
-            T* out = static_cast<T*>(p.out);
-#pragma unroll
-            for (int c = 0; c < TJ; ++c) {
-                const int j = tj + c * p.nj;
-                const long long m = j0 + j;
-                if (m >= J) continue;
-                const long long rr = m / Wc;
-                const int w = static_cast<int>(m - rr * Wc) * s.stride + cb;
-                const long long n = rr / Hc;
-                const int h = static_cast<int>(rr - n * Hc) * s.stride + ca;
-                T* o = out + ((n * s.H + h) * s.W + w) * s.Cin + i;
-                store(o, acc[r][c].x);
-                store(o + s.Qin, acc[r][c].y);
-                store(o + 2 * s.Qin, acc[r][c].z);
-                store(o + 3 * s.Qin, acc[r][c].w);
-            }
+            long long n;
+            int h, w;
+            dx_pixel(m, n, h, w);
+            if (!sum_inside<T, OP, SEP>(p, i, static_cast<int>(n), h, w, 0, 0, v)) continue;
+            store4(out + ((n * s.H + h) * s.W + w) * s.Cin + i, s.Qin, v);
         } else {
-#pragma unroll
-            for (int c = 0; c < TJ; ++c) {
-                const long long j = j0 + tj + c * p.nj;
-                if (j >= J) continue;
-                const long long o = static_cast<long long>(i) * J + j;
-                atomicAdd(p.dw[0] + o, acc[r][c].x);
-                atomicAdd(p.dw[1] + o, acc[r][c].y);
-                atomicAdd(p.dw[2] + o, acc[r][c].z);
-                atomicAdd(p.dw[3] + o, acc[r][c].w);
-            }
+            const int tap = static_cast<int>(m / s.Qin), dh = tap / s.kw;
+            const int ci = static_cast<int>(m - static_cast<long long>(tap) * s.Qin);
+            sum_inside<T, OP, SEP>(p, i, ci, dh, tap - dh * s.kw, kbeg, kbeg + K, v);
+            add4(p.dw, static_cast<long long>(i) * J + m, v);
         }
     }
 }

@@ -98,3 +98,24 @@ def assert_f32_close(got, ref, what=""):
     assert max_abs <= F32_MAX_ABS_RMS * rms, "%s: max-abs %.3e > %.1e * RMS %.3e" % (
         what, max_abs, F32_MAX_ABS_RMS, rms)
     return rel_l2, max_abs, rms
+
+
+def inject(bits, dtype, *values):
+    """A copy of a generated tensor (bf16 as bits) with (index, value) pairs set in it."""
+    out = np.array(bits, copy=True)
+    for idx, v in values:
+        if dtype == "bf16":
+            out[idx] = (np.float32(v).view(np.uint32) >> 16).astype(out.dtype)
+        else:
+            out[idx] = v
+    return out
+
+
+def assert_same_finite(got, ref, close, what=""):
+    """Finite values where the reference has them, and those by `close`.  (Which sums with an
+    infinite factor are infinite and which NaN depends on how a form orders its products.)"""
+    got, ref = np.asarray(got, dtype=np.float64), np.asarray(ref, dtype=np.float64)
+    fin = np.isfinite(ref)
+    assert not fin.all() and fin.any(), what + ": the case has both kinds"
+    assert np.array_equal(np.isfinite(got), fin), what
+    close(got[fin], ref[fin], what)

@@ -10,7 +10,8 @@ torch = pytest.importorskip("torch")
 
 import oracle
 from paper_2509_05512_gb300 import build, inputs, quan
-from tests._util import assert_bf16_close, assert_f32_close, host_f64, out_f64, to_dev
+from tests._util import (assert_bf16_close, assert_f32_close, assert_same_finite, host_f64, inject,
+                         out_f64, to_dev)
 
 pytestmark = pytest.mark.gpu
 
@@ -214,6 +215,35 @@ def test_cuda_core_gradients(case, sep):
     assert path == quan.QUAN_PATH_SIMT
     assert_bf16_close(got, oracle_bwd_data(d, sep), name + " dx")
     check_weight(d, separable=sep, path=quan.QUAN_PATH_SIMT)
+
+
+PADDING_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad: off the tcgen05 grid, on each kernel
+    ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1),
+    ("inf_mma_s2", 2, 9, 8, 20, 68, 3, 2, 1),
+    ("inf_core_s5", 1, 12, 11, 20, 28, 3, 5, 1),
+    ("inf_core_c260", 1, 6, 5, 260, 12, 3, 1, 1),
+]
+
+
+@pytest.mark.parametrize("sep", [False, True], ids=["full", "sep"])
+@pytest.mark.parametrize("case", PADDING_CASES, ids=[c[0] for c in PADDING_CASES])
+def test_padding_is_no_factor(case, sep):
+    # infinite and NaN weights (dx) and output gradients (dW) reach the sums whose taps read
+    # them inside the image, and no others
+    name, N, H, W, Cin, Cout, k, s, p = case
+    d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(617, len(name))))
+    e = dict(d)
+    e["wi"] = inject(d["wi"], "bf16", ((1, 0, 0, 1), np.inf), ((2, k - 1, k - 1, 4), np.nan))
+    got, _, _ = gpu_bwd_data(e, separable=sep, path=quan.QUAN_PATH_SIMT)
+    with np.errstate(invalid="ignore"):
+        assert_same_finite(got, oracle_bwd_data(e, sep), assert_bf16_close, name + " dx")
+        e = dict(d)
+        e["dy"] = inject(d["dy"], "bf16", ((0, 0, 0, 1), np.inf), ((0, -1, 0, 2), np.nan))
+        got, _ = gpu_bwd_weight(e, separable=sep, path=quan.QUAN_PATH_SIMT)
+        ref = oracle_bwd_weight(e, sep)
+    for L in range(4):
+        assert_same_finite(got[L], ref[L], assert_f32_close, "%s dW[%d]" % (name, L))
 
 
 def test_bwd_data_rectangular_filter():

@@ -12,8 +12,8 @@ torch = pytest.importorskip("torch")
 
 import oracle
 from paper_2509_05512_gb300 import build, inputs, quan
-from tests._util import (assert_bf16_close, assert_f32_close, host_f64, out_f64, to_dev,
-                         to_dev_f32)
+from tests._util import (assert_bf16_close, assert_f32_close, assert_same_finite, host_f64,
+                         inject, out_f64, to_dev, to_dev_f32)
 
 pytestmark = pytest.mark.gpu
 
@@ -738,6 +738,38 @@ def test_f32_layers(case):
     name, N, H, W, Cin, Cout, k, s, p = case
     check(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, dtype="f32", bias=True,
                              act=quan.QUAN_ACT_SILU, seed=(303, len(name))))
+
+
+PADDING_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad, dtype, sep
+    ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1, "bf16", False),
+    ("inf_mma_sep", 2, 9, 7, 24, 68, 3, 1, 1, "bf16", True),
+    ("inf_mma_s2", 2, 9, 12, 12, 20, 5, 2, 2, "bf16", False),
+    ("inf_core", 1, 6, 7, 60, 36, 7, 1, 3, "bf16", False),
+    ("inf_core_sep", 1, 6, 7, 60, 36, 7, 1, 3, "bf16", True),
+    ("inf_f32", 2, 9, 8, 12, 20, 3, 1, 1, "f32", False),
+]
+
+
+@pytest.mark.parametrize("case", PADDING_CASES, ids=[c[0] for c in PADDING_CASES])
+def test_padding_is_no_factor(case):
+    # an infinite and a NaN weight reach the outputs whose taps read them inside the image,
+    # and no others: the padding is left out of the sums, not multiplied as zeros
+    name, N, H, W, Cin, Cout, k, s, p, dtype, sep = case
+    d = inputs.layer_inputs(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, dtype=dtype,
+                                               bias=True, seed=(307, len(name))))
+    d["wi"] = inject(d["wi"], dtype, ((1, 0, 0, 2), np.inf), ((3, k - 1, k - 1, 0), np.nan))
+    x = to_dev(d["x"], dtype)
+    w = [to_dev(d[n], dtype) for n in ("wr", "wi", "wj", "wk")]
+    bias, scale, shift = (to_dev_f32(d[n]) for n in ("bias", "scale", "shift"))
+    y = quan.qconv2d(x, *w, stride=s, pad=p, bias=bias, scale=scale, shift=shift,
+                     separable=sep)
+    fn = oracle.qconv2d_separable if sep else oracle.qconv2d
+    with np.errstate(invalid="ignore"):
+        ref = fn(host_f64(d["x"], dtype), *(host_f64(d[n], dtype) for n in ("wr", "wi", "wj", "wk")),
+                 stride=s, pad=p, bias=d["bias"], scale=d["scale"], shift=d["shift"])
+    assert_same_finite(out_f64(y), ref,
+                        assert_bf16_close if dtype == "bf16" else assert_f32_close, name)
 
 
 def test_simt_fp32_shapes():
