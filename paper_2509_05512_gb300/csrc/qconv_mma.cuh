@@ -24,7 +24,10 @@
 // memory ([n][k], k contiguous) for a persistent run over tiles of 64 pixels, whose gathered
 // rows ([pixel][k]) are double-buffered.  WGRAD runs over tiles of 64 pixels of a chunk with
 // the gathered rows of a group of taps and dy's rows double-buffered, all of a 64 x 256 tile
-// of G in registers.
+// of G in registers.  Its MMA sums are of one tile each and added up in fp32: a block of a wide
+// layer (few blocks along the pixels) otherwise chains thousands of MMA steps.  Relative error
+// against 64 bits, normal inputs, 252 -> 252 channels, 8 images of 126 x 126, 3x3: 3.6e-5 in one
+// chain, 4.1e-7 so (2.33 and 1.97 ms), 1.5e-6 with a thread per weight.
 #pragma once
 
 namespace quan {
@@ -477,13 +480,14 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
     };
 
     // warp: column tiles of 16 at 16 (warp + 8 t), t = 0, 1; all row tiles of 16
-    float acc[4][4][4];  // [row tile][column tile of 8][..]
+    float acc[4][4][4];  // [row tile][column tile of 8][..]: the sums of one pixel tile
+    float sum[4][4][4];  // of all tiles
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[a][b][e] = 0.f;
+            for (int e = 0; e < 4; ++e) acc[a][b][e] = sum[a][b][e] = 0.f;
     int buf = 0;
     long long lm = beg;  // the next tile to request
     for (long long m0 = beg; m0 < end; m0 += PX) {
@@ -523,6 +527,17 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
                 }
             }
         }
+        // The MMAs round each step towards zero, so a chain of them loses accuracy with its
+        // length: fp32 additions, rounded to nearest, take over after every tile's four.
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    sum[a][t][e] += acc[a][t][e];
+                    acc[a][t][e] = 0.f;
+                }
         __syncthreads();
         buf ^= 1;
     }
@@ -542,8 +557,8 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
             if (n >= p.cols) continue;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                sG[(16 * a + lane / 4 + 8 * (e >> 1)) * ldg + n + (e & 1)] = acc[a][t][e];
-                check = fmaf(acc[a][t][e], 0.f, check);
+                sG[(16 * a + lane / 4 + 8 * (e >> 1)) * ldg + n + (e & 1)] = sum[a][t][e];
+                check = fmaf(sum[a][t][e], 0.f, check);
             }
         }
     }

@@ -217,6 +217,23 @@ def test_cuda_core_gradients(case, sep):
     check_weight(d, separable=sep, path=quan.QUAN_PATH_SIMT)
 
 
+def test_bwd_weight_long_chunks():
+    # 36 groups of outputs leave four blocks along 100,800 pixels.  An MMA step rounds towards
+    # zero by at most 2^-23 of its sum: the four of a tile of 64 pixels by 4 2^-23 sqrt(64) of
+    # one product (of random sign), n tiles by sqrt(n) times that against a result of
+    # sqrt(64 n): 4.8e-7; the additions of a block's 394 tiles sqrt(394) 2^-25 = 5.9e-7 at most
+    d = layer(inputs.small_layer("long", 7, 120, 120, 252, 252, 3, 1, 1, seed=(618, 0)))
+    got, kernel = gpu_bwd_weight(d)
+    assert kernel == "bwd_weight_simt_kernel"
+    part = [0, 40]  # output channels of the reference
+    sub = dict(d)
+    sub["dy"] = np.concatenate([d["dy"][..., [63 * q + c for c in part]] for q in range(4)], -1)
+    ref = oracle_bwd_weight(sub)
+    for L in range(4):
+        rel, _, _ = assert_f32_close(got[L][part], ref[L], "dW[%d]" % L)
+        assert rel < 1.1e-6, (L, rel)
+
+
 PADDING_CASES = [
     # name, N, H, W, Cin, Cout, k, stride, pad: off the tcgen05 grid, on each kernel
     ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1),
