@@ -169,13 +169,14 @@ cudaError_t launch_mma_bwd_weight(const ConvShape& s, const void* x, const void*
     const long long tiles = (s.M + qm::PX - 1) / qm::PX;
     if (chunks > tiles) chunks = tiles;
     p.chunk = (tiles + chunks - 1) / chunks * qm::PX;
-    chunks = (s.M + p.chunk - 1) / p.chunk;
+    p.chunks = static_cast<int>((s.M + p.chunk - 1) / p.chunk);
     auto kern = s.sep ? qm::qconv_mma_dw_kernel<true> : qm::qconv_mma_dw_kernel<false>;
     static std::atomic<unsigned long long> done[2];
     const cudaError_t e = allow_smem(kern, smem, done[s.sep ? 1 : 0]);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(y)),
-                      dim3(qm::THREADS), static_cast<size_t>(smem), stream, p);
+    // (at most 4096 taps x 16 row tiles: a line of blocks, as they pass a grid's second dimension)
+    return launch_pdl(kern, dim3(static_cast<unsigned>(p.chunks * y)), dim3(qm::THREADS),
+                      static_cast<size_t>(smem), stream, p);
 }
 
 }  // namespace quan

@@ -78,7 +78,8 @@ struct WParams {
     int tg, groups;               // taps per group, groups
     int mt;                       // row tiles of 64
     int cols, rows;               // tg * Cin rounded up to 16; rows of a row tile rounded up
-    long long chunk;              // pixels per blockIdx.x (a multiple of PX)
+    int chunks;                   // blocks along the pixels
+    long long chunk;              // pixels of each (a multiple of PX)
 };
 
 __device__ __forceinline__ void cp8(uint32_t dst, const void* src, bool ok) {
@@ -412,7 +413,8 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
     __nv_bfloat16* sX = reinterpret_cast<__nv_bfloat16*>(smem);  // [2][PX][ldx]
     __nv_bfloat16* sY = sX + 2 * PX * ldx;                       // [2][PX][ldy]
     __shared__ int tab[WG_COLS / 4];
-    const int grp = static_cast<int>(blockIdx.y) % p.groups, mt = blockIdx.y / p.groups;
+    const int by = static_cast<int>(blockIdx.x) / p.chunks;
+    const int grp = by % p.groups, mt = by / p.groups;
     const int tap0 = grp * p.tg, taps_all = s.kh * s.kw;
     const int tn = taps_all - tap0 < p.tg ? taps_all - tap0 : p.tg;
     const int r0 = mt * MAX_N;
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, 1) qconv_mma_dw_kernel(const __grid_c
         const int r = i / (ldy - rn);
         sY[r * ldy + rn + i - r * (ldy - rn)] = __float2bfloat16_rn(0.f);
     }
-    const long long beg = blockIdx.x * p.chunk;
+    const long long beg = (static_cast<int>(blockIdx.x) - by * p.chunks) * p.chunk;
     long long end = beg + p.chunk;
     if (end > s.M) end = s.M;
     const uint32_t aX = smem_u32(sX), aY = smem_u32(sY);

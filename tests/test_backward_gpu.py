@@ -234,6 +234,22 @@ def test_bwd_weight_long_chunks():
         assert rel < 1.1e-6, (L, rel)
 
 
+def test_bwd_weight_most_blocks():
+    # 4096 taps in groups of one and 16 row tiles: 65,536 blocks
+    rng = np.random.default_rng(619)
+    bits = lambda n: (rng.standard_normal(n).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
+    x, dy = bits((1, 64, 64, 132)), bits((1, 1, 1, 1024))
+    out = tuple(torch.full((256, 64, 64, 33), float("nan"), device="cuda") for _ in range(4))
+    quan.qconv2d_backward_weight(to_dev(x, "bf16"), to_dev(dy, "bf16"), kh=64, kw=64, out=out)
+    torch.cuda.synchronize()
+    part = [0, 255]
+    sub = np.concatenate([dy[..., [256 * q + c for c in part]] for q in range(4)], -1)
+    ref = oracle.qconv2d_bwd_weight(host_f64(x, "bf16"), host_f64(sub, "bf16"), kh=64, kw=64)
+    for L in range(4):
+        assert bool(torch.isfinite(out[L]).all())
+        assert_f32_close(out_f64(out[L][part]), ref[L], "dW[%d]" % L)
+
+
 PADDING_CASES = [
     # name, N, H, W, Cin, Cout, k, stride, pad: off the tcgen05 grid, on each kernel
     ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1),
