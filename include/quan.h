@@ -316,9 +316,10 @@ quan_status_t quan_qconv2d_sep_bwd_data(const void* dy, const void* wr, const vo
  * aligned, pairwise disjoint and disjoint from x and dy): zeroed on the stream, then
  * accumulated over all N * Ho * Wo output pixels (fp32 partial sums added with atomics,
  * so the summation order, and the last bits, vary from run to run).  Stride 1 or 2 with Cin
- * and Cout multiples of 64 (Cout <= 256 or a multiple of 256) and 16-byte aligned x and dy
- * runs on the tensor cores (the real weight gradient of every tap as one product over
- * the pixels, folded into the four letters), other shapes on CUDA cores;
+ * and Cout multiples of 64 (Cout <= 256 or a multiple of 256), output rows of at most 256
+ * pixels (128 at stride 2), filters of up to 128 + pad taps a side, pad <= 128 and 16-byte
+ * aligned x and dy runs on the tensor cores (the real weight gradient of every tap as one
+ * product over the pixels, folded into the four letters), other shapes as QUAN_PATH_SIMT;
  * quan_set_path(QUAN_PATH_TC) makes those fail with QUAN_ERR_UNSUPPORTED.
  * x is the forward input, bf16 [N][H][W][Cin].
  */

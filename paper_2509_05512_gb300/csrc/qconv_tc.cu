@@ -1655,8 +1655,8 @@ void dw_row_share(const ConvShape& s, int* ndw, int* slots, int* n0) {
 }
 
 // The shapes the kernel is offered: output rows of at most 256 pixels (128 at stride 2) whose
-// blocks of whole rows would fit, corner offsets of the walk within the im2col encoding, and a
-// walk of 32-bit positions.
+// blocks of whole rows would fit, corner and tap offsets of the walk within the im2col encoding,
+// and a walk of 32-bit positions.
 bool dw_accepts(const ConvShape& s) {
     if (s.stride < 1 || s.stride > 2 || s.Cin % 64 != 0 || s.Cout % 64 != 0) return false;
     if (s.Cout > 256 && s.Cout % 256 != 0) return false;
@@ -1666,6 +1666,9 @@ bool dw_accepts(const ConvShape& s) {
     if (static_cast<long long>(s.N) * s.Ho * Wp > 0x7fffffffLL - 4096) return false;
     auto corner = [](int v) { return v >= -128 && v <= 127; };
     if (!corner(org) || n0 > 128) return false;
+    // a tap's distance from the walk's first row and column: 8 bits in a 4-D map
+    auto offset = [&](int k) { return s.stride == 1 ? k - 1 : ((k - 1 - s.pad) >> 1) - org; };
+    if (offset(s.kh) > 255 || offset(s.kw) > 255) return false;
     for (int a = 0; a < s.stride; ++a) {
         const int Hc = (s.H - (a < s.H ? a : 0) + s.stride - 1) / s.stride;
         const int Wc = (s.W - (a < s.W ? a : 0) + s.stride - 1) / s.stride;

@@ -234,6 +234,18 @@ def test_bwd_weight_long_chunks():
         assert rel < 1.1e-6, (L, rel)
 
 
+def test_bwd_weight_tap_offset_limit():
+    # the last tap row lies 256 rows below the walk's first: past the copies' 8-bit offsets
+    d = layer(inputs.small_layer("tap257", 1, 129, 1, 64, 64, 257, 1, 128, kw=9, seed=(620, 0)))
+    with pytest.raises(quan.QuanError):
+        gpu_bwd_weight(d, path=quan.QUAN_PATH_TC)
+    got, kernel = gpu_bwd_weight(d)
+    assert kernel == "bwd_weight_simt_kernel"
+    ref = oracle_bwd_weight(d)
+    for L in range(4):
+        assert_f32_close(got[L], ref[L], "dW[%d]" % L)
+
+
 def test_bwd_weight_most_blocks():
     # 4096 taps in groups of one and 16 row tiles: 65,536 blocks
     rng = np.random.default_rng(619)
