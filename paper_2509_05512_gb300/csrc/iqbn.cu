@@ -141,13 +141,16 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
     sum = t;
 }
 
-// Sum of the partial rows per channel in a fixed order (row lane rl takes rows rl, rl + 128,
-// ..., compensated fp32; then the 128 lanes as a tree, also compensated), then
+// Sum of the partial rows per channel in a fixed order (row lane rl takes every 128th or
+// 32nd, compensated fp32; then the lanes as a tree, also compensated), then
 // mean = K + S1 / n and var = max(S2 / n - (S1 / n)^2, 0) (these last few operations per
 // channel in fp64; the sums stay in fp32 pairs, the double-precision rate of this part being
-// low: the tree in fp64 took 9 us).
+// low: the tree in fp64 took 9 us, and these operations, with the division 1 / n on the device
+// and by a warp for each of the block's channels, 1.2 us: one warp does them for all, and the
+// host divides).
 // Block: 8 channels x 128 row lanes, so a lane's chain is a few loads long (32 channels x 32
-// lanes, 19 rows each and 32 lanes added one by one, took 8.4 us for 256 channels).
+// lanes, 19 rows each and 32 lanes added one by one, took 8.4 us for 256 channels); x 32 lanes
+// for up to 64 rows (small tensors).
 constexpr int FIN_C = 8;
 // (s, e) += (s2, e2): the sum's rounding error, exact by Knuth's two-sum, goes to e.
 __device__ __forceinline__ void pair_add(float& s, float& e, float s2, float e2) {
@@ -156,20 +159,20 @@ __device__ __forceinline__ void pair_add(float& s, float& e, float s2, float e2)
     s = t;
 }
 __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16* __restrict__ x,
-                                                             long long npix, int C, int rows,
+                                                             double inv_n, int C, int rows,
                                                              const float* __restrict__ part,
                                                              float* __restrict__ mean,
                                                              float* __restrict__ var) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    __shared__ float2 red[2][FIN_C][32];
+    __shared__ float2 red[2][FIN_C][32], total[2][FIN_C];
     const int cl = threadIdx.x % FIN_C, rl = threadIdx.x / FIN_C;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int c = blockIdx.x * FIN_C + cl;
     float t1 = 0.f, t2 = 0.f, e1 = 0.f, e2 = 0.f;
     if (c < C) {
 #pragma unroll 4
-        for (int r = rl; r < rows; r += 1024 / FIN_C) {
+        for (int r = rl; r < rows; r += blockDim.x / FIN_C) {
             kahan_add(t1, e1, part[static_cast<size_t>(r) * 2 * C + c]);
             kahan_add(t2, e2, part[static_cast<size_t>(r) * 2 * C + C + c]);
         }
@@ -193,21 +196,26 @@ __global__ void __launch_bounds__(1024) iqbn_finalize_kernel(const __nv_bfloat16
     }
     __syncthreads();
     if (warp < FIN_C) {  // warp w finishes channel w
-        t1 = red[0][warp][lane].x;
-        e1 = red[0][warp][lane].y;
-        t2 = red[1][warp][lane].x;
-        e2 = red[1][warp][lane].y;
+        const bool in = lane < blockDim.x / 32;
+        t1 = in ? red[0][warp][lane].x : 0.f;
+        e1 = in ? red[0][warp][lane].y : 0.f;
+        t2 = in ? red[1][warp][lane].x : 0.f;
+        e2 = in ? red[1][warp][lane].y : 0.f;
 #pragma unroll
         for (int k = 1; k < 32; k *= 2) merge(k);
-        const double d1 = static_cast<double>(t1) + e1, d2 = static_cast<double>(t2) + e2;
-        const int cw = blockIdx.x * FIN_C + warp;
-        if (lane == 0 && cw < C) {
-            const double inv_n = 1.0 / static_cast<double>(npix);
-            const double m1 = d1 * inv_n;
-            const double m2 = d2 * inv_n - m1 * m1;
-            mean[cw] = static_cast<float>(static_cast<double>(__bfloat162float(x[cw])) + m1);
-            var[cw] = m2 > 0.0 ? static_cast<float>(m2) : 0.0f;
+        if (lane == 0) {
+            total[0][warp] = make_float2(t1, e1);
+            total[1][warp] = make_float2(t2, e2);
         }
+    }
+    __syncthreads();
+    const int cw = blockIdx.x * FIN_C + threadIdx.x;
+    if (threadIdx.x < FIN_C && cw < C) {
+        const float2 s1 = total[0][threadIdx.x], s2 = total[1][threadIdx.x];
+        const double m1 = (static_cast<double>(s1.x) + s1.y) * inv_n;
+        const double m2 = (static_cast<double>(s2.x) + s2.y) * inv_n - m1 * m1;
+        mean[cw] = static_cast<float>(static_cast<double>(__bfloat162float(x[cw])) + m1);
+        var[cw] = m2 > 0.0 ? static_cast<float>(m2) : 0.0f;
     }
 }
 
@@ -310,11 +318,14 @@ bool iqbn_layout(int C, int W, long long npix, int num_sms, int per_sm, int* G, 
 
 // Channels per access: 8 (16 bytes), 4 (8 bytes: the quaternion channel counts that are no
 // multiple of 8; a scalar access each instead took 135 us, now 50 us, for the statistics and
-// the normalisation of 40 M elements in 44 channels), or 1.
-int iqbn_width(int C, const void* a, const void* b) {
+// the normalisation of 40 M elements in 44 channels), or 1.  Small tensors keep the scalar
+// accesses: with four channels a thread a block spans more pixels, and its last additions, row
+// after row, take longer than the loads (1024 pixels of 12 channels, statistics and normalisation:
+// 7.5 us with 8-byte accesses, 5.5 with scalar ones; 16,384: 8.4 and 10.2).
+int iqbn_width(int C, long long npix, const void* a, const void* b) {
     if (iqbn_vec_ok(C, a, b)) return 8;
     const uintptr_t bits = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
-    return C % 4 == 0 && bits % 8 == 0 ? 4 : 1;
+    return C % 4 == 0 && bits % 8 == 0 && (C > 256 || npix * C >= 131072) ? 4 : 1;
 }
 
 }  // namespace
@@ -334,7 +345,7 @@ size_t iqbn_stats_workspace_bytes(int C) {
 
 cudaError_t launch_iqbn_stats(const void* x, long long npix, int C, void* workspace,
                               float* mean, float* var, int num_sms, cudaStream_t stream) {
-    const int W = iqbn_width(C, x, x);
+    const int W = iqbn_width(C, npix, x, x);
     int G = 0, block = 0, grid = 0;
     if (!iqbn_layout(C, W, npix, num_sms, 4, &G, &block, &grid)) return cudaErrorInvalidValue;
     if (grid > IQBN_MAX_PARTIALS) grid = IQBN_MAX_PARTIALS;
@@ -344,14 +355,15 @@ cudaError_t launch_iqbn_stats(const void* x, long long npix, int C, void* worksp
     auto kern = W == 8 ? iqbn_stats_kernel<8> : W == 4 ? iqbn_stats_kernel<4> : iqbn_stats_kernel<1>;
     cudaError_t e = launch_pdl(kern, dim3(grid), dim3(block), smem, stream, xb, npix, C, G, part);
     if (e != cudaSuccess) return e;
-    return launch_pdl(iqbn_finalize_kernel, dim3((C + FIN_C - 1) / FIN_C), dim3(1024), 0, stream, xb,
-                      npix, C, grid, static_cast<const float*>(part), mean, var);
+    return launch_pdl(iqbn_finalize_kernel, dim3((C + FIN_C - 1) / FIN_C),
+                      dim3(grid <= 64 ? 256 : 1024), 0, stream, xb, 1.0 / static_cast<double>(npix), C, grid, static_cast<const float*>(part),
+                      mean, var);
 }
 
 cudaError_t launch_iqbn_apply(const void* x, long long npix, int C, const float* mean,
                               const float* var, const float* gamma, const float* beta, float eps,
                               int act, void* out, int num_sms, cudaStream_t stream) {
-    const int W = iqbn_width(C, x, out);
+    const int W = iqbn_width(C, npix, x, out);
     int G = 0, block = 0, grid = 0;
     if (!iqbn_layout(C, W, npix, num_sms, 8, &G, &block, &grid)) return cudaErrorInvalidValue;
     const auto* xb = static_cast<const __nv_bfloat16*>(x);

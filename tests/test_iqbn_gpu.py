@@ -70,11 +70,12 @@ def test_batch_stats(case):
 
 
 @pytest.mark.parametrize("shape,off", [
-    ((3, 5, 7, 44), 4),       # 8-byte accesses, x 8- but not 16-byte aligned, odd pixel count
+    ((3, 5, 7, 44), 4),       # x 8- but not 16-byte aligned, odd pixel count: scalar accesses
+    ((3, 31, 33, 44), 4),     # 8-byte ones, from 131,072 elements
     ((1, 1, 1, 4), 0),        # one pixel, one channel group
     ((2, 60, 61, 252), 0),    # 63 groups, several pixels per thread
     ((2, 9, 11, 2040), 0),    # 255 finishing blocks, the last group of 16-byte accesses
-], ids=["c44", "c4", "c252", "c2040"])
+], ids=["c44", "c44_large", "c4", "c252", "c2040"])
 def test_access_widths(shape, off):
     rng = np.random.default_rng(840 + shape[-1])
     C = shape[-1]
