@@ -97,9 +97,18 @@ bool pw_ok(const ConvShape& s, const EpilogueArgs& ep) {
     return true;
 }
 
-// CTA pairs: stride 1, two channel blocks to a pair, at least one whole tile of pixels.
-bool pw_cg2_ok(const ConvShape& s) {
-    return s.stride == 1 && s.Cout % 256 == 0 && s.M >= PW_NPIX;
+// CTA pairs: stride 1, two channel blocks to a pair, at least one whole tile of pixels.  The
+// ring alone is deep enough for few input channels (five or more stages), and a pair hands
+// every accumulator over twice: pairs are slower there and in short runs, where their set-up
+// shows.  Measured (us, alone and in pairs): 512 -> 1024 at 102,400 pixels 110 and 87, at 12,544
+// 20.4 and 20.4, at 3,136 10.8 and 12.0; 512 -> 512 at 25,600 22.4 and 21.3; 320 -> 256 at
+// 102,400 25.2 and 23.4, 320 -> 1024 at 25,600 21.8 and 21.8; 256 -> 512 at 102,400 31.1 and
+// 33.2; 64 -> 1024 at 3,136 4.6 and 5.8.  So five K chunks at least, and 20 chunks x tiles x
+// blocks a CTA.
+bool pw_cg2_ok(const ConvShape& s, int ctas) {
+    if (s.stride != 1 || s.Cout % 256 != 0 || s.M < PW_NPIX || s.Cin < 320) return false;
+    const long long tiles = (s.M + PW_NPIX - 1) / PW_NPIX;
+    return tiles * (s.Cout / 128) * (s.Cin / 64) >= 20LL * ctas;
 }
 
 // A[R][k] for the CTA's channel block, K-major 64-channel chunks of 128 rows x 128 bytes

@@ -1372,7 +1372,7 @@ cudaError_t launch_pw(const ConvShape& s, const void* x, const void* const w[4],
     prm.wait_limit_ns = opt.wait_limit_ns;
     prm.inject_stall = opt.inject_stall;
     prm.kchunks = s.Cin / 64;
-    const bool cg2 = pw_cg2_ok(s);
+    const bool cg2 = pw_cg2_ok(s, opt.max_ctas > 0 ? opt.max_ctas : num_sms);
     prm.stages = PwCfg::max_stages(prm.kchunks, cg2 ? PwCfg::STAGE / 2 : PwCfg::STAGE);
     prm.mblocks = s.Cout / 128;
     prm.npix = s.M;

@@ -620,11 +620,17 @@ def test_simt_small_layers(case):
 
 
 PW_PAIR_CASES = [
-    # name, N, H, W, Cin, Cout, extra, max_ctas: 1x1 stride 1 on CTA pairs
+    # name, N, H, W, Cin, Cout, extra, max_ctas: 1x1 stride 1 layers of an even number of
+    # channel blocks; the last four on CTA pairs (320 input channels and 20 chunks x tiles x
+    # blocks a CTA at least)
     ("pwp_one_tile", 1, 16, 16, 64, 256, {}, 0),
-    ("pwp_tail", 2, 17, 19, 128, 512, {"bias": True, "act": quan.QUAN_ACT_SILU}, 0),  # odd CTA's
-    ("pwp_tail_half", 1, 18, 19, 512, 256, {"iqbn": False}, 0),   # tail ends in the even half
-    ("pwp_wrap", 8, 24, 25, 192, 768, {"act": quan.QUAN_ACT_NONE}, 6),  # several tiles a pair
+    ("pwp_tail", 2, 17, 19, 128, 512, {"bias": True, "act": quan.QUAN_ACT_SILU}, 0),
+    ("pwp_tail_half", 1, 18, 19, 512, 256, {"iqbn": False}, 0),
+    ("pwp_wrap", 8, 24, 25, 192, 768, {"act": quan.QUAN_ACT_NONE}, 6),
+    ("pwp_cg2_line", 4, 16, 16, 320, 256, {}, 2),                  # four whole tiles
+    ("pwp_cg2_tail", 2, 21, 22, 384, 512, {"bias": True, "act": quan.QUAN_ACT_SILU}, 4),  # odd CTA's
+    ("pwp_cg2_half", 1, 46, 19, 512, 256, {"iqbn": False}, 2),     # tail ends in the even half
+    ("pwp_cg2_wrap", 8, 24, 25, 448, 768, {"act": quan.QUAN_ACT_NONE}, 6),  # many tiles a pair
 ]
 
 
@@ -942,9 +948,8 @@ def test_bounded_wait_timeout_every_kernel(mode, issuers):
     if mode == 4:
         spec = inputs.small_layer("inject_m", 2, 32, 32, 4, 64, 7, 2, 3, seed=(401, mode))
     elif mode == 5:
-        spec = inputs.small_layer("inject_m", 2, 16, 16, 64, 256 if issuers else 128, 1, 1, 0,
-                                  seed=(401, mode))
-        issuers = 0
+        spec = inputs.small_layer("inject_m", 2, 16, 16, 320 if issuers else 64,
+                                  512 if issuers else 128, 1, 1, 0, seed=(401, mode))
     elif mode == 6:
         spec = inputs.small_layer("inject_m", 2, 16, 16, 128 if issuers == 2 else 64, 128, 3,
                                   1 if issuers == 0 else 2, 1, seed=(401, mode))
@@ -955,8 +960,8 @@ def test_bounded_wait_timeout_every_kernel(mode, issuers):
     x = to_dev(d["x"], "bf16")
     w = [to_dev(d[k], "bf16") for k in ("wr", "wi", "wj", "wk")]
     quan.quan_set_path(quan.QUAN_PATH_TC)
-    quan.quan_set_tc_tiles(0, 16 if mode == 2 else 0, 0, mode)
-    quan.quan_set_tc_issuers(issuers)
+    quan.quan_set_tc_tiles(0, 16 if mode == 2 else 0, 2 if mode == 5 and issuers else 0, mode)
+    quan.quan_set_tc_issuers(issuers if mode < 5 else 0)
     quan.quan_set_wait_limit_ns(5_000_000)
     quan.quan_set_fault_injection(True)
     quan.qconv2d(x, *w, stride=spec.stride, pad=spec.pad, act=spec.act)
