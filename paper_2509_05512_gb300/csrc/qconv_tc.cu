@@ -1030,31 +1030,73 @@ int grid_for(const TcOptions& opt, int num_sms, int num_tiles) {
     return grid < 1 ? 1 : grid;
 }
 
-// Channel tile of the pair mode: the BNQ with the fewest estimated clocks over the waves of
-// tiles.  A K block's copies set the pace, at 1.6-1.9 clocks per row they write (512 of pixels,
-// 4 BNQ of letters, 32- and 64-byte rows alike).  Where no tile of 64 fits, the last tile may
-// reach past Qout (letter rows there are zero, their columns not stored): 80 channels are two
-// tiles of 48 and not five of 16, which copy the pixels five times (145 us against 80 us for
-// 320 -> 320 channels, 16 images of 40 x 40, 3x3).  split: K ranges split evenly between one
-// and two waves.
-// x_rows: pixel rows copied per K block.  narrowest: the smallest tile.  *cost: the estimate.
-int pair_pick_bnq(int Qout, long long m_tiles, int grid, bool split, int x_rows = 4 * BM,
-                  int narrowest = 16, double* cost = nullptr) {
+// Channel tiles of the pair mode that fit Qout: divisors, and where no tile of 64 fits 48 and 64
+// whose last tile reaches past Qout (letter rows there are zero, their columns not stored): 80
+// channels are two tiles of 48 and not five of 16 (145 us against 80 us for 320 -> 320 channels,
+// 16 images of 40 x 40, 3x3).
+bool pair_tile_ok(int Qout, int b) { return Qout % b == 0 || (Qout % 64 != 0 && b >= 48); }
+
+// Estimated time (ns) of `tiles` pair-mode tiles of b channels and ktiles K blocks each on a grid
+// of `grid` CTAs.  A K block takes the same time for every b, set by its hand-over between the
+// roles, while every TPC runs one CTA, and somewhat longer for the wider letters when both of its
+// SMs copy; an output column (4 b of them) takes 25 ns of the epilogue, which the next tile's K
+// blocks hide.  Fitted to 1,430 layers of random sizes: 5% of them took less than 0.89 or
+// more than 1.14 of it.  split: K ranges split evenly between one and two waves, at the
+// cost of about 0.4 wave.
+double pair_time(int Qout, int b, bool walk, int kappa, long long tiles, int grid, bool split,
+                 double ktiles) {
+    const bool both = 2 * tiles > grid;
+    const double block = walk          ? (both ? 470.0 : 425.0)
+                         : kappa == 16 ? (both ? 440.0 + 1.6 * b : 390.0)
+                                       : (both ? 630.0 + 1.4 * b : 600.0);
+    double waves = static_cast<double>((tiles + grid - 1) / grid);
+    if (split && tiles > grid && tiles < 2LL * grid) waves = static_cast<double>(tiles) / grid + 0.4;
+    const double main = ktiles * block, epi = 100.0 * b * (Qout % b != 0 || b == 48 ? 1.15 : 1.0);
+    const double longer = main > epi ? main : epi, shorter = main > epi ? epi : main;
+    return waves * longer + shorter + 0.3 * shorter * (waves - 1.0);
+}
+
+// The tile with the least of it.  The rows that a K block copies (512 of pixels, 4 b of letters)
+// do not decide: tiles of 16 or 32 that more CTAs share, chosen by them, took 1.2 to 1.5 times as
+// long as 64 (192 -> 512 channels, 135 images of 12 x 12, 5x5, stride 2: 39.6 and 58.3 us).
+int pair_pick_bnq(int Qout, long long m_tiles, int grid, bool split, int kappa, double ktiles,
+                  double* time = nullptr) {
     int best = 64;
     double best_t = 1e30;
-    for (int b = 64; b >= narrowest; b -= 16) {
-        if (Qout % b != 0 && (Qout % 64 == 0 || b < 48)) continue;
-        const long long tiles = m_tiles * ((Qout + b - 1) / b);
-        double waves = static_cast<double>((tiles + grid - 1) / grid);
-        if (split && tiles > grid && tiles < 2LL * grid)
-            waves = static_cast<double>(tiles) / grid;
-        const double t = waves * (x_rows + 4 * b);
+    for (int b = 64; b >= 16; b -= 16) {
+        if (!pair_tile_ok(Qout, b)) continue;
+        const double t = pair_time(Qout, b, false, kappa, m_tiles * ((Qout + b - 1) / b), grid,
+                                   split, ktiles);
         if (t < best_t) {
             best_t = t;
             best = b;
         }
     }
-    if (cost != nullptr) *cost = best_t;
+    if (time != nullptr) *time = best_t;
+    return best;
+}
+
+// Images smaller than the filter keep the widest tile that divides the channels: their pixel
+// boxes are mostly padding, and the more CTAs copy such boxes the longer each copy takes
+// (64 -> 512 channels, 4 images of 2 x 51, 7x7: 44 us in tiles of 64, 140 in tiles of 16).
+bool pair_picks(int H, int W, int kh, int kw) { return H >= kh && W >= kw; }
+
+// Rows copied per K block over the waves of tiles, x_rows of pixels and 4 b of letters each, for
+// the tile of at least `narrowest` channels with the fewest.
+double pair_rows(int Qout, long long m_tiles, int grid, bool split, int x_rows, int narrowest,
+                 int* bnq) {
+    double best = 1e30;
+    for (int b = 64; b >= narrowest; b -= 16) {
+        if (!pair_tile_ok(Qout, b)) continue;
+        const long long tiles = m_tiles * ((Qout + b - 1) / b);
+        double waves = static_cast<double>((tiles + grid - 1) / grid);
+        if (split && tiles > grid && tiles < 2LL * grid) waves = static_cast<double>(tiles) / grid;
+        const double t = waves * (x_rows + 4 * b);
+        if (t < best) {
+            best = t;
+            *bnq = b;
+        }
+    }
     return best;
 }
 
@@ -1925,17 +1967,27 @@ cudaError_t launch_qconv_tc(const ConvShape& s, const void* x, const void* const
     if (mode == MODE_PAIR && opt.mode == 0 && opt.bnq == 0 && opt.kappa == 0) {
         const int ctas = opt.max_ctas > 0 ? opt.max_ctas : num_sms;
         const bool split = opt.sk_ws != nullptr;
-        double cost = 0, walk_cost = 0;
-        bnq = pair_pick_bnq(s.Qout, m_tiles, ctas, split, 4 * BM, 16, &cost);
-        // The walk where it copies fewer rows, its padding included, in channel tiles of 48 or
-        // 64 (in tiles of 16 its 8 short MMAs per K block set the pace: 57 against 53 us for
-        // 320 -> 192 channels, 8 images of 20 x 20, 5x5).
+        double time = 1e30;
+        if (pair_picks(s.H, s.W, s.kh, s.kw))
+            bnq = pair_pick_bnq(s.Qout, m_tiles, ctas, split, kappa,
+                                static_cast<double>(s.kh) * s.kw * (s.Qin / kappa), &time);
+        // The walk, in channel tiles of 48 or 64 (in tiles of 16 its 8 short MMAs per K block set
+        // the pace: 57 against 53 us for 320 -> 192 channels, 8 images of 20 x 20, 5x5), where it
+        // copies fewer rows, its padding included.  Within one wave, where copies are no limit,
+        // also only where its estimate is the lower one: 256 -> 192 channels, 3 images of 50 x 50,
+        // 20.4 us without and 21.4 with it (past a wave: 32 and 25.5, see above).
         if (kappa == 16 && s.Qout >= 48 && walk_ok(s)) {
             const long long Mp = static_cast<long long>(s.N) * s.Ho * (s.W + s.pad);
             const long long wm_tiles = (Mp + BM - 1) / BM;
-            const int wbnq = pair_pick_bnq(s.Qout, wm_tiles, ctas, split,
-                                           4 * (BM + s.kw - 1) / s.kw, 48, &walk_cost);
-            if (walk_cost < cost) {
+            int pbnq = 64, wbnq = 64;
+            const double rows = pair_rows(s.Qout, m_tiles, ctas, split, 4 * BM, 16, &pbnq);
+            const double walk_rows = pair_rows(s.Qout, wm_tiles, ctas, split,
+                                               4 * (BM + s.kw - 1) / s.kw, 48, &wbnq);
+            const long long wtiles = wm_tiles * ((s.Qout + wbnq - 1) / wbnq);
+            if (walk_rows < rows &&
+                (wtiles > ctas ||
+                 pair_time(s.Qout, wbnq, true, kappa, wtiles, ctas, split,
+                           static_cast<double>(s.kh) * s.kw * (s.Qin / kappa)) < time)) {
                 walk = true;
                 m_tiles = wm_tiles;
                 bnq = wbnq;
@@ -2122,9 +2174,10 @@ cudaError_t launch_qconv_tc_parity(const ConvShape& f, const void* dy, const voi
     long long m_tiles = 0;
     for (int c = 0; c < 4; ++c)
         m_tiles += (static_cast<long long>(f.N) * sh[c >> 1].n * sw[c & 1].n + BM - 1) / BM;
-    const int bnq = s.sep ? pick_bnq(s.Qout, 0)
+    const int bnq = s.sep || !pair_picks(f.H, f.W, f.kh, f.kw)
+                          ? pick_bnq(s.Qout, 0)
                           : pair_pick_bnq(s.Qout, m_tiles, opt.max_ctas > 0 ? opt.max_ctas : num_sms,
-                                          false);
+                                          false, kappa, 0.25 * f.kh * f.kw * (s.Qin / kappa));
     const int num_n = (s.Qout + bnq - 1) / bnq;
     if (m_tiles * num_n > 0x7fffffffLL) {
         snprintf(err, errlen, "too many tiles");

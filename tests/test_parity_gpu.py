@@ -279,13 +279,13 @@ def test_tc_split_k_layers(case):
 
 
 SPLITK_SHARED_CASES = [
-    # name, N, H, W, Cout, extra, grid, bnq: 3x3 layers of 128 input channels whose channel
-    # tiles and grids differ, in turn on one workspace that is not cleared between them
-    ("skw_64", 5, 15, 17, 256, {}, 6, 64),                     # 10 tiles
-    ("skw_32", 4, 12, 12, 256, {"residual": True}, 9, 32),     # 10
-    ("skw_48", 2, 13, 11, 320, {}, 5, 48),                     # 6
-    ("skw_16", 2, 13, 11, 256, {}, 11, 16),                    # 12
-    ("skw_64_grid3", 4, 12, 12, 256, {"bias": True}, 3, 64),   # 5
+    # name, N, H, W, Cout, extra, grid, bnq, tiles: 3x3 layers of 128 input channels whose
+    # channel tiles and grids differ, in turn on one workspace that is not cleared between them
+    ("skw_64", 5, 15, 17, 256, {}, 6, 64, (0, 0, 0)),                      # 10 tiles
+    ("skw_32", 4, 12, 12, 256, {"residual": True}, 9, 32, (32, 32, 2)),    # 10
+    ("skw_48", 2, 13, 11, 320, {}, 5, 48, (0, 0, 0)),                      # 6
+    ("skw_16", 2, 13, 11, 256, {}, 11, 16, (32, 16, 2)),                   # 12
+    ("skw_64_grid3", 4, 12, 12, 256, {"bias": True}, 3, 64, (0, 0, 0)),    # 5
 ]
 
 
@@ -293,10 +293,10 @@ def test_tc_split_k_shared_workspace():
     ws = quan.fwd_workspace()
     first = {}
     for rep in range(2):
-        for name, N, H, W, Cout, extra, grid, bnq in SPLITK_SHARED_CASES:
+        for name, N, H, W, Cout, extra, grid, bnq, tiles in SPLITK_SHARED_CASES:
             d = inputs.layer_inputs(inputs.small_layer(name, N, H, W, 128, Cout, 3, 1, 1,
                                                        seed=(213, len(name)), **extra))
-            y, kernel = run_split(d, ws, grid, (0, 0, 0))
+            y, kernel = run_split(d, ws, grid, tiles)
             assert kernel == "qconv_tc_kernel<pair,kappa=32,bnq=%d,splitk>" % bnq, kernel
             assert int(split_flags(ws).count_nonzero()) == 0, name
             if rep == 0:
