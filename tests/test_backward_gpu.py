@@ -234,6 +234,13 @@ def test_bwd_weight_long_chunks():
         assert rel < 1.1e-6, (L, rel)
 
 
+@pytest.mark.parametrize("Cin,Cout,k", [(124, 40, 1), (152, 8, 3)])
+def test_bwd_weight_shared_memory_line(Cin, Cout, k):
+    # rows and columns that add up to 176: 48 KB of dynamic shared memory beside the static part
+    check_weight(layer(inputs.small_layer("smem48", 2, 9, 7, Cin, Cout, k, 1, k // 2,
+                                          seed=(621, k))))
+
+
 def test_bwd_weight_tap_offset_limit():
     # the last tap row lies 256 rows below the walk's first: past the copies' 8-bit offsets
     d = layer(inputs.small_layer("tap257", 1, 129, 1, 64, 64, 257, 1, 128, kw=9, seed=(620, 0)))
