@@ -81,7 +81,13 @@ cudaError_t launch_qconv_tc_shortcut(const ConvShape& s, const void* x, const vo
 // Name of the tensor-core kernel the calling thread's last launch_qconv_tc used.
 const char* last_tc_kernel();
 
-// CUDA-core path, any shape; T = __nv_bfloat16 or float.
+// Which form the calling thread's last launch of a kernel with several behind one name took
+// (for the tests, through quan_last_variant): "direct", "mma" or "tiles" for the kernels without
+// tcgen05, "single" or "pairs" for the pointwise kernel.
+extern thread_local const char* last_variant;
+
+// Without tcgen05, any shape: a thread per output (qconv_direct.cuh), warp-level MMAs (bf16) or
+// tiled CUDA-core products, whichever takes least; T = __nv_bfloat16 or float.
 cudaError_t launch_qconv_simt_bf16(const ConvShape& s, const void* x, const void* const w[4],
                                    const EpilogueArgs& ep, void* out, int num_sms,
                                    cudaStream_t stream);
@@ -94,6 +100,9 @@ cudaError_t launch_qconv_simt_f32(const ConvShape& s, const void* x, const void*
 bool mma_fwd_supported(const ConvShape& s, const void* x, const void* out, const void* residual);
 cudaError_t launch_mma_fwd(const ConvShape& s, const void* x, const void* const w[4],
                            const EpilogueArgs& ep, void* out, int num_sms, cudaStream_t stream);
+// Estimated time (us) of the first two.
+double mma_fwd_time(const ConvShape& s, int num_sms);
+double mma_bwd_data_time(const ConvShape& s, int num_sms);
 bool mma_bwd_data_supported(const ConvShape& s, const void* dy, const void* dx);
 cudaError_t launch_mma_bwd_data(const ConvShape& s, const void* dy, const void* const w[4],
                                 void* dx, int num_sms, cudaStream_t stream);
@@ -138,7 +147,7 @@ cudaError_t launch_bwd_transform(int Cin, int Cout, int kh, int kw, const void* 
 // 16-byte aligned): the input of a strided forward's input-gradient convolution.
 cudaError_t launch_bwd_upsample(const void* dy, int N, int Ho, int Wo, int C, int s, int Hu,
                                 int Wu, void* u, int num_sms, cudaStream_t stream);
-// dx [N][H][W][Cin] from dy [N][Ho][Wo][Cout] on CUDA cores, any stride.
+// dx [N][H][W][Cin] from dy [N][Ho][Wo][Cout] without tcgen05, any stride.
 cudaError_t launch_bwd_data_simt(const ConvShape& s, const void* dy, const void* const w[4],
                                  void* dx, int num_sms, cudaStream_t stream);
 // Library-owned device scratch of quan_qconv2d_bwd_data_static (one per device, in the
@@ -154,7 +163,7 @@ cudaError_t launch_bwd_weight_tc(const ConvShape& s, const void* x, const void* 
                                  char* err, size_t errlen);
 // Four fp32 arrays of n elements set to zero in one launch.
 cudaError_t launch_zero4(float* const t[4], long long n, int num_sms, cudaStream_t stream);
-// dW_L fp32 [Qout][kh][kw][Qin] (zeroed, then accumulated) on CUDA cores.
+// dW_L fp32 [Qout][kh][kw][Qin] (zeroed, then accumulated) without tcgen05.
 cudaError_t launch_bwd_weight_simt(const ConvShape& s, const void* x, const void* dy,
                                    float* const dw[4], int num_sms, cudaStream_t stream);
 

@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "qconv_direct.cuh"
 #include "qgemm_simt.cuh"
 
 namespace quan {
@@ -154,8 +155,18 @@ cudaError_t launch_bwd_transform(int Cin, int Cout, int kh, int kw, const void* 
 
 cudaError_t launch_bwd_data_simt(const ConvShape& s, const void* dy, const void* const w[4],
                                  void* dx, int num_sms, cudaStream_t stream) {
-    if (mma_bwd_data_supported(s, dy, dx))
-        return launch_mma_bwd_data(s, dy, w, dx, num_sms, stream);
+    if (mma_bwd_data_supported(s, dy, dx)) {
+        if (qd::dx_time(s, num_sms) >= mma_bwd_data_time(s, num_sms))
+            return launch_mma_bwd_data(s, dy, w, dx, num_sms, stream);
+        last_variant = "direct";
+        using T = __nv_bfloat16;
+        return qd::launch(s.sep ? qd::dx_kernel<true> : qd::dx_kernel<false>,
+                          static_cast<long long>(s.N) * s.H * s.W * s.Qin, stream, s,
+                          static_cast<const T*>(dy), static_cast<const T*>(w[0]),
+                          static_cast<const T*>(w[1]), static_cast<const T*>(w[2]),
+                          static_cast<const T*>(w[3]), static_cast<T*>(dx));
+    }
+    last_variant = "tiles";
     qg::Params p = {};
     p.s = s;
     for (int l = 0; l < 4; ++l) p.a[l] = w[l];
@@ -176,6 +187,7 @@ cudaError_t launch_bwd_weight_simt(const ConvShape& s, const void* x, const void
                                    float* const dw[4], int num_sms, cudaStream_t stream) {
     if (mma_bwd_weight_supported(s, x, dy))
         return launch_mma_bwd_weight(s, x, dy, dw, num_sms, stream);
+    last_variant = "tiles";
     const long long J = static_cast<long long>(s.kh) * s.kw * s.Qin;
     const cudaError_t e = launch_zero4(dw, J * s.Qout, num_sms, stream);
     if (e != cudaSuccess) return e;

@@ -17,8 +17,8 @@
 namespace quan {
 namespace qd {
 
-// y for one (pixel, output quaternion channel).  Two partial sums per component, of the even and
-// the odd input channels.
+// y for one (pixel, output quaternion channel).  Two partial sums per component, by the parity of
+// the input channel.
 template <typename T, bool SEP>
 __global__ void __launch_bounds__(256) fwd_kernel(ConvShape s, const T* __restrict__ x,
                                                   const T* __restrict__ wr,
@@ -45,20 +45,25 @@ __global__ void __launch_bounds__(256) fwd_kernel(ConvShape s, const T* __restri
             if (w < 0 || w >= s.W) continue;
             const T* xp = x + ((static_cast<long long>(n) * s.H + h) * s.W + w) * s.Cin;
             const long long o = ((static_cast<long long>(co) * s.kh + dh) * s.kw + dw) * s.Qin;
-            auto term = [&](int ci, float4& acc) {
-                const float4 q = make_float4(qg::to_f32(__ldg(wr + o + ci)),
-                                             qg::to_f32(__ldg(wi + o + ci)),
-                                             qg::to_f32(__ldg(wj + o + ci)),
-                                             qg::to_f32(__ldg(wk + o + ci)));
-                qg::product<SEP>(acc, q, qg::quat(xp + ci, s.Qin));
+            auto letters = [&](int ci) {
+                return make_float4(qg::to_f32(__ldg(wr + o + ci)), qg::to_f32(__ldg(wi + o + ci)),
+                                   qg::to_f32(__ldg(wj + o + ci)), qg::to_f32(__ldg(wk + o + ci)));
             };
             int ci = 0;
 #pragma unroll 1
-            for (; ci + 1 < s.Qin; ci += 2) {
-                term(ci, a[0]);
-                term(ci + 1, a[1]);
+            for (; ci + 3 < s.Qin; ci += 4) {  // (the loads of four channels before their products)
+                float4 q[4], v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    q[i] = letters(ci + i);
+                    v[i] = qg::quat(xp + ci + i, s.Qin);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) qg::product<SEP>(a[i & 1], q[i], v[i]);
             }
-            if (ci < s.Qin) term(ci, a[0]);
+#pragma unroll 1
+            for (; ci < s.Qin; ++ci)
+                qg::product<SEP>(a[0], letters(ci), qg::quat(xp + ci, s.Qin));
         }
     }
     const float4 v = make_float4(a[0].x + a[1].x, a[0].y + a[1].y, a[0].z + a[1].z, a[0].w + a[1].w);
@@ -137,9 +142,17 @@ inline double time(const Cost& c, int Q, int Qs, long long px, int row, int taps
 
 inline int least(long long a, long long b) { return static_cast<int>(a < b ? a : b); }
 
-// Forward: a letter is a line per channel of the warp.
+// Forward: a letter is a line per channel of the warp, an input component a line per pixel; where
+// the channels' rows (the pixels, for few channels) are a multiple of 64 or 128 bytes apart those
+// lines evict one another (1.4 and 2.5 times the steps' estimate).
 inline double fwd_time(const ConvShape& s, bool f32, int num_sms) {
-    return time(f32 ? FWD_F32 : FWD_BF16, s.Qout, s.Qin, s.M, s.Wo, s.kh * s.kw, least(s.kh, s.H),
+    Cost c = f32 ? FWD_F32 : FWD_BF16;
+    const long long pitch = static_cast<long long>(s.kh) * s.kw * s.Qin * (f32 ? 4 : 2);
+    const bool pixels = s.Qout < 16 && static_cast<long long>(s.stride) * s.Cin * (f32 ? 4 : 2) % 128 == 0;
+    const double evict = pixels || pitch % 128 == 0 ? 2.5 : pitch % 64 == 0 ? 1.4 : 1.0;
+    c.step *= evict;
+    c.load *= evict;
+    return time(c, s.Qout, s.Qin, s.M, s.Wo, s.kh * s.kw, least(s.kh, s.H),
                 least(s.kh, s.H + (s.Ho - 1LL) * s.stride), least(s.kw, s.W),
                 least(s.kw, s.W + (s.Wo - 1LL) * s.stride), 1.0, num_sms);
 }

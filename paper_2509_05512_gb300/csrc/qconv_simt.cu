@@ -17,15 +17,28 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "qconv_direct.cuh"
 #include "qgemm_simt.cuh"
 
 namespace quan {
 namespace {
 
 template <typename T>
+cudaError_t launch_direct(const ConvShape& s, const void* x, const void* const w[4],
+                          const EpilogueArgs& ep, void* out, cudaStream_t stream) {
+    last_variant = "direct";
+    auto kern = s.sep ? qd::fwd_kernel<T, true> : qd::fwd_kernel<T, false>;
+    return qd::launch(kern, s.M * s.Qout, stream, s, static_cast<const T*>(x),
+                      static_cast<const T*>(w[0]), static_cast<const T*>(w[1]),
+                      static_cast<const T*>(w[2]), static_cast<const T*>(w[3]), ep,
+                      static_cast<T*>(out));
+}
+
+template <typename T>
 cudaError_t launch_fwd(const ConvShape& s, const void* x, const void* const w[4],
                        const EpilogueArgs& ep, void* out, int num_sms, cudaStream_t stream) {
     if (s.M == 0 || s.Qout == 0) return cudaSuccess;
+    last_variant = "tiles";
     qg::Params p = {};
     p.s = s;
     for (int l = 0; l < 4; ++l) p.a[l] = w[l];
@@ -41,14 +54,19 @@ cudaError_t launch_fwd(const ConvShape& s, const void* x, const void* const w[4]
 cudaError_t launch_qconv_simt_bf16(const ConvShape& s, const void* x, const void* const w[4],
                                    const EpilogueArgs& ep, void* out, int num_sms,
                                    cudaStream_t stream) {
-    if (mma_fwd_supported(s, x, out, ep.residual))
-        return launch_mma_fwd(s, x, w, ep, out, num_sms, stream);
+    const bool mma = mma_fwd_supported(s, x, out, ep.residual);
+    if (qd::fwd_time(s, false, num_sms) <
+        (mma ? mma_fwd_time(s, num_sms) : qg::fwd_time(s, num_sms)))
+        return launch_direct<__nv_bfloat16>(s, x, w, ep, out, stream);
+    if (mma) return launch_mma_fwd(s, x, w, ep, out, num_sms, stream);
     return launch_fwd<__nv_bfloat16>(s, x, w, ep, out, num_sms, stream);
 }
 
 cudaError_t launch_qconv_simt_f32(const ConvShape& s, const void* x, const void* const w[4],
                                   const EpilogueArgs& ep, void* out, int num_sms,
                                   cudaStream_t stream) {
+    if (qd::fwd_time(s, true, num_sms) < qg::fwd_time(s, num_sms))
+        return launch_direct<float>(s, x, w, ep, out, stream);
     return launch_fwd<float>(s, x, w, ep, out, num_sms, stream);
 }
 

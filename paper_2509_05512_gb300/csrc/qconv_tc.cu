@@ -1453,6 +1453,7 @@ cudaError_t launch_pw(const ConvShape& s, const void* x, const void* const w[4],
     if (grid < prm.mblocks) grid = prm.mblocks;
     set_kernel_name(s.stride == 1 ? "qconv_pw_kernel<s1>" : "qconv_pw_kernel<s2>");
     const int act = s.act;
+    last_variant = cg2 ? "pairs" : "single";
     if (cg2) {
         if (act == 1) return launch_pw_pairs<1>(maps[0], prm, grid, stream);
         if (act == 2) return launch_pw_pairs<2>(maps[0], prm, grid, stream);

@@ -178,14 +178,25 @@ __device__ __forceinline__ bool sum_inside(const Params& p, int i, int n, int h,
     return outside;
 }
 
+// The epilogue's vectors for output quaternion channel i.
+__device__ __forceinline__ void vectors(const EpilogueArgs& ep, int Qout, int i, float (&bi)[4],
+                                        float (&sc)[4], float (&sh)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int c = q * Qout + i;
+        bi[q] = ep.bias ? __ldg(ep.bias + c) : 0.f;
+        sc[q] = ep.scale ? __ldg(ep.scale + c) : 1.f;
+        sh[q] = ep.scale ? __ldg(ep.shift + c) : 0.f;
+    }
+}
+
 // One output quaternion of FWD at offset o (component q at o + q Qout): Eq. 7's mix of the
 // separable form, then act(scale (y + bias) + shift + residual).
 template <typename T, bool SEP>
-__device__ __forceinline__ void finish(const Params& p, const float4& v, const float (&bi)[4],
+__device__ __forceinline__ void finish(const ConvShape& s, const EpilogueArgs& ep, T* out,
+                                       const float4& v, const float (&bi)[4],
                                        const float (&sc)[4], const float (&sh)[4], long long o) {
-    const ConvShape& s = p.s;
-    const T* res = static_cast<const T*>(p.ep.residual);
-    T* out = static_cast<T*>(p.out);
+    const T* res = static_cast<const T*>(ep.residual);
     float z[4] = {v.x, v.y, v.z, v.w};
     if constexpr (SEP) {
         z[0] = v.x - v.y - v.z - v.w;
@@ -196,7 +207,7 @@ __device__ __forceinline__ void finish(const Params& p, const float4& v, const f
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         float y = z[q] + bi[q];
-        if (p.ep.scale) y = fmaf(sc[q], y, sh[q]);
+        if (ep.scale) y = fmaf(sc[q], y, sh[q]);
         if (res) y += to_f32(res[o + q * s.Qout]);
         store(out + o + q * s.Qout, activate(y, s.act));
     }
@@ -452,17 +463,7 @@ __global__ void __launch_bounds__(THREADS, 1) qgemm_kernel(const __grid_constant
     }
     if (!active || grp != 0) return;
 
-    // output channel i's vectors (FWD)
-    float bi[4], sc[4], sh[4];
-    auto vectors = [&](int i) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = q * s.Qout + i;
-            bi[q] = p.ep.bias ? __ldg(p.ep.bias + c) : 0.f;
-            sc[q] = p.ep.scale ? __ldg(p.ep.scale + c) : 1.f;
-            sh[q] = p.ep.scale ? __ldg(p.ep.shift + c) : 0.f;
-        }
-    };
+    float bi[4], sc[4], sh[4];  // FWD: the epilogue's vectors
     // DGRAD: dx pixel (n, h, w) of the class's pixel m
     auto dx_pixel = [&](long long m, long long& n, int& h, int& w) {
         const long long rr = m / Wc;
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(THREADS, 1) qgemm_kernel(const __grid_constant
     for (int r = 0; r < TI; ++r) {
         const int i = i0 + ti + r * p.ni;
         if (i >= p.I) continue;
-        if constexpr (OP == FWD) vectors(i);
+        if constexpr (OP == FWD) vectors(p.ep, s.Qout, i, bi, sc, sh);
 #pragma unroll
         for (int c = 0; c < TJ; ++c) {
             const long long m = j0 + tj + c * p.nj;
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(THREADS, 1) qgemm_kernel(const __grid_constant
             const bool bad = not_finite(v);
             if (bad) odd |= 1u << (r * TJ + c);
             if constexpr (OP == FWD) {
-                finish<T, SEP>(p, v, bi, sc, sh, m * s.Cout + i);
+                finish<T, SEP>(s, p.ep, out, v, bi, sc, sh, m * s.Cout + i);
             } else if constexpr (OP == DGRAD) {
                 long long n;
                 int h, w;
@@ -506,8 +507,8 @@ __global__ void __launch_bounds__(THREADS, 1) qgemm_kernel(const __grid_constant
         if constexpr (OP == FWD) {
             const int4 px = tab[jl];
             if (!sum_inside<T, OP, SEP>(p, i, px.x, px.y, px.z, 0, 0, v)) continue;
-            vectors(i);
-            finish<T, SEP>(p, v, bi, sc, sh, m * s.Cout + i);
+            vectors(p.ep, s.Qout, i, bi, sc, sh);
+            finish<T, SEP>(s, p.ep, out, v, bi, sc, sh, m * s.Cout + i);
         } else if constexpr (OP == DGRAD) {
             long long n;
             int h, w;
@@ -552,17 +553,34 @@ inline long long jtiles(const Params& p, long long J) {
     return (J + w - 1) / w;
 }
 
-// The thread tile: 2 x 4 or 2 x 2 where that still gives four SMs of five a block, else (small problems, where the chain of products of one thread is the time) 1 x 1.
-// outer: WGRAD's pixel chunks, DGRAD's pixel classes.
+constexpr int TILES[3][2] = {{2, 4}, {2, 2}, {1, 1}};
+
+// The thread tile: 2 x 4 or 2 x 2 where that still gives four SMs of five a block, else (small
+// problems, where the chain of products of one thread is the time) 1 x 1.
+// outer: WGRAD's pixel chunks, DGRAD's pixel classes.  The index of TILES.
+inline int pick(Params* p, int I, long long J, long long outer, int num_sms) {
+    for (int v = 0;; ++v) {
+        layout(p, I, J, TILES[v][0], TILES[v][1]);
+        if (v == 2 || jtiles(*p, J) * p->itiles * outer * 5 >= 4LL * num_sms) return v;
+    }
+}
+
+// Estimated time (us) of FWD: the waves of blocks, each a start and its slices of 32 products.
+// (Fitted to 545 fp32 layers of random sizes: 80% between 0.9 and 1.1 of it.)
+inline double fwd_time(const ConvShape& s, int num_sms) {
+    Params p = {};
+    const int v = pick(&p, s.Qout, s.M, 1, num_sms);
+    const double blocks = static_cast<double>(jtiles(p, s.M)) * p.itiles / num_sms;
+    const double waves = blocks < 1 ? 1 : blocks < 4 ? static_cast<int>(blocks + 0.999) : blocks;
+    const double slices = (static_cast<double>(s.kh) * s.kw * s.Qin + KC - 1) / KC;
+    return 1.8 + waves * (static_cast<long long>(slices) * (v == 0 ? 3.7 : v == 1 ? 2.1 : 1.1) +
+                          (v == 0 ? 3.7 : v == 1 ? 2.5 : 1.5));
+}
+
 template <typename T, int OP, bool SEP>
 cudaError_t launch(Params p, int I, long long J, long long outer, int num_sms,
                    cudaStream_t stream) {
-    const int tiles[3][2] = {{2, 4}, {2, 2}, {1, 1}};
-    int v = 0;
-    for (; v < 3; ++v) {
-        layout(&p, I, J, tiles[v][0], tiles[v][1]);
-        if (v == 2 || jtiles(p, J) * p.itiles * outer * 5 >= 4LL * num_sms) break;
-    }
+    const int v = pick(&p, I, J, outer, num_sms);
     p.jt = jtiles(p, J);
     const long long blocks = p.jt * p.itiles * (OP == DGRAD ? outer : 1);
     const long long chunks = OP == DGRAD ? 1 : outer;

@@ -355,7 +355,12 @@ quan_status_t run_bwd_weight(const void* x, const void* dy, int N, int H, int W,
 
 }  // namespace
 
+thread_local const char* quan::last_variant = "";
+
 extern "C" {
+
+// Not part of the public header (see internal.h).
+const char* quan_last_variant(void) { return quan::last_variant; }
 
 quan_status_t quan_qconv2d_fwd(const void* x, const void* wr, const void* wi, const void* wj,
                                const void* wk, const float* bias, const float* iqbn_scale,

@@ -107,6 +107,8 @@ def load():
         lib.quan_last_error_message.argtypes = []
         lib.quan_last_error_message.restype = ctypes.c_char_p
         lib.quan_version.argtypes = []
+        lib.quan_last_variant.argtypes = []
+        lib.quan_last_variant.restype = ctypes.c_char_p
         lib.quan_packed_call.argtypes = [_i, ctypes.c_char_p]
         lib.quan_packed_call.restype = _i
         lib.quan_packed_bwd_workspace.argtypes = [ctypes.c_char_p]

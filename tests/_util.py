@@ -100,6 +100,12 @@ def assert_f32_close(got, ref, what=""):
     return rel_l2, max_abs, rms
 
 
+def last_variant():
+    """The form the last launch of a kernel with several behind one name took."""
+    from paper_2509_05512_gb300 import quan
+    return quan.load().quan_last_variant().decode()
+
+
 def inject(bits, dtype, *values):
     """A copy of a generated tensor (bf16 as bits) with (index, value) pairs set in it."""
     out = np.array(bits, copy=True)

@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 import oracle
 from paper_2509_05512_gb300 import build, inputs, quan
 from tests._util import (assert_bf16_close, assert_f32_close, assert_same_finite, host_f64, inject,
-                         out_f64, to_dev)
+                         last_variant, out_f64, to_dev)
 
 pytestmark = pytest.mark.gpu
 
@@ -188,33 +188,37 @@ def test_bwd_data_cuda_cores(case):
 
 
 EDGE_SIMT_CASES = [
-    # the warp-level MMA gradients: K and row tails, several row tiles, one and many pixel
-    # chunks, tap groups, strides beyond the filter
-    ("qs_one", 1, 1, 1, 4, 4, 1, 1, 0),
-    ("qs_q17", 2, 6, 5, 68, 68, 3, 1, 1),            # 17 rows: two row tiles
-    ("qs_q15_q1", 3, 11, 9, 60, 4, 3, 1, 1),
-    ("qs_many", 16, 45, 37, 24, 40, 3, 1, 1),
-    ("qs_groups", 2, 9, 8, 60, 60, 3, 1, 1),         # three groups of three taps
-    ("qs_s2_odd", 9, 33, 21, 20, 56, 3, 2, 1),
-    ("qs_s3_k1", 2, 10, 7, 12, 8, 1, 3, 0),          # eight classes no tap reaches
-    ("qs_s4_small", 2, 3, 2, 8, 12, 3, 4, 1),        # stride larger than the image
-    ("qs_k5_pad3", 1, 9, 12, 36, 20, 5, 2, 3),
+    # (.., the form of dx, of dW) the warp-level MMA gradients: K and row tails, several row
+    # tiles, one and many pixel chunks, tap groups, strides beyond the filter; dx of few products
+    # by a thread per quaternion
+    ("qs_one", 1, 1, 1, 4, 4, 1, 1, 0, "direct", "mma"),
+    ("qs_q17", 2, 6, 5, 68, 68, 3, 1, 1, "mma", "mma"),          # 17 rows: two row tiles
+    ("qs_q15_q1", 3, 11, 9, 60, 4, 3, 1, 1, "direct", "mma"),
+    ("qs_many", 16, 45, 37, 24, 40, 3, 1, 1, "mma", "mma"),
+    ("qs_groups", 2, 9, 8, 60, 60, 3, 1, 1, "mma", "mma"),       # three groups of three taps
+    ("qs_s2_odd", 9, 33, 21, 20, 56, 3, 2, 1, "mma", "mma"),
+    ("qs_s3_k1", 2, 10, 7, 12, 8, 1, 3, 0, "direct", "mma"),     # eight classes no tap reaches
+    ("qs_s3_k1_wide", 16, 20, 19, 24, 248, 1, 3, 0, "mma", "mma"),
+    ("qs_s4_small", 2, 3, 2, 8, 12, 3, 4, 1, "direct", "mma"),   # stride larger than the image
+    ("qs_s4_wide", 16, 19, 18, 8, 60, 3, 4, 1, "mma", "mma"),
+    ("qs_k5_pad3", 1, 9, 12, 36, 20, 5, 2, 3, "mma", "mma"),
     # too wide for those: the tiled CUDA-core products
-    ("qs_core_s5", 1, 12, 11, 20, 28, 3, 5, 1),      # dx: more than 16 pixel classes
-    ("qs_core_c260", 1, 6, 5, 260, 8, 3, 1, 1),      # dW
-    ("qs_core_k", 1, 7, 6, 20, 132, 5, 1, 2),        # dx: K = 3300
+    ("qs_core_s5", 1, 12, 11, 20, 28, 3, 5, 1, "tiles", "mma"),      # more than 16 pixel classes
+    ("qs_core_c260", 1, 6, 5, 260, 8, 3, 1, 1, "direct", "tiles"),
+    ("qs_core_k", 1, 7, 6, 20, 132, 5, 1, 2, "tiles", "mma"),        # K = 3300
 ]
 
 
 @pytest.mark.parametrize("sep", [False, True], ids=["full", "sep"])
 @pytest.mark.parametrize("case", EDGE_SIMT_CASES, ids=[c[0] for c in EDGE_SIMT_CASES])
 def test_cuda_core_gradients(case, sep):
-    name, N, H, W, Cin, Cout, k, s, p = case
+    name, N, H, W, Cin, Cout, k, s, p, dx_form, dw_form = case
     d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(616, len(name))))
     got, path, _ = gpu_bwd_data(d, separable=sep, path=quan.QUAN_PATH_SIMT)
-    assert path == quan.QUAN_PATH_SIMT
+    assert path == quan.QUAN_PATH_SIMT and last_variant() == dx_form
     assert_bf16_close(got, oracle_bwd_data(d, sep), name + " dx")
     check_weight(d, separable=sep, path=quan.QUAN_PATH_SIMT)
+    assert last_variant() == dw_form
 
 
 def test_bwd_weight_long_chunks():
@@ -270,11 +274,11 @@ def test_bwd_weight_most_blocks():
 
 
 PADDING_CASES = [
-    # name, N, H, W, Cin, Cout, k, stride, pad: off the tcgen05 grid, on each kernel
-    ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1),
-    ("inf_mma_s2", 2, 9, 8, 20, 68, 3, 2, 1),
-    ("inf_core_s5", 1, 12, 11, 20, 28, 3, 5, 1),
-    ("inf_core_c260", 1, 6, 5, 260, 12, 3, 1, 1),
+    # name, N, H, W, Cin, Cout, k, stride, pad, forms of dx and dW
+    ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1, "mma", "mma"),
+    ("inf_mma_s2", 2, 9, 8, 20, 68, 3, 2, 1, "mma", "mma"),
+    ("inf_core_s5", 1, 12, 11, 20, 28, 3, 5, 1, "tiles", "mma"),
+    ("inf_core_c260", 1, 6, 5, 260, 12, 3, 1, 1, "direct", "tiles"),
 ]
 
 
@@ -283,17 +287,19 @@ PADDING_CASES = [
 def test_padding_is_no_factor(case, sep):
     # infinite and NaN weights (dx) and output gradients (dW) reach the sums whose taps read
     # them inside the image, and no others
-    name, N, H, W, Cin, Cout, k, s, p = case
+    name, N, H, W, Cin, Cout, k, s, p, dx_form, dw_form = case
     d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(617, len(name))))
     e = dict(d)
     e["wi"] = inject(d["wi"], "bf16", ((1, 0, 0, 1), np.inf), ((2, k - 1, k - 1, 4), np.nan))
     got, _, _ = gpu_bwd_data(e, separable=sep, path=quan.QUAN_PATH_SIMT)
+    assert last_variant() == dx_form
     with np.errstate(invalid="ignore"):
         assert_same_finite(got, oracle_bwd_data(e, sep), assert_bf16_close, name + " dx")
         e = dict(d)
         e["dy"] = inject(d["dy"], "bf16", ((0, 0, 0, 1), np.inf), ((0, -1, 0, 2), np.nan))
         got, _ = gpu_bwd_weight(e, separable=sep, path=quan.QUAN_PATH_SIMT)
         ref = oracle_bwd_weight(e, sep)
+    assert last_variant() == dw_form
     for L in range(4):
         assert_same_finite(got[L], ref[L], assert_f32_close, "%s dW[%d]" % (name, L))
 

@@ -13,7 +13,7 @@ torch = pytest.importorskip("torch")
 import oracle
 from paper_2509_05512_gb300 import build, inputs, quan
 from tests._util import (assert_bf16_close, assert_f32_close, assert_same_finite, host_f64,
-                         inject, out_f64, to_dev, to_dev_f32)
+                         inject, last_variant, out_f64, to_dev, to_dev_f32)
 
 pytestmark = pytest.mark.gpu
 
@@ -710,50 +710,61 @@ def test_silu_range(cout, k):
 
 
 NARROW_CASES = [
-    # name, N, H, W, Cin, Cout, k, stride, pad, extra: bf16 layers off the tcgen05 channel
-    # grid on warp-level MMAs: K tails, channel tiles past 64, one pixel buffer, few pixels
-    ("nw_one", 1, 1, 1, 4, 4, 1, 1, 0, {}),
-    ("nw_k_tail", 3, 13, 11, 12, 20, 3, 1, 1, {"bias": True, "act": quan.QUAN_ACT_SILU}),
-    ("nw_res", 16, 45, 37, 24, 40, 3, 1, 1, {"residual": True}),
-    ("nw_two_tiles", 2, 9, 10, 20, 132, 3, 2, 1, {"iqbn": False}),
-    ("nw_one_buffer", 1, 10, 9, 100, 24, 3, 1, 1, {}),   # K = 900
-    ("nw_wide_k", 1, 6, 7, 60, 36, 7, 1, 3, {}),         # K = 2940: CUDA cores
-    ("nw_wrap", 40, 33, 35, 8, 28, 1, 1, 0, {}),         # several tiles per block
+    # name, N, H, W, Cin, Cout, k, stride, pad, extra, form: bf16 layers off the tcgen05 channel
+    # grid: a thread per output where there are few products; warp-level MMAs (K tails, channel
+    # tiles past 64, one pixel buffer, several tiles per block); tiles where K is too long
+    ("nw_one", 1, 1, 1, 4, 4, 1, 1, 0, {}, "direct"),
+    ("nw_k_tail", 3, 13, 11, 12, 20, 3, 1, 1, {"bias": True, "act": quan.QUAN_ACT_SILU}, "direct"),
+    ("nw_res", 16, 45, 37, 24, 40, 3, 1, 1, {"residual": True}, "mma"),
+    ("nw_two_tiles", 2, 9, 10, 20, 132, 3, 2, 1, {"iqbn": False}, "direct"),
+    ("nw_one_buffer", 1, 10, 9, 100, 24, 3, 1, 1, {}, "tiles"),        # K = 900
+    ("nw_wide_k", 1, 6, 7, 60, 36, 7, 1, 3, {}, "tiles"),              # K = 2940
+    ("nw_wrap", 40, 33, 35, 8, 28, 1, 1, 0, {}, "direct"),
+    ("nw_m_k_tail", 48, 40, 39, 12, 20, 3, 1, 1, {"bias": True, "act": quan.QUAN_ACT_SILU}, "mma"),
+    ("nw_m_two_tiles", 8, 33, 30, 60, 132, 3, 2, 1, {"iqbn": False}, "mma"),
+    ("nw_m_one_buffer", 16, 21, 19, 80, 24, 3, 1, 1, {}, "mma"),       # K = 720
+    ("nw_m_wrap", 64, 40, 39, 20, 28, 3, 1, 1, {}, "mma"),
+    ("nw_d_odd", 2, 5, 7, 20, 24, 3, 2, 1, {"residual": True, "bias": True}, "direct"),
 ]
 
 
 @pytest.mark.parametrize("case", NARROW_CASES, ids=[c[0] for c in NARROW_CASES])
 def test_narrow_layers(case):
-    name, N, H, W, Cin, Cout, k, s, p, extra = case
+    name, N, H, W, Cin, Cout, k, s, p, extra, form = case
     check(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(304, len(name)), **extra))
+    assert last_variant() == form
 
 
 F32_CASES = [
-    # name, N, H, W, Cin, Cout, k, stride, pad: every thread tile of the CUDA-core kernel,
-    # row and column tails
-    ("f32_one", 1, 1, 1, 4, 4, 1, 1, 0),
-    ("f32_q17", 2, 6, 5, 12, 68, 3, 1, 1),
-    ("f32_2x2", 8, 32, 32, 64, 64, 3, 1, 1),
-    ("f32_2x4", 16, 40, 40, 36, 20, 3, 1, 1),
-    ("f32_s3_pad2", 3, 13, 10, 20, 28, 5, 3, 2),
+    # name, N, H, W, Cin, Cout, k, stride, pad, form: every thread tile of the CUDA-core kernel,
+    # row and column tails, and a thread per output where there are few products
+    ("f32_one", 1, 1, 1, 4, 4, 1, 1, 0, "direct"),
+    ("f32_q17", 2, 6, 5, 12, 68, 3, 1, 1, "tiles"),
+    ("f32_2x2", 8, 32, 32, 64, 64, 3, 1, 1, "tiles"),
+    ("f32_2x4", 16, 40, 40, 36, 20, 3, 1, 1, "direct"),
+    ("f32_2x4_wide", 16, 40, 39, 68, 60, 3, 1, 1, "tiles"),
+    ("f32_s3_pad2", 3, 13, 10, 20, 28, 5, 3, 2, "tiles"),
+    ("f32_1x1", 20, 60, 31, 12, 84, 1, 1, 0, "direct"),
 ]
 
 
 @pytest.mark.parametrize("case", F32_CASES, ids=[c[0] for c in F32_CASES])
 def test_f32_layers(case):
-    name, N, H, W, Cin, Cout, k, s, p = case
+    name, N, H, W, Cin, Cout, k, s, p, form = case
     check(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, dtype="f32", bias=True,
                              act=quan.QUAN_ACT_SILU, seed=(303, len(name))))
+    assert last_variant() == form
 
 
 PADDING_CASES = [
-    # name, N, H, W, Cin, Cout, k, stride, pad, dtype, sep
-    ("inf_mma", 2, 9, 7, 24, 40, 3, 1, 1, "bf16", False),
-    ("inf_mma_sep", 2, 9, 7, 24, 68, 3, 1, 1, "bf16", True),
-    ("inf_mma_s2", 2, 9, 12, 12, 20, 5, 2, 2, "bf16", False),
-    ("inf_core", 1, 6, 7, 60, 36, 7, 1, 3, "bf16", False),
-    ("inf_core_sep", 1, 6, 7, 60, 36, 7, 1, 3, "bf16", True),
-    ("inf_f32", 2, 9, 8, 12, 20, 3, 1, 1, "f32", False),
+    # name, N, H, W, Cin, Cout, k, stride, pad, dtype, sep, form
+    ("inf_mma", 16, 19, 17, 24, 40, 3, 1, 1, "bf16", False, "mma"),
+    ("inf_mma_sep", 16, 19, 17, 24, 68, 3, 1, 1, "bf16", True, "mma"),
+    ("inf_mma_s2", 32, 19, 22, 12, 20, 5, 2, 2, "bf16", False, "mma"),
+    ("inf_direct", 2, 9, 7, 24, 40, 3, 1, 1, "bf16", False, "direct"),
+    ("inf_core", 1, 6, 7, 60, 36, 7, 1, 3, "bf16", False, "tiles"),
+    ("inf_core_sep", 1, 6, 7, 60, 36, 7, 1, 3, "bf16", True, "tiles"),
+    ("inf_f32", 2, 9, 8, 12, 20, 3, 1, 1, "f32", False, "tiles"),
 ]
 
 
@@ -761,7 +772,7 @@ PADDING_CASES = [
 def test_padding_is_no_factor(case):
     # an infinite and a NaN weight reach the outputs whose taps read them inside the image,
     # and no others: the padding is left out of the sums, not multiplied as zeros
-    name, N, H, W, Cin, Cout, k, s, p, dtype, sep = case
+    name, N, H, W, Cin, Cout, k, s, p, dtype, sep, form = case
     d = inputs.layer_inputs(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, dtype=dtype,
                                                bias=True, seed=(307, len(name))))
     d["wi"] = inject(d["wi"], dtype, ((1, 0, 0, 2), np.inf), ((3, k - 1, k - 1, 0), np.nan))
@@ -774,6 +785,7 @@ def test_padding_is_no_factor(case):
     with np.errstate(invalid="ignore"):
         ref = fn(host_f64(d["x"], dtype), *(host_f64(d[n], dtype) for n in ("wr", "wi", "wj", "wk")),
                  stride=s, pad=p, bias=d["bias"], scale=d["scale"], shift=d["shift"])
+    assert last_variant() == form
     assert_same_finite(out_f64(y), ref,
                         assert_bf16_close if dtype == "bf16" else assert_f32_close, name)
 
