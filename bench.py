@@ -114,8 +114,10 @@ KERNEL_SOURCES = {
     "qconv_pw_kernel": ("qconv_tc.cu", "qconv_pw.cuh"),
     "qconv_tc_kernel": ("qconv_tc.cu",),
     "qconv_dw_kernel": ("qconv_tc.cu", "qconv_dw.cuh"),
-    "qconv_simt_kernel": ("qconv_simt.cu", "qgemm_simt.cuh", "qconv_mma.cu", "qconv_mma.cuh"),
-    "bwd_data_simt_kernel": ("qconv_bwd.cu", "qgemm_simt.cuh", "qconv_mma.cu", "qconv_mma.cuh"),
+    "qconv_simt_kernel": ("qconv_simt.cu", "qconv_direct.cuh", "qgemm_simt.cuh", "qconv_mma.cu",
+                          "qconv_mma.cuh"),
+    "bwd_data_simt_kernel": ("qconv_bwd.cu", "qconv_direct.cuh", "qgemm_simt.cuh",
+                             "qconv_mma.cu", "qconv_mma.cuh"),
     "bwd_weight_simt_kernel": ("qconv_bwd.cu", "qgemm_simt.cuh", "qconv_mma.cu",
                                "qconv_mma.cuh"),
     "iqbn_apply_kernel": ("iqbn.cu",),

@@ -123,7 +123,7 @@ TC_CASES = [
     ("pad0", 2, 11, 12, 64, 128, 3, 1, 0),           # transposed padding 2
     ("k5_pad2", 1, 12, 11, 64, 64, 5, 1, 2),
     ("k5_pad1", 1, 12, 11, 128, 64, 5, 1, 1),        # transposed padding 3
-    # strided: dy spread out with zeros in the workspace, then the stride-1 convolution
+    # stride 2: the parity classes of dx's pixels
     ("s2_odd", 2, 15, 17, 64, 128, 3, 2, 1),
     ("s2_16to16", 1, 16, 16, 64, 64, 3, 2, 1),       # weight-stationary kernel
     ("s2_shortcut", 2, 14, 14, 64, 128, 1, 2, 0),
@@ -140,6 +140,29 @@ def test_bwd_data_tensor_cores(case):
     assert path == quan.QUAN_PATH_TC, kernel
     assert kernel.startswith("qconv_"), kernel
     assert_bf16_close(got, oracle_bwd_data(d), name + " dx")
+
+
+SPREAD_DATA_CASES = [
+    # name, N, H, W, Cin, Cout, k, stride, pad, tiles: dy spread out with zeros in the
+    # workspace, then the stride-1 convolution (strides above 2; stride 2 with tile overrides)
+    ("spread_s3", 2, 13, 17, 64, 128, 3, 3, 1, (0, 0, 0, 0)),
+    ("spread_s3_k5", 1, 16, 14, 128, 64, 5, 3, 2, (0, 0, 0, 0)),
+    ("spread_s4", 2, 15, 18, 64, 64, 5, 4, 2, (0, 0, 0, 0)),
+    ("spread_s4_edge", 1, 11, 10, 128, 192, 3, 4, 0, (0, 0, 0, 0)),  # rows no output reads
+    ("spread_s2_tiles", 2, 15, 17, 64, 128, 3, 2, 1, (16, 16, 0, 2)),
+]
+
+
+@pytest.mark.parametrize("sep", [False, True], ids=["full", "sep"])
+@pytest.mark.parametrize("case", SPREAD_DATA_CASES, ids=[c[0] for c in SPREAD_DATA_CASES])
+def test_bwd_data_spread_out(case, sep):
+    name, N, H, W, Cin, Cout, k, s, p, tiles = case
+    quan.quan_set_tc_tiles(*((16, 16, 0, 0) if sep and any(tiles) else tiles))
+    d = layer(inputs.small_layer(name, N, H, W, Cin, Cout, k, s, p, seed=(622, len(name))))
+    got, path, kernel = gpu_bwd_data(d, separable=sep, path=quan.QUAN_PATH_TC)
+    assert path == quan.QUAN_PATH_TC and "parity" not in kernel, kernel
+    assert kernel.startswith("qconv_tc_kernel<sep_t," if sep else "qconv_"), kernel
+    assert_bf16_close(got, oracle_bwd_data(d, sep), name + " dx")
 
 
 PARITY_DATA_CASES = [

@@ -641,6 +641,7 @@ def test_pointwise_cta_pairs(case):
     check(inputs.small_layer(name, N, H, W, Cin, Cout, 1, 1, 0, seed=(306, len(name)), **extra),
           path=quan.QUAN_PATH_TC)
     assert quan.quan_last_kernel() == "qconv_pw_kernel<s1>"
+    assert last_variant() == ("pairs" if "cg2" in name else "single")
 
 
 PAIR_TILE_CASES = [
@@ -977,6 +978,8 @@ def test_bounded_wait_timeout_every_kernel(mode, issuers):
     quan.quan_set_wait_limit_ns(5_000_000)
     quan.quan_set_fault_injection(True)
     quan.qconv2d(x, *w, stride=spec.stride, pad=spec.pad, act=spec.act)
+    if mode == 5:
+        assert last_variant() == ("pairs" if issuers else "single")
     st, bits = quan.quan_device_status()
     assert st == quan.QUAN_ERR_DEVICE_TIMEOUT and bits != 0
     quan.quan_set_fault_injection(False)
