@@ -75,7 +75,7 @@ typedef enum {
     QUAN_PATH_AUTO = 0, /* tensor-core path when the shape allows it, else as SIMT */
     QUAN_PATH_TC = 1,   /* tcgen05 implicit GEMM; UNSUPPORTED if the shape does not allow it */
     QUAN_PATH_SIMT = 2  /* kernels without tcgen05: fp32 on CUDA cores, bf16 on warp-level MMAs
-                           (CUDA cores where those do not apply) */
+                           (CUDA cores where those do not apply, or for few products) */
 } quan_path_t;
 
 /*
@@ -97,7 +97,7 @@ typedef enum {
  * pixels and either Cin/4 and Cout/4 multiples of 16, or Cin = 4, Cout = 64, stride 2
  * and an even W (the 4-channel stem: kh * P <= 32, where P = ceil((kw + pad mod 2) / 2)
  * rounded up to even is the number of 2-pixel pairs a filter row spans); other shapes
- * run on CUDA cores.  Returns QUAN_OK once launched.
+ * run as QUAN_PATH_SIMT.  Returns QUAN_OK once launched.
  */
 quan_status_t quan_qconv2d_fwd(const void* x, const void* wr, const void* wi, const void* wj,
                                const void* wk, const float* bias, const float* iqbn_scale,
@@ -190,7 +190,7 @@ quan_status_t quan_qconv2d_fwd_shortcut(
  *   y_j = c_r - c_i + c_j + c_k,   y_k = c_r + c_i - c_j + c_k,
  * a quarter of the full form's multiply-adds (the cross-component terms W_L x_p, L != p,
  * are dropped, as the paper describes).  The tensor-core path needs Cin/4 and Cout/4
- * multiples of 16 and 16-byte aligned pointers; other shapes run on CUDA cores.  MMA-mode
+ * multiples of 16 and 16-byte aligned pointers; other shapes run as QUAN_PATH_SIMT.  MMA-mode
  * overrides (quan_set_tc_tiles' mode) must be 0: UNSUPPORTED otherwise.
  */
 quan_status_t quan_qconv2d_sep_fwd(const void* x, const void* wr, const void* wi,
@@ -261,8 +261,7 @@ size_t quan_qconv2d_bwd_data_workspace_size_ex(int N, int H, int W, int Cin, int
  * convolution of dy with its share of the filter taps; for other strides dy is first spread
  * out with zeros between its pixels (stride - 1 of them), which multiplies the MMAs by
  * stride^2 but keeps them on the tensor cores.  Other shapes, or a strided forward with the
- * smaller workspace, run without them: bf16 products of narrow layers on warp-level MMAs,
- * the rest on the CUDA cores.
+ * smaller workspace, run as QUAN_PATH_SIMT.
  * quan_set_path(QUAN_PATH_TC) makes a shape the tensor-core path cannot run fail with
  * QUAN_ERR_UNSUPPORTED.
  */
@@ -303,8 +302,8 @@ quan_status_t quan_qconv2d_bwd_data_static(const void* dy, const void* wr, const
 /* Separable form (Eq. 8-9) of the input gradient; same arguments and paths.  The
  * tensor-core path (a square filter, pad < kh, Cin/4 and Cout/4 multiples of 16) writes the
  * letters transposed and rotated (not conjugated) into the workspace and runs one
- * convolution of dy whose block (q, p) is M[q][p] W'_q, M of Eq. 9; other shapes run on
- * CUDA cores (the workspace is then checked but not used). */
+ * convolution of dy whose block (q, p) is M[q][p] W'_q, M of Eq. 9; other shapes run as
+ * QUAN_PATH_SIMT (the workspace is then checked but not used). */
 quan_status_t quan_qconv2d_sep_bwd_data(const void* dy, const void* wr, const void* wi,
                                         const void* wj, const void* wk, int N, int H, int W,
                                         int Cin, int Cout, int kh, int kw, int stride, int pad,

@@ -352,11 +352,14 @@ cudaError_t launch_iqbn_stats(const void* x, long long npix, int C, void* worksp
     const auto* xb = static_cast<const __nv_bfloat16*>(x);
     auto* part = static_cast<float*>(workspace);
     const size_t smem = static_cast<size_t>(2) * block * W * sizeof(float);
-    auto kern = W == 8 ? iqbn_stats_kernel<8> : W == 4 ? iqbn_stats_kernel<4> : iqbn_stats_kernel<1>;
+    auto kern = W == 8   ? iqbn_stats_kernel<8>
+                : W == 4 ? iqbn_stats_kernel<4>
+                         : iqbn_stats_kernel<1>;
     cudaError_t e = launch_pdl(kern, dim3(grid), dim3(block), smem, stream, xb, npix, C, G, part);
     if (e != cudaSuccess) return e;
     return launch_pdl(iqbn_finalize_kernel, dim3((C + FIN_C - 1) / FIN_C),
-                      dim3(grid <= 64 ? 256 : 1024), 0, stream, xb, 1.0 / static_cast<double>(npix), C, grid, static_cast<const float*>(part),
+                      dim3(grid <= 64 ? 256 : 1024), 0, stream, xb,
+                      1.0 / static_cast<double>(npix), C, grid, static_cast<const float*>(part),
                       mean, var);
 }
 

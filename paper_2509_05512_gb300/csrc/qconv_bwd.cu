@@ -13,11 +13,13 @@
 //     (qconv_tc.cu), and one of any other stride as the same stride-1 convolution of dy with
 //     s - 1 zero rows and columns inserted between its pixels (bwd_upsample_kernel, into
 //     the workspace after the letters), when the caller's workspace would hold that tensor;
-//     otherwise the direct CUDA-core kernel below runs;
+//     otherwise a kernel without tcgen05 runs;
 //   * the weight gradient is a reduction over output pixels: on the tensor cores
-//     (qconv_dw.cuh), or on CUDA cores chunk by chunk of pixels, fp32 partial sums added to
+//     (qconv_dw.cuh), or without tcgen05 chunk by chunk of pixels, fp32 partial sums added to
 //     the zeroed output with atomicAdd.
-// The CUDA-core kernels of both gradients are the tiled products of qgemm_simt.cuh.
+// Without tcgen05 both run on warp-level MMAs (qconv_mma.cuh), or, where those do not apply, as
+// the tiled CUDA-core products of qgemm_simt.cuh; an input gradient of few products takes a thread
+// per quaternion (qconv_direct.cuh), by the estimated times.
 // Separable form (Eq. 7): Eq. 8-10 -- the output gradients are first mixed by the matrix M
 // of Eq. 9 (g_p = sum_m M[p][m] dy_m, M transposed equal to Eq. 7's sign table), then
 // dL/dx_p is the transposed convolution of g_p with W_p alone and dL/dW_p the correlation

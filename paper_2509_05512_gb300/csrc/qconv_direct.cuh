@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(256) fwd_kernel(ConvShape s, const T* __restri
                 qg::product<SEP>(a[0], letters(ci), qg::quat(xp + ci, s.Qin));
         }
     }
-    const float4 v = make_float4(a[0].x + a[1].x, a[0].y + a[1].y, a[0].z + a[1].z, a[0].w + a[1].w);
+    const float4 v =
+        make_float4(a[0].x + a[1].x, a[0].y + a[1].y, a[0].z + a[1].z, a[0].w + a[1].w);
     float bi[4], sc[4], sh[4];
     qg::vectors(ep, s.Qout, co, bi, sc, sh);
     qg::finish<T, SEP>(s, ep, out, v, bi, sc, sh, m * s.Cout + co);
@@ -136,8 +137,8 @@ inline double time(const Cost& c, int Q, int Qs, long long px, int row, int taps
     const double steps = Qs * h * w;
     const double lines = 4 * (Q < 32 ? Q : 32) * line < 4 ? 4 : 4 * (Q < 32 ? Q : 32) * line;
     const double loads = lines + 4 * (Q < 32 ? 32.0 / Q : 1.0) + 12;
-    return c.fixed + steps * occ * c.step + taps * occ * c.tap + wsm * steps * loads / 1900 * c.load +
-           wsm / 64 * c.warp;
+    return c.fixed + steps * occ * c.step + taps * occ * c.tap +
+           wsm * steps * loads / 1900 * c.load + wsm / 64 * c.warp;
 }
 
 inline int least(long long a, long long b) { return static_cast<int>(a < b ? a : b); }
@@ -148,7 +149,8 @@ inline int least(long long a, long long b) { return static_cast<int>(a < b ? a :
 inline double fwd_time(const ConvShape& s, bool f32, int num_sms) {
     Cost c = f32 ? FWD_F32 : FWD_BF16;
     const long long pitch = static_cast<long long>(s.kh) * s.kw * s.Qin * (f32 ? 4 : 2);
-    const bool pixels = s.Qout < 16 && static_cast<long long>(s.stride) * s.Cin * (f32 ? 4 : 2) % 128 == 0;
+    const bool pixels =
+        s.Qout < 16 && static_cast<long long>(s.stride) * s.Cin * (f32 ? 4 : 2) % 128 == 0;
     const double evict = pixels || pitch % 128 == 0 ? 2.5 : pitch % 64 == 0 ? 1.4 : 1.0;
     c.step *= evict;
     c.load *= evict;

@@ -9,7 +9,7 @@
 // where the CUDA-core form (qgemm_simt.cuh) loads and converts every bf16 by itself.
 // Measured on that layer (forward, input gradient, weight gradient, caches cold): 18, 23 and
 // 19 us, against 24, 37 and 60 us on CUDA cores in the tiled form and 32, 43 and 97 us with a
-// thread per output.  These kernels run a few thousand instructions per warp, so code size
+// thread per output; layers of fewer products go to qconv_direct.cuh.  These kernels run a few thousand instructions per warp, so code size
 // shows: unrolled gather loops inlined at three places made the weight gradient 43 us.
 //
 // As real contractions, with the signed block weight B[q][p] = sign(q, p) W_{q xor p} of Eq. 6
@@ -27,7 +27,7 @@
 // of G in registers.  Its MMA sums are of one tile each and added up in fp32: a block of a wide
 // layer (few blocks along the pixels) otherwise chains thousands of MMA steps.  Relative error
 // against 64 bits, normal inputs, 252 -> 252 channels, 8 images of 126 x 126, 3x3: 3.6e-5 in one
-// chain, 4.1e-7 so (2.33 and 1.97 ms), 1.5e-6 with a thread per weight.
+// chain, 4.1e-7 so (2.33 and 2.01 ms), 1.5e-6 with a thread per weight.
 #pragma once
 
 namespace quan {

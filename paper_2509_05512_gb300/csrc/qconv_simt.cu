@@ -1,9 +1,11 @@
-// qconv_simt.cu -- CUDA-core quaternion convolution (fp32 FFMA accumulation).
+// qconv_simt.cu -- quaternion convolution without tcgen05 (fp32 accumulation).
 //
 // Handles every shape the tensor-core path does not: fp32 tensors, quaternion channel
-// counts that are not multiples of 16, unaligned pointers and the 4-channel stem.
-// A tiled product of quaternions (qgemm_simt.cuh) of the Hamilton-product expansion of Eq. 5
-// (Sec. III-B):
+// counts that are not multiples of 16, unaligned pointers and the 4-channel stem.  Three forms,
+// chosen by their estimated times: a thread per output (qconv_direct.cuh) for few products,
+// warp-level MMAs (bf16; qconv_mma.cuh) where the tensors are aligned and a filter's channels fit
+// shared memory, else a tiled product of quaternions on CUDA cores (qgemm_simt.cuh).  All of
+// the Hamilton-product expansion of Eq. 5 (Sec. III-B):
 //   y_r = W_r x_r - W_i x_i - W_j x_j - W_k x_k
 //   y_i = W_r x_i + W_i x_r + W_j x_k - W_k x_j
 //   y_j = W_r x_j - W_i x_k + W_j x_r + W_k x_i

@@ -89,7 +89,7 @@ struct TcParams {
     EpilogueArgs ep;
     int kchunks;      // Qin / KAPPA
     int ktiles;       // kh * kw * kchunks K blocks per tile
-    int num_n_tiles;  // Qout / BNQ
+    int num_n_tiles;  // Qout / BNQ, rounded up
     int num_tiles;
     void* y;          // output [M][Cout]
     unsigned long long wait_limit_ns;
@@ -100,15 +100,14 @@ struct TcParams {
     long long Mp;     //            N * Ho * Wp
 };
 
-// WALK form (pair mode, 16-channel K blocks, stride 1, filters wider than one column).  The input pixels of a tap
-// row are walked in rows of Wp = W + pad positions, the pad zero columns before each image row
+// WALK form (pair mode, 16-channel K blocks, stride 1, filters wider than one column).  The
+// input pixels of a tap row are walked in rows of Wp = W + pad positions, the pad zero columns before each image row
 // also serving as the ones after the row above it.  The pixel at position m then reads
 // position m + dw for tap dw, so one box of 128 + kw - 1 positions serves all taps of a tap
 // row as row offsets of the A descriptor (the swizzle applies to absolute addresses, so any
 // row may start an operand).  Positions that are no output pixel (Wp - Wo per row) are
-// computed and not stored.  A box per tap instead copies a tap row's pixels kw times, and with
-// 32-byte rows the copies, at 1.6-1.9 clocks per row, take longer than the MMAs: 80 us, now
-// 67 us, for 320 -> 320 channels, 16 images of 40 x 40, 3x3; 32 and 25.5 us for 64 -> 256, 64 of
+// computed and not stored.  A box per tap instead copies a tap row's pixels kw times, which past
+// one wave, when every SM copies, takes longer than the MMAs with 32-byte rows: 80 us, now 67 us, for 320 -> 320 channels, 16 images of 40 x 40, 3x3; 32 and 25.5 us for 64 -> 256, 64 of
 // 28 x 28; 36 and 35 us for 448 -> 320, 32 of 14 x 14 (7% of its positions are padding).  K
 // blocks of 32 channels wait for the MMAs themselves: there the walk's padding and second
 // ring cost 2-8% (159 against 155 us for 256 -> 256, 64 of 56 x 56).

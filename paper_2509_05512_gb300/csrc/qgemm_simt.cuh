@@ -3,8 +3,9 @@
 // (fp32 tensors, quaternion channel counts that are not multiples of 16, unaligned pointers).
 //
 // bf16 layers come here only where qconv_mma.cuh does not take them (unaligned tensors, very
-// wide filters).  All three are the contraction  out[i][j] = sum over k of A[i][k] (x) B[k][j]  of quaternions
-// (Hamilton product of Eq. 3, 16 FFMAs), or componentwise products for the separable form:
+// wide filters), layers of few products go to qconv_direct.cuh.  All three are the contraction
+// out[i][j] = sum over k of A[i][k] (x) B[k][j]  of quaternions (Hamilton product of Eq. 3, 16
+// FFMAs), or componentwise products for the separable form:
 //   FWD    i = output channel, j = output pixel, k = (tap, input channel):
 //          A = W, B = x  (Eq. 5; separable: the products c_p, mixed by Eq. 7 at the end)
 //   DGRAD  i = input channel, j = input pixel, k = (tap, output channel):
@@ -21,10 +22,9 @@
 // with 1.7 warps to issue from).  The next slice's global loads are
 // in flight during the products.  ITILE = NI TI follows the channel count (10 channels: 5
 // threads of 2), so little of a tile is padding.
-// What bounds it: FFMA issue (TI = 2, TJ = 4: 6 LDS.128 per 128 FFMA).  One thread per output
-// quaternion straight from global memory, the form this replaces, was bound by load
-// instructions: 97 us for the fp32 layer of 8 images of 32 x 32, 64 -> 64 channels, 3x3, against
-// 23 us.
+// What bounds it: FFMA issue (TI = 2, TJ = 4: 6 LDS.128 per 128 FFMA).  A thread per output
+// quaternion straight from global memory is bound by load instructions: 97 us for the fp32 layer
+// of 8 images of 32 x 32, 64 -> 64 channels, 3x3, against 23 us.
 #pragma once
 #include <cuda_bf16.h>
 

@@ -201,8 +201,8 @@ struct EpiTile {
 };
 
 // Tile geometry functors of the QUAD/PAIR kernel's epilogue: tile index -> EpiTile, the output
-// pixel of a tile's row (kScattered, negative for none; else consecutive from m0), and whether a tile has
-// no K blocks (its accumulator is never written and the output is zero).
+// pixel of a tile's row (kScattered, negative for none; else consecutive from m0), and whether a
+// tile has no K blocks (its accumulator is never written and the output is zero).
 template <typename TileOf>
 struct LinearGeo {  // tiles of consecutive output pixels
     static constexpr bool kScattered = false;
@@ -408,7 +408,8 @@ __device__ __forceinline__ bool gflag_wait_or_abort(const unsigned* flag, uint64
 // warps 4..7 take output components r and i of every tile, warps 8..11 components j and k).
 // Accumulator buffer b (of two, used round robin over the CTA's tiles) lives at TMEM
 // columns [4 BNQ b, 4 BNQ (b+1)), component q at offset q BNQ.  A warp's share of a tile
-// is NB = 2 BNQ / CH blocks of its 32 rows x CH = min(BNQ, 32) columns; for each block it
+// is NB = 2 BNQ / CH blocks of its 32 rows x CH = 32 columns (16 for tiles of 16 and 48); for
+// each block it
 //   1. loads the block with one tcgen05.ld (after the last load of a tile it releases the
 //      accumulator buffer: acce, 256 arrivals per tile);
 //   2. transposes, within each group of NCH = CH / 8 lanes, the NCH x NCH matrix of
